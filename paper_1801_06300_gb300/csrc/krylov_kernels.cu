@@ -711,69 +711,103 @@ cudaError_t launch_group_reduce(PartPtrs slots, int nparts, int n, double* out, 
 }
 
 // ------------------------------------------------------------------ phi kernel
-// exp(A) by scaling and squaring with the [8/8] diagonal Pade approximant
-//   r(X) = N(X) / N(-X),  N(X) = sum_j c_j X^j,  c_j = (16-j)! 8! / (16! j! (8-j)!),
-// applied to X = A / 2^s with ||X||_1 <= 1 (the Pade error is far below FP64 rounding).
+// exp(A) by scaling and squaring of the Taylor polynomial of degree 16 at X = A / 2^s with
+// ||X||_1 <= 1/2 (remainder (1/2)^17 / 17! < 3e-20, far below FP64 rounding; Paterson &
+// Stockmeyer 1973 for the evaluation).
 // For phi: A = [[dt H_k, e_1, 0], [0, 0, 1], [0, 0, 0]]; column k of exp(A) holds
 // phi_1(dt H) e_1 and column k+1 holds phi_2(dt H) e_1.
 //
-// FP64 issues at a few instructions per clock per SM on this GPU, so one CTA would
-// spend ~10 us per (m+2)^3 product.  The kernels run as a cluster of PHI_CTAS CTAs:
-// every CTA keeps a full copy of the matrices in shared memory (5 buffers), computes
-// its share of the rows of each product and writes them into every CTA of the cluster
-// (distributed shared memory), then the cluster barrier publishes them.  The Pade solve
-// factors the denominator redundantly in each CTA and splits the right-hand-side columns.
+// The kernels are bound by the FP64 pipe of the SMs they run on (2 FMA per clock and SM: one
+// (m+2)^3 product costs one SM ~10 us) and by the chain of products.  They run as a cluster of
+// PHI_CTAS CTAs: every CTA keeps a full copy of the matrices in shared memory (5 buffers),
+// computes its share of the rows of each product and writes them into every CTA of the cluster
+// (distributed shared memory), then the cluster barrier publishes them.  A polynomial needs no
+// linear solve: a rational approximant's LU is a serial chain of m+2 pivot columns repeated in
+// every CTA (two thirds of the kernel's time with the [8/8] Pade form, 157 us at k = 30 on the
+// 192 x 64 bump against 36 us).  Of its six products, X^3 and X^4 share one phase, and the
+// three Horner steps P X^4 + B need only the CTA's own rows of P, hence no cluster barrier.  The
+// last product forms only the columns the caller reads.
 constexpr int PN = MMAX + 2;      // phi: (m+2) x (m+2)
 constexpr int PN2 = 2 * PN;       // phi adjoint: block-triangular 2 (m+2) x 2 (m+2)
 constexpr int PHI_CTAS = 8;
 
 namespace cg = cooperative_groups;
 
-// C = A B for rows i = rank, rank + PHI_CTAS, ... ; results broadcast to all CTAs.
+// sum_l a[l] B[l][0], two accumulators (the FP64 latency is longer than the issue interval of a
+// CTA's few warps)
 template <int LD>
-__device__ void mat_mul_cluster(cg::cluster_group& cl, const double* A, const double* B, double* C, int n) {
+PCEXP_DEV double dot_col(const double* a, const double* B, int n, double init) {
+  double s0 = init, s1 = 0;
+  int l = 0;
+#pragma unroll 2
+  for (; l + 1 < n; l += 2) {
+    s0 = fma(a[l], B[l * LD], s0);
+    s1 = fma(a[l + 1], B[(l + 1) * LD], s1);
+  }
+  if (l < n) s0 = fma(a[l], B[l * LD], s0);
+  return s0 + s1;
+}
+
+// Columns [c0, c0 + nc) of this CTA's rows (i = rank, rank + PHI_CTAS, ...) of A B, written into
+// the first `dst` CTAs of the cluster.  The caller synchronises.
+template <int LD>
+__device__ void mat_mul_rows(cg::cluster_group& cl, const double* A, const double* B, double* C, int n, int c0, int nc,
+                             int dst) {
   const int rank = (int)cl.block_rank();
   const int nrow = (n - rank + PHI_CTAS - 1) / PHI_CTAS;
-  for (int t = threadIdx.x; t < nrow * n; t += blockDim.x) {
-    const int i = rank + (t / n) * PHI_CTAS, jj = t % n;
-    double a = 0;
-    for (int l = 0; l < n; ++l) a = fma(A[i * LD + l], B[l * LD + jj], a);
-#pragma unroll
-    for (int r = 0; r < PHI_CTAS; ++r) cl.map_shared_rank(C, r)[i * LD + jj] = a;
+  for (int t = threadIdx.x; t < nrow * nc; t += blockDim.x) {
+    const int i = rank + (t / nc) * PHI_CTAS, jj = c0 + t % nc;
+    const double a = dot_col<LD>(A + i * LD, B + jj, n, 0.0);
+    for (int r = 0; r < dst; ++r) cl.map_shared_rank(C, r)[i * LD + jj] = a;
   }
-  cl.sync();
+}
+
+// 1 / j! to the last bit of a double division of exact integers (16! < 2^53)
+PCEXP_DEV constexpr double inv_factorial(int j) {
+  double f = 1.0;
+  for (int i = 2; i <= j; ++i) f *= i;
+  return 1.0 / f;
 }
 
 // exp of the n x n matrix held (identically) in buffer A of every CTA of the cluster.
-// sm holds 5 LD x LD buffers; returns the buffer with the result (same in all CTAs),
-// or nullptr if the input is not finite.  Must be called by all threads of all CTAs.
+// sm holds 5 LD x LD buffers; returns the buffer with the result, or nullptr if the input is
+// not finite.  With nc == n the result is complete in all CTAs; with nc < n only its columns
+// [c0, c0 + nc) are formed, in CTA 0.  Must be called by all threads of all CTAs.
 template <int LD>
-__device__ double* expm_cluster(cg::cluster_group& cl, double* sm, int n) {
+__device__ double* expm_cluster(cg::cluster_group& cl, double* sm, int n, int c0, int nc) {
   double* A = sm;
-  double* B2 = A + LD * LD;
-  double* B4 = B2 + LD * LD;
-  double* B6 = B4 + LD * LD;
-  double* Vb = B6 + LD * LD;
+  double* X2 = A + LD * LD;
+  double* X3 = X2 + LD * LD;
+  double* X4 = X3 + LD * LD;
+  double* Y = X4 + LD * LD;
+  constexpr int LROWS = (LD + PHI_CTAS - 1) / PHI_CTAS;
+  __shared__ double prow[2][LROWS * LD];  // this CTA's rows of the Horner polynomials
   __shared__ int s_sq;
-  __shared__ int piv_row;
-  __shared__ float colsum[LD];
+  __shared__ float colsum[4][LD];
   const int rank = (int)cl.block_rank();
   // ||A||_1 from parallel column sums in FP32 (it only selects s; the same arithmetic in
   // every CTA gives the same s)
-  for (int jj = threadIdx.x; jj < n; jj += blockDim.x) {
+  for (int t = threadIdx.x; t < 4 * n; t += blockDim.x) {
+    const int part = t / n, jj = t - part * n;
     float c = 0.f;
-    for (int i = 0; i < n; ++i) c += fabsf((float)A[i * LD + jj]);
-    colsum[jj] = c;
+    for (int i = part; i < n; i += 4) c += fabsf((float)A[i * LD + jj]);
+    colsum[part][jj] = c;
   }
   __syncthreads();
   if (threadIdx.x < 32) {
     float m = 0.f;
-    for (int jj = threadIdx.x; jj < n; jj += 32) m = fmaxf(m, colsum[jj]);
+    bool finite = true;
+    for (int jj = threadIdx.x; jj < n; jj += 32) {
+      const float c = (colsum[0][jj] + colsum[1][jj]) + (colsum[2][jj] + colsum[3][jj]);
+      finite = finite && c <= 3.0e38f;  // false for NaN too
+      m = fmaxf(m, c);
+    }
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    finite = __all_sync(0xffffffffu, finite);
     if (threadIdx.x == 0) {
       int s = 0;
-      if (m > 1.0f) s = (int)ceilf(log2f(m)) + 1;  // +1 covers the FP32 estimate
-      if (!(m <= 3.0e38f) || s > 1000) s = -1;     // NaN or overflow
+      if (m > 0.5f) s = (int)ceilf(log2f(m)) + 1;  // ||X||_1 <= 1/2 up to the FP32 estimate's rounding
+      if (!finite || s > 1000) s = -1;             // NaN or overflow
       s_sq = s;
     }
   }
@@ -782,126 +816,47 @@ __device__ double* expm_cluster(cg::cluster_group& cl, double* sm, int n) {
   if (sq < 0) return nullptr;  // uniform across the cluster (same data, same arithmetic)
   const double sc = ldexp(1.0, -sq);
   for (int t = threadIdx.x; t < n * n; t += blockDim.x) A[(t / n) * LD + t % n] *= sc;
-  // every CTA must have finished writing its own A before remote products land
+  cl.sync();  // every CTA runs and has its scaled A before remote products land
+  mat_mul_rows<LD>(cl, A, A, X2, n, 0, n, PHI_CTAS);
   cl.sync();
-  double c[9];
-  c[0] = 1.0;
-  for (int jj = 1; jj <= 8; ++jj) c[jj] = c[jj - 1] * (double)(8 - jj + 1) / (double)(jj * (16 - jj + 1));
-  mat_mul_cluster<LD>(cl, A, A, B2, n);
-  mat_mul_cluster<LD>(cl, B2, B2, B4, n);
-  mat_mul_cluster<LD>(cl, B4, B2, B6, n);
-  // V = c0 I + c2 B2 + c4 B4 + c6 B6 (Vb);  W = c1 I + c3 B2 + c5 B4 + c7 B6 (into B6)
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    const int i = t / n, jj = t - i * n, o = i * LD + jj;
-    const double id = (i == jj) ? 1.0 : 0.0;
-    const double b2 = B2[o], b4 = B4[o], b6 = B6[o];
-    Vb[o] = c[0] * id + c[2] * b2 + c[4] * b4 + c[6] * b6;
-    B6[o] = c[1] * id + c[3] * b2 + c[5] * b4 + c[7] * b6;
-  }
-  cl.sync();  // B2 is overwritten remotely next
-  mat_mul_cluster<LD>(cl, B4, B4, B2, n);  // B8
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    const int o = (t / n) * LD + t % n;
-    Vb[o] += c[8] * B2[o];
-  }
-  cl.sync();  // B4 is overwritten remotely next
-  mat_mul_cluster<LD>(cl, A, B6, B4, n);  // U = X W
-  // N = V + U (Vb), D = V - U (B2)
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    const int o = (t / n) * LD + t % n;
-    const double V = Vb[o], U = B4[o];
-    Vb[o] = V + U;
-    B2[o] = V - U;
-  }
-  __syncthreads();
-  // solve D X = N: LU with partial pivoting repeated in every CTA (identical); this CTA
-  // keeps the right-hand-side columns jj = rank, rank + PHI_CTAS, ...
-  double* Dm = B2;
-  double* Nm = Vb;
-  const int ncol = (n - rank + PHI_CTAS - 1) / PHI_CTAS;
-  for (int col = 0; col < n; ++col) {
-    if (threadIdx.x < 32) {
-      // partial pivoting by warp argmax on the bit patterns of |x|
-      unsigned long long best = 0ull;
-      int bi = col;
-      for (int i = col + threadIdx.x; i < n; i += 32) {
-        const unsigned long long key = (unsigned long long)__double_as_longlong(Dm[i * LD + col]) & 0x7fffffffffffffffull;
-        if (key > best || i == col) {
-          best = key;
-          bi = i;
-        }
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) {
-          best = ob;
-          bi = oi;
-        }
-      }
-      if (threadIdx.x == 0) piv_row = bi;
-    }
-    __syncthreads();
-    const int pr = piv_row;
-    if (pr != col) {
-      for (int t = threadIdx.x; t < n; t += blockDim.x) {
-        double a = Dm[col * LD + t];
-        Dm[col * LD + t] = Dm[pr * LD + t];
-        Dm[pr * LD + t] = a;
-      }
-      for (int t = threadIdx.x; t < ncol; t += blockDim.x) {
-        const int jj = rank + t * PHI_CTAS;
-        double b = Nm[col * LD + jj];
-        Nm[col * LD + jj] = Nm[pr * LD + jj];
-        Nm[pr * LD + jj] = b;
-      }
-      __syncthreads();
-    }
-    const double piv = Dm[col * LD + col];
-    const int nr = n - col - 1, w = (n - col - 1) + ncol;
-    for (int t = threadIdx.x; t < nr * w; t += blockDim.x) {
-      const int i = col + 1 + t / w, q = t % w;
-      const double f = Dm[i * LD + col] / piv;
-      if (q < n - col - 1) {
-        const int jj = col + 1 + q;
-        Dm[i * LD + jj] -= f * Dm[col * LD + jj];
-      } else {
-        const int jj = rank + (q - (n - col - 1)) * PHI_CTAS;
-        Nm[i * LD + jj] -= f * Nm[col * LD + jj];
-      }
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nr; t += blockDim.x) Dm[(col + 1 + t) * LD + col] = 0.0;
-    __syncthreads();
-  }
-  for (int col = n - 1; col >= 0; --col) {
-    const double piv = Dm[col * LD + col];
-    for (int t = threadIdx.x; t < ncol; t += blockDim.x) Nm[col * LD + rank + t * PHI_CTAS] /= piv;
-    __syncthreads();
-    for (int t = threadIdx.x; t < col * ncol; t += blockDim.x) {
-      const int i = t / ncol, jj = rank + (t % ncol) * PHI_CTAS;
-      Nm[i * LD + jj] -= Dm[i * LD + col] * Nm[col * LD + jj];
-    }
-    __syncthreads();
-  }
-  // publish this CTA's solution columns once every CTA has finished its own solve
+  mat_mul_rows<LD>(cl, X2, A, X3, n, 0, n, PHI_CTAS);
+  mat_mul_rows<LD>(cl, X2, X2, X4, n, 0, n, PHI_CTAS);
   cl.sync();
-  for (int t = threadIdx.x; t < n * ncol; t += blockDim.x) {
-    const int i = t / ncol, jj = rank + (t % ncol) * PHI_CTAS;
-    const double v = Nm[i * LD + jj];
+  // P = c16 X4 + B_3, then P <- P X4 + B_k for k = 2, 1, 0 with
+  // B_k = c_4k I + c_4k+1 X + c_4k+2 X2 + c_4k+3 X3; the last one goes to every CTA
+  const int nrow = (n - rank + PHI_CTAS - 1) / PHI_CTAS;
+  constexpr double c[17] = {inv_factorial(0),  inv_factorial(1),  inv_factorial(2),  inv_factorial(3),
+                            inv_factorial(4),  inv_factorial(5),  inv_factorial(6),  inv_factorial(7),
+                            inv_factorial(8),  inv_factorial(9),  inv_factorial(10), inv_factorial(11),
+                            inv_factorial(12), inv_factorial(13), inv_factorial(14), inv_factorial(15),
+                            inv_factorial(16)};
 #pragma unroll
-    for (int r = 0; r < PHI_CTAS; ++r)
-      if (r != rank) cl.map_shared_rank(Nm, r)[i * LD + jj] = v;
+  for (int k = 3; k >= 0; --k) {
+    const double* P = prow[(k & 1) ^ 1];  // of the previous step
+    for (int t = threadIdx.x; t < nrow * n; t += blockDim.x) {
+      const int r = t / n, i = rank + r * PHI_CTAS, jj = t - r * n, o = i * LD + jj;
+      double b = fma(c[4 * k + 3], X3[o], fma(c[4 * k + 2], X2[o], c[4 * k + 1] * A[o]));
+      if (i == jj) b += c[4 * k];
+      if (k == 3) b = fma(c[16], X4[o], b);
+      else b = dot_col<LD>(P + r * LD, X4 + jj, n, b);
+      if (k > 0) {
+        prow[k & 1][r * LD + jj] = b;
+      } else {
+        for (int q = 0; q < PHI_CTAS; ++q) cl.map_shared_rank(Y, q)[o] = b;
+      }
+    }
+    if (k > 0) __syncthreads();
   }
   cl.sync();
-  // squaring (X in Vb, B4 as the other buffer)
-  double* X = Vb;
-  double* Y = B4;
+  double* X = Y;
+  double* Z = X2;
   for (int it = 0; it < sq; ++it) {
-    mat_mul_cluster<LD>(cl, X, X, Y, n);
+    const bool part = it == sq - 1 && nc < n;
+    mat_mul_rows<LD>(cl, X, X, Z, n, part ? c0 : 0, part ? nc : n, part ? 1 : PHI_CTAS);
+    cl.sync();
     double* t = X;
-    X = Y;
-    Y = t;
+    X = Z;
+    Z = t;
   }
   return X;
 }
@@ -914,10 +869,12 @@ __device__ double* expm_cluster(cg::cluster_group& cl, double* sm, int n) {
 //   est = dt h_{k+1,k} |e_k^T phi_2(dt H_k) e_1| / ||phi_1(dt H_k) e_1||,
 // from the phi_2 column of the same exponential.  check_tol > 0 is a checkpoint of the
 // adaptive dimension: only est is formed, and ks->done is raised when est <= check_tol.
+// The scalars at the end run on one warp, an entry of y per lane.
 __global__ void __cluster_dims__(PHI_CTAS, 1, 1) __launch_bounds__(256)
     phi_kernel(KState* ks, const double* dt_dev, double dt_host, double factor, StepState* ss, int stage, int which,
                const double* dt_prev, double check_tol) {
   extern __shared__ double sm[];
+  static_assert(MMAX <= 32, "one lane per Krylov column");
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
   const int k = ks->k;
@@ -937,51 +894,51 @@ __global__ void __cluster_dims__(PHI_CTAS, 1, 1) __launch_bounds__(256)
   }
   const int n = k + 2;
   double* A = sm;
-  for (int t = threadIdx.x; t < PN * PN; t += blockDim.x) A[t] = 0.0;
-  __syncthreads();
-  for (int t = threadIdx.x; t < k * k; t += blockDim.x) {
-    const int i = t / k, jj = t - i * k;
-    A[i * PN + jj] = dt * ks->H[i * MMAX + jj];
-  }
-  if (threadIdx.x == 0) {
-    A[0 * PN + k] = 1.0;
-    A[k * PN + k + 1] = 1.0;
+  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
+    const int i = t / n, jj = t - i * n;
+    double a = 0.0;
+    if (i < k && jj < k) a = dt * ks->H[i * MMAX + jj];
+    else if ((i == 0 && jj == k) || (i == k && jj == k + 1)) a = 1.0;
+    A[i * PN + jj] = a;
   }
   __syncthreads();
-  const double* X = expm_cluster<PN>(cl, sm, n);
-  if (rank == 0 && threadIdx.x == 0) {
-    if (!X) {
+  const double* X = expm_cluster<PN>(cl, sm, n, k, 2);
+  if (rank != 0 || threadIdx.x >= 32) return;
+  const int i = threadIdx.x;
+  if (!X) {
+    if (i == 0) {
       ks->err = 1;
       if (ss) ss->err = 1;
-      return;
     }
-    double n1 = 0.0;
-    for (int i = 0; i < k; ++i) n1 += X[i * PN + k] * X[i * PN + k];
-    const double est = dt * fabs(ks->H[k * MMAX + k - 1]) * fabs(X[(k - 1) * PN + k + 1]) / sqrt(n1);
-    ks->err_est = est;
-    if (check_tol > 0.0) {
-      if (est <= check_tol) ks->done = 1;  // the estimate may be NaN: then the process goes on
-      return;
-    }
-    const double beta = ks->beta;
-    const double f = dt_prev ? factor * dt / *dt_prev : factor;
-    bool ok = true;
-    for (int i = 0; i < k; ++i) {
-      const double y1 = X[i * PN + k], y2 = X[i * PN + k + 1];
-      ks->y[i] = y1;
-      ks->y2[i] = y2;
-      ks->acoef[i] = f * dt * beta * (which == 2 ? y2 : y1) * ks->s[i];
-      ok = ok && isfinite(ks->acoef[i]);
-    }
-    for (int i = k; i <= MMAX; ++i) ks->acoef[i] = 0.0;
-    if (!ok) ks->err = 1;
-    if (ss) {
-      ss->k[stage] = k;
-      ss->beta[stage] = beta;
-      ss->kerr[stage] = est;
-      ss->pass2[stage] = ks->pass2;
-      if (!ok) ss->err = 1;
-    }
+    return;
+  }
+  const double y1 = i < k ? X[i * PN + k] : 0.0, y2 = i < k ? X[i * PN + k + 1] : 0.0;
+  double n1 = y1 * y1;
+  for (int o = 16; o > 0; o >>= 1) n1 += __shfl_xor_sync(0xffffffffu, n1, o);
+  const double est = dt * fabs(ks->H[k * MMAX + k - 1]) * fabs(__shfl_sync(0xffffffffu, y2, k - 1)) / sqrt(n1);
+  if (i == 0) ks->err_est = est;
+  if (check_tol > 0.0) {
+    if (i == 0 && est <= check_tol) ks->done = 1;  // the estimate may be NaN: then the process goes on
+    return;
+  }
+  const double beta = ks->beta;
+  const double f = dt_prev ? factor * dt / *dt_prev : factor;
+  const double ac = i < k ? f * dt * beta * (which == 2 ? y2 : y1) * ks->s[i] : 0.0;
+  const bool ok = __all_sync(0xffffffffu, isfinite(ac));
+  if (i < k) {
+    ks->y[i] = y1;
+    ks->y2[i] = y2;
+  }
+  ks->acoef[i] = ac;
+  if (i != 0) return;
+  for (int q = 32; q <= MMAX; ++q) ks->acoef[q] = 0.0;
+  if (!ok) ks->err = 1;
+  if (ss) {
+    ss->k[stage] = k;
+    ss->beta[stage] = beta;
+    ss->kerr[stage] = est;
+    ss->pass2[stage] = ks->pass2;
+    if (!ok) ss->err = 1;
   }
 }
 
@@ -1014,7 +971,7 @@ __global__ void __cluster_dims__(PHI_CTAS, 1, 1) __launch_bounds__(256)
     M[(n0 + k + 1) * PN2 + n0 + k] = 1.0;
   }
   __syncthreads();
-  const double* X = expm_cluster<PN2>(cl, sm, n);
+  const double* X = expm_cluster<PN2>(cl, sm, n, 0, n);
   if (rank == 0) {
     if (!X) {
       if (threadIdx.x == 0) *err = 1;
