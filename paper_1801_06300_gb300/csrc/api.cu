@@ -17,6 +17,7 @@
 #include <mutex>
 #include <string>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "host_setup.h"
@@ -456,16 +457,19 @@ template <class T> T* shadow(pcexp_ctx* c, int i) {
   return c->fp32 ? reinterpret_cast<T*>(c->S32[i]) : reinterpret_cast<T*>(c->U64[i]);
 }
 
-// Input state-shaped double array (host or device) -> internal basis in T (dst, device).
+// Input state-shaped double array (host or device) -> internal basis in T (dst, device), and in
+// FP32 in sh (nullable).
 template <class T>
-int import_vec(pcexp_ctx* c, const double* src, int on_device, T* dst) {
+int import_vec(pcexp_ctx* c, const double* src, int on_device, T* dst, float* sh = nullptr) {
   const double* s = src;
   if (!on_device) {
     PCEXP_CK(cudaMemcpyAsync(c->io64a, src, c->K * sizeof(double), cudaMemcpyHostToDevice, c->st));
     s = c->io64a;
   }
-  if (c->basis_io == PCEXP_BASIS_PAPER) PCEXP_CK(launch_paper_to_internal<T>(s, dst, c->Q, c->E, c->nb, c->nv, c->st));
+  if (c->basis_io == PCEXP_BASIS_PAPER) PCEXP_CK(launch_paper_to_internal<T>(s, dst, c->Q, c->E, c->nb, c->nv, c->st, sh));
   else PCEXP_CK(launch_cast<double, T>(s, dst, c->K, c->st));
+  if constexpr (std::is_same<T, double>::value)
+    if (sh && c->basis_io != PCEXP_BASIS_PAPER) PCEXP_CK(launch_cast<double, float>(dst, sh, c->K, c->st));
   return PCEXP_OK;
 }
 
@@ -1171,7 +1175,7 @@ int create_impl(pcexp_ctx* c, const pcexp_mesh* mesh, int p, const pcexp_physics
     PCEXP_TRY(upload<double>(c, &c->fgeo, s.fgeo));
   }
   void* q = nullptr;
-  PCEXP_TRY(upload<double>(c, &q, s.Q));
+  PCEXP_TRY(upload<double>(c, &q, pack_basis_change(s.Q, s.E, s.nb, s.dim)));
   c->Q = reinterpret_cast<double*>(q);
   PCEXP_TRY(dalloc(c, &c->ef, s.ef.size()));
   PCEXP_TRY(dalloc(c, &c->fel, s.fel.size() + 2));
@@ -1554,8 +1558,8 @@ int pcexp_sizes(const pcexp_ctx* c, int64_t* n_elem, int32_t* n_basis, int32_t* 
 int pcexp_set_state(pcexp_ctx* c, const double* U, int on_device) {
   PCEXP_TRY(check_ctx(c));
   if (!U) return PCEXP_ERR_INVALID_ARG;
-  PCEXP_TRY(import_vec<double>(c, U, on_device, c->U64[c->cur]));
-  PCEXP_TRY(refresh_shadow<double>(c, c->cur));
+  float* sh = c->fp32 ? reinterpret_cast<float*>(c->S32[c->cur]) : nullptr;
+  PCEXP_TRY(import_vec<double>(c, U, on_device, c->U64[c->cur], sh));
   PCEXP_CK(cudaStreamSynchronize(c->st));
   c->etd2_prev = false;
   return PCEXP_OK;

@@ -7,34 +7,108 @@
 namespace pcexp {
 
 // ------------------------------------------------------------ basis conversion
-template <class T>
-__global__ void paper_to_internal_kernel(const double* __restrict__ src, T* __restrict__ dst,
-                                         const double* __restrict__ Q, int64_t E, int nb, int nv) {
-  const int64_t n = E * nv * nb;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = idx / (nv * nb);
-    const int r = (int)(idx - e * nv * nb), v = r / nb, j = r - v * nb;
-    const double* q = Q + e * nb * nb;
-    const double* s = src + e * nv * nb + v * nb;
-    double a = 0;
-    for (int i = 0; i < nb; ++i) a += q[i * nb + j] * s[i];
-    dst[idx] = (T)a;
+// Both bases are orthonormal and graded by total degree (each spans P^0, P^1, ... in turn), so
+// Q_e couples functions of equal degree only: one block per degree, of 1, 2, 3, 4 (triangles) or
+// 1, 3, 6 (tetrahedra) functions, and the degree-0 block is 1.  The blocks of degrees 1..p are
+// stored packed, row-major, [E][QN] (pack_basis_change).
+//
+// A conversion is bound by the FP64 pipe (the FP64 rate is 1/62 of FP32's): the blocks take 45
+// instead of 100 FMAs per variable on tetrahedra at p = 2.  One thread per (element, variable)
+// row forms the whole row, so a warp runs the same block sizes; rows and blocks are staged in
+// shared memory for coalesced global access.  Tetrahedra at p = 2, 33^3 cubes (K = 10.8 M): the
+// three conversions of an FP32-mixed J v call (two in, one out) take 357 us together, against 852
+// us with a thread per output and the full matrix.
+template <int D, int P> struct QBlocks {
+  static constexpr int NV = D + 2, NB = D == 2 ? (P + 1) * (P + 2) / 2 : (P + 1) * (P + 2) * (P + 3) / 6;
+  __host__ __device__ static constexpr int size(int deg) { return D == 2 ? deg + 1 : (deg + 1) * (deg + 2) / 2; }
+  __host__ __device__ static constexpr int first(int deg) { return deg == 0 ? 0 : first(deg - 1) + size(deg - 1); }
+  __host__ __device__ static constexpr int offset(int deg) { return deg <= 1 ? 0 : offset(deg - 1) + size(deg - 1) * size(deg - 1); }
+  static constexpr int QN = offset(P + 1);
+  static constexpr int ET = D == 2 ? 64 : 48, NT = ET * NV;  // elements and threads per block
+  static constexpr int ROW = NB | 1;                          // padded shared-memory row
+};
+
+// x[block of degree DEG, ...] = Q (or Q^T) in, for degrees DEG..P
+template <int D, int P, bool TRANS, int DEG>
+PCEXP_DEV void apply_blocks(const double* q, const double (&in)[QBlocks<D, P>::NB], double* x) {
+  using B = QBlocks<D, P>;
+  if constexpr (DEG <= P) {
+    constexpr int n = B::size(DEG), f = B::first(DEG), o = B::offset(DEG);
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      double a = 0;
+#pragma unroll
+      for (int j = 0; j < n; ++j) a = fma(TRANS ? q[o + j * n + i] : q[o + i * n + j], in[f + j], a);
+      x[f + i] = a;
+    }
+    apply_blocks<D, P, TRANS, DEG + 1>(q, in, x);
   }
 }
 
-template <class T>
-__global__ void internal_to_paper_kernel(const T* __restrict__ src, double* __restrict__ dst,
-                                         const double* __restrict__ Q, int64_t E, int nb, int nv) {
-  const int64_t n = E * nv * nb;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = idx / (nv * nb);
-    const int r = (int)(idx - e * nv * nb), v = r / nb, i = r - v * nb;
-    const double* q = Q + e * nb * nb + i * nb;
-    const T* s = src + e * nv * nb + v * nb;
-    double a = 0;
-    for (int j = 0; j < nb; ++j) a += q[j] * (double)s[j];
-    dst[idx] = a;
+// TRANS: dst = Q^T src (paper -> internal), else dst = Q src.  dst2 (nullable): a second, FP32 copy.
+template <class Tin, class Tout, int D, int P, bool TRANS>
+__global__ void __launch_bounds__(QBlocks<D, P>::NT) change_basis_kernel(const Tin* __restrict__ src,
+                                                                        Tout* __restrict__ dst,
+                                                                        float* __restrict__ dst2,
+                                                                        const double* __restrict__ Q, int64_t E) {
+  using B = QBlocks<D, P>;
+  constexpr int NB = B::NB, NV = B::NV, QN = B::QN, ROW = B::ROW;
+  __shared__ double sq[B::ET * QN + 1];
+  __shared__ double sx[B::NT * ROW];
+  const int64_t e0 = (int64_t)blockIdx.x * B::ET;
+  const int ne = (int)((E - e0) < B::ET ? (E - e0) : B::ET);
+  for (int i = threadIdx.x; i < ne * QN; i += B::NT) sq[i] = Q[e0 * QN + i];
+  for (int i = threadIdx.x; i < ne * NV * NB; i += B::NT) sx[i / NB * ROW + i % NB] = (double)src[e0 * NV * NB + i];
+  __syncthreads();
+  if (threadIdx.x < ne * NV) {
+    double* x = sx + threadIdx.x * ROW;
+    const double* q = sq + threadIdx.x / NV * QN;
+    double in[NB];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) in[j] = x[j];
+    apply_blocks<D, P, TRANS, 1>(q, in, x);
   }
+  __syncthreads();
+  for (int i = threadIdx.x; i < ne * NV * NB; i += B::NT) {
+    const double a = sx[i / NB * ROW + i % NB];
+    dst[e0 * NV * NB + i] = (Tout)a;
+    if (dst2) dst2[e0 * NV * NB + i] = (float)a;
+  }
+}
+
+template <class Tin, class Tout, int D, int P, bool TRANS>
+static cudaError_t change_basis_p(const Tin* src, Tout* dst, float* dst2, const double* Q, int64_t E, cudaStream_t st) {
+  using B = QBlocks<D, P>;
+  change_basis_kernel<Tin, Tout, D, P, TRANS>
+      <<<(unsigned)((E + B::ET - 1) / B::ET), B::NT, 0, st>>>(src, dst, dst2, Q, E);
+  return cudaGetLastError();
+}
+template <class Tin, class Tout, bool TRANS>
+static cudaError_t change_basis(const Tin* src, Tout* dst, float* dst2, const double* Q, int64_t E, int nb, int nv,
+                                cudaStream_t st) {
+  switch (nv * 16 + nb) {
+    case 4 * 16 + 1: return change_basis_p<Tin, Tout, 2, 0, TRANS>(src, dst, dst2, Q, E, st);
+    case 4 * 16 + 3: return change_basis_p<Tin, Tout, 2, 1, TRANS>(src, dst, dst2, Q, E, st);
+    case 4 * 16 + 6: return change_basis_p<Tin, Tout, 2, 2, TRANS>(src, dst, dst2, Q, E, st);
+    case 4 * 16 + 10: return change_basis_p<Tin, Tout, 2, 3, TRANS>(src, dst, dst2, Q, E, st);
+    case 5 * 16 + 1: return change_basis_p<Tin, Tout, 3, 0, TRANS>(src, dst, dst2, Q, E, st);
+    case 5 * 16 + 4: return change_basis_p<Tin, Tout, 3, 1, TRANS>(src, dst, dst2, Q, E, st);
+    case 5 * 16 + 10: return change_basis_p<Tin, Tout, 3, 2, TRANS>(src, dst, dst2, Q, E, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+std::vector<double> pack_basis_change(const std::vector<double>& Q, int64_t E, int nb, int dim) {
+  std::vector<double> out;
+  out.reserve(Q.size());
+  for (int64_t e = 0; e < E; ++e)
+    for (int deg = 1, f = 1; f < nb; ++deg) {
+      const int n = dim == 2 ? deg + 1 : (deg + 1) * (deg + 2) / 2;
+      for (int i = 0; i < n; ++i)
+        for (int j = 0; j < n; ++j) out.push_back(Q[((size_t)e * nb + f + i) * nb + f + j]);
+      f += n;
+    }
+  return out;
 }
 
 static unsigned grid_for(int64_t n) {
@@ -44,14 +118,13 @@ static unsigned grid_for(int64_t n) {
 }
 
 template <class T>
-cudaError_t launch_paper_to_internal(const double* src, T* dst, const double* Q, int64_t E, int nb, int nv, cudaStream_t st) {
-  paper_to_internal_kernel<T><<<grid_for(E * nb * nv), 256, 0, st>>>(src, dst, Q, E, nb, nv);
-  return cudaGetLastError();
+cudaError_t launch_paper_to_internal(const double* src, T* dst, const double* Q, int64_t E, int nb, int nv,
+                                     cudaStream_t st, float* dst32) {
+  return change_basis<double, T, true>(src, dst, dst32, Q, E, nb, nv, st);
 }
 template <class T>
 cudaError_t launch_internal_to_paper(const T* src, double* dst, const double* Q, int64_t E, int nb, int nv, cudaStream_t st) {
-  internal_to_paper_kernel<T><<<grid_for(E * nb * nv), 256, 0, st>>>(src, dst, Q, E, nb, nv);
-  return cudaGetLastError();
+  return change_basis<T, double, false>(src, dst, nullptr, Q, E, nb, nv, st);
 }
 
 template <class T>
@@ -275,7 +348,7 @@ cudaError_t launch_zero_range(T* x, int64_t from, int64_t to, cudaStream_t st) {
 
 #define PCEXP_INST(T)                                                                                         \
   template cudaError_t launch_paper_to_internal<T>(const double*, T*, const double*, int64_t, int, int,        \
-                                                   cudaStream_t);                                              \
+                                                   cudaStream_t, float*);                                      \
   template cudaError_t launch_internal_to_paper<T>(const T*, double*, const double*, int64_t, int, int,        \
                                                    cudaStream_t);                                              \
   template cudaError_t launch_scale_elements<T>(T*, const T*, int64_t, int, cudaStream_t);                     \

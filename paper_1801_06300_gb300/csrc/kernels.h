@@ -1,6 +1,7 @@
 // Launchers of the device kernels (host-callable), shared by the C API.
 #pragma once
 #include <cstdint>
+#include <vector>
 #include <cuda_runtime.h>
 
 #include "../../include/pcexp.h"
@@ -248,9 +249,12 @@ cudaError_t launch_vortex_param_grad(const DGData<T>& d, const T* u, const doubl
                     : launch_vortex_param_grad_d<T, 2>(d, u, xq, prm, dvel, out, partials, counter, st);
 }
 // ---- dimension-free kernels (dg_common.cu)
-// basis conversions at the interface (Q_e: paper <- internal)
+// basis conversions at the interface (Q_e: paper <- internal; its diagonal blocks of degrees 1..p
+// packed by pack_basis_change).  dst32 (nullable): the converted vector in FP32 as well
+std::vector<double> pack_basis_change(const std::vector<double>& Q, int64_t E, int nb, int dim);
 template <class T>
-cudaError_t launch_paper_to_internal(const double* src, T* dst, const double* Q, int64_t E, int nb, int nv, cudaStream_t st);
+cudaError_t launch_paper_to_internal(const double* src, T* dst, const double* Q, int64_t E, int nb, int nv,
+                                     cudaStream_t st, float* dst32 = nullptr);
 template <class T>
 cudaError_t launch_internal_to_paper(const T* src, double* dst, const double* Q, int64_t E, int nb, int nv, cudaStream_t st);
 // x[e][:] *= s[e] (block of nvb entries per element)
