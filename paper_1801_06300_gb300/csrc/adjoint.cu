@@ -266,6 +266,27 @@ __global__ void bbar_kernel(const double* __restrict__ Z, const double* __restri
     bbar[r] = s0 * Vb[r] + cz * Z[r];
 }
 
+// acc[k] += sum_i sums[i][k], k = 0, 1 (one block, fixed order)
+__global__ void __launch_bounds__(256) theta_sum_kernel(const double* __restrict__ sums, int64_t n, double* acc) {
+  __shared__ double red[2][256];
+  double a = 0, b = 0;
+  for (int64_t i = threadIdx.x; i < n; i += 256) {
+    a += sums[2 * i];
+    b += sums[2 * i + 1];
+  }
+  red[0][threadIdx.x] = a;
+  red[1][threadIdx.x] = b;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if ((int)threadIdx.x < o) {
+      red[0][threadIdx.x] += red[0][threadIdx.x + o];
+      red[1][threadIdx.x] += red[1][threadIdx.x + o];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x < 2) acc[threadIdx.x] += red[threadIdx.x][0];
+}
+
 template <int NC>
 void launch_upd(int mode, const double* Z, int64_t ldz, const double* Vb, const double* win, double* wb, int64_t Kp,
                 int j, int last_col, const KState* ks, AdjState* as, double* partials, cudaStream_t st) {
@@ -335,6 +356,12 @@ cudaError_t launch_adj_bbar_from(const double* Z, const double* Vb, double* bbar
 cudaError_t launch_adj_finish(int kind, int mode, int j, int k, double fdt, const KState* ks, AdjState* as,
                               cudaStream_t st) {
   finish_kernel<<<1, 256, 0, st>>>(kind, mode, j, k, fdt, ks, as);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_theta_sum(const double* sums, int64_t n, double* acc, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  theta_sum_kernel<<<1, 256, 0, st>>>(sums, n, acc);
   return cudaGetLastError();
 }
 

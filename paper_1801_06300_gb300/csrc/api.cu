@@ -70,6 +70,7 @@ struct pcexp_ctx {
          *b_rb = nullptr, *b_gin = nullptr;
   double* b_small = nullptr;  // 2 MMAX^2 doubles: H and Hbar of pcexp_phi_adjoint
   double* b_theta = nullptr;  // adjoint of (Mach, alpha in degrees) of the reverse step (2 doubles)
+  double* b_tsum = nullptr;   // its second-order terms per boundary-face point (ThetaSums)
   KState* b_ks1 = nullptr;
   AdjState* b_as = nullptr;
   KState* ks = nullptr;
@@ -1257,6 +1258,7 @@ int alloc_backward(pcexp_ctx* c) {
   PCEXP_TRY(dalloc(c, &c->b_Vb, Vn));
   PCEXP_TRY(dalloc(c, &c->b_small, (size_t)2 * MMAX * MMAX));
   PCEXP_TRY(dalloc(c, &c->b_theta, 2));
+  PCEXP_TRY(dalloc(c, &c->b_tsum, (size_t)(c->F - c->host.F_interior) * c->nfq * 2 + 1));
   PCEXP_TRY(dalloc(c, &c->b_ks1, 1));
   PCEXP_TRY(dalloc(c, &c->b_as, 1));
   if (c->grp) {  // partition of a group: the reverse reductions are summed over the partitions
@@ -1278,14 +1280,12 @@ void freestream_velocity_derivatives(const pcexp_physics& ph, double dvel[4]) {
   dvel[3] = ph.mach * cinf * std::cos(a) * M_PI / 180.0;
 }
 
-// theta_bar += (d(...)/dtheta)^T w for the reverse step: order 1 with u (R(u)), order 2 with
-// u and t (J(u) t), scaled by osc (and *osc_dev)
-int param_adjoint(pcexp_ctx* c, const DGData<double>& d, int order, const double* u, const double* t, const double* w,
-                  double osc, const double* osc_dev) {
+// theta_bar += osc (dR(u)/dtheta)^T w for the reverse step
+int param_adjoint(pcexp_ctx* c, const DGData<double>& d, const double* u, const double* w, double osc) {
   double dvel[4];
   freestream_velocity_derivatives(c->phys, dvel);
-  PCEXP_CK(launch_param_adjoint<double>(d, c->host.F_interior, order, u, t, w, osc, osc_dev, dvel, c->b_theta,
-                                        c->partials, &c->b_as->counter, c->st));
+  PCEXP_CK(launch_param_adjoint<double>(d, c->host.F_interior, u, w, osc, dvel, c->b_theta, c->partials,
+                                        &c->b_as->counter, c->st));
   return PCEXP_OK;
 }
 
@@ -1336,12 +1336,20 @@ int adj_jt(pcexp_ctx* c, const DGData<double>& d, double* w, double* out) {
 }
 
 // out = (d(J(u) v)/du)^T w at u = b_un (v's and w's halo rows from the owners; v's restored to
-// zero when it is a Krylov vector)
-int adj_hess(pcexp_ctx* c, const DGData<double>& d, double* v, bool v_krylov, double* w, double* out) {
+// zero when it is a Krylov vector); b_tsum += osc (*osc_dev) (d(J(u; theta) v)/dtheta)^T w per
+// boundary-face point
+int adj_hess(pcexp_ctx* c, const DGData<double>& d, double* v, bool v_krylov, double* w, double* out, double osc,
+             const double* osc_dev) {
   PCEXP_TRY(group_exchange<double>(c, v));
   PCEXP_TRY(group_exchange<double>(c, w));
+  ThetaSums<double> th;
+  th.sums = c->b_tsum;
+  th.f0 = c->host.F_interior;
+  th.osc = osc;
+  th.osc_dev = osc_dev;
+  freestream_velocity_derivatives(c->phys, th.dvel);
   PCEXP_CK(launch_jvp_state_adjoint<double>(d, c->b_un, v, w, out, reinterpret_cast<double*>(c->GT), nullptr, 1.0,
-                                            c->st));
+                                            c->st, th));
   if (v_krylov) PCEXP_TRY(group_zero_halo<double>(c, v));
   return group_zero_halo<double>(c, out);
 }
@@ -1357,11 +1365,10 @@ int reverse_krylov(pcexp_ctx* c, const DGData<double>& d, double* Z, const KStat
     // w0 = J_n v_j: vbar_j += J_n^T w0bar;  ubar_n += (d(J(u) v_j)/du)^T w0bar, v_j = s_j z_j
     PCEXP_TRY(adj_jt(c, d, c->b_wb0, c->b_t1));
     PCEXP_CK(launch_axpy(c->b_Vb + (int64_t)j * Kp, c->b_t1, nullptr, 1.0, Kp, c->st));
-    PCEXP_TRY(adj_hess(c, d, Z + (int64_t)j * Kp, true, c->b_wb0, c->b_t2));
+    // (and theta_bar += s_j (d(J(u_n; theta) z_j)/dtheta)^T w0bar)
+    PCEXP_TRY(adj_hess(c, d, Z + (int64_t)j * Kp, true, c->b_wb0, c->b_t2, 1.0, &ks->s[j]));
     PCEXP_CK(launch_axpy(c->b_ubn, c->b_t2, &ks->s[j], 1.0, Kp, c->st));
     PCEXP_TRY(group_zero_halo<double>(c, c->b_wb0));
-    // theta_bar += s_j (d(J(u_n; theta) z_j)/dtheta)^T w0bar
-    PCEXP_TRY(param_adjoint(c, d, 2, c->b_un, Z + (int64_t)j * Kp, c->b_wb0, 1.0, &ks->s[j]));
   }
   PCEXP_CK(launch_adj_b0dot(Z, c->b_Vb, Kp, c->b_as, c->partials, c->st));
   PCEXP_TRY(adj_round(c, ADJ_B0, 0, 0, 0, 0.0, ks));
@@ -1409,6 +1416,7 @@ int step_backward_impl(pcexp_ctx* c, const double* U, double dt, int m, const do
   const int k1 = h1.k, k2 = h2.k;
   // ---- reverse
   PCEXP_CK(cudaMemsetAsync(c->b_theta, 0, 2 * sizeof(double), c->st));
+  PCEXP_CK(cudaMemsetAsync(c->b_tsum, 0, (size_t)(c->F - c->host.F_interior) * c->nfq * 2 * sizeof(double), c->st));
   PCEXP_CK(cudaMemsetAsync(c->b_ubn, 0, vbytes, c->st));
   PCEXP_CK(cudaMemsetAsync(c->b_rb, 0, vbytes, c->st));
   PCEXP_CK(cudaMemsetAsync(c->b_db, 0, vbytes, c->st));
@@ -1421,13 +1429,13 @@ int step_backward_impl(pcexp_ctx* c, const double* U, double dt, int m, const do
     // N_* - N_n = R(u_*) - R_n - J_n delta, with bbar_2 = b_bb
     PCEXP_TRY(adj_jt(c, d, c->b_bb, c->b_t1));
     PCEXP_CK(launch_axpy(c->b_db, c->b_t1, nullptr, -1.0, Kp, c->st));
-    PCEXP_TRY(adj_hess(c, d, c->b_dl, false, c->b_bb, c->b_t2));
+    // theta_bar -= (d(J(u_n; theta) delta)/dtheta)^T bbar_2
+    PCEXP_TRY(adj_hess(c, d, c->b_dl, false, c->b_bb, c->b_t2, -1.0, nullptr));
     PCEXP_CK(launch_axpy(c->b_ubn, c->b_t2, nullptr, -1.0, Kp, c->st));
     PCEXP_TRY(group_zero_halo<double>(c, c->b_bb));
     PCEXP_CK(launch_axpy(c->b_rb, c->b_bb, nullptr, -1.0, Kp, c->st));
-    // theta_bar -= (d(J(u_n; theta) delta)/dtheta)^T bbar_2;  += (dR(u_*; theta)/dtheta)^T bbar_2
-    PCEXP_TRY(param_adjoint(c, d, 2, c->b_un, c->b_dl, c->b_bb, -1.0, nullptr));
-    PCEXP_TRY(param_adjoint(c, d, 1, c->b_us, nullptr, c->b_bb, 1.0, nullptr));
+    // theta_bar += (dR(u_*; theta)/dtheta)^T bbar_2
+    PCEXP_TRY(param_adjoint(c, d, c->b_us, c->b_bb, 1.0));
     PCEXP_TRY(linearize<double>(c, d, c->b_us));
     PCEXP_TRY(adj_jt(c, d, c->b_bb, c->b_t1));
     PCEXP_CK(launch_axpy(c->b_ubs, c->b_t1, nullptr, 1.0, Kp, c->st));
@@ -1447,7 +1455,8 @@ int step_backward_impl(pcexp_ctx* c, const double* U, double dt, int m, const do
   PCEXP_TRY(adj_jt(c, d, c->b_rb, c->b_t1));
   PCEXP_CK(launch_axpy(c->b_ubn, c->b_t1, nullptr, 1.0, Kp, c->st));
   PCEXP_TRY(group_zero_halo<double>(c, c->b_rb));
-  PCEXP_TRY(param_adjoint(c, d, 1, c->b_un, nullptr, c->b_rb, 1.0, nullptr));
+  PCEXP_TRY(param_adjoint(c, d, c->b_un, c->b_rb, 1.0));
+  PCEXP_CK(launch_theta_sum(c->b_tsum, (c->F - c->host.F_interior) * c->nfq, c->b_theta, c->st));
   c->prof = prof;
   PCEXP_TRY(export_vec<double>(c, c->b_ubn, ubar, on_device));
   int aerr = 0;

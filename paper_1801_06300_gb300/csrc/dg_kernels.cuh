@@ -1204,18 +1204,31 @@ cudaError_t jac_adjoint_p(const DGData<T>& d, LinData<T> lin, const T* w, T* out
 }
 
 // ------------------------------------------- second-order adjoint (d(J(u) v)/du)^T w
-// S(u) = w~^T J(u) v is differentiated with respect to the linearisation state u:
-// every flux is evaluated on hyper-dual numbers (value, D+2 seeded partials, the
-// directional derivative along the traces of v, its partials), contracted with the
-// transposed test (volume) or transposed lift (faces) of w~ and mapped back through the
-// transposed traces.  Same output factors and scratch layout as the adjoint kernels.
+// S(u) = w~^T J(u) v is differentiated with respect to the linearisation state u: at every
+// point the transposed test (volume) or transposed lift (faces) of w~ is the adjoint of the flux,
+// the reverse sweep of the flux (roe_flux_vjp, euler_flux_vjp, the ghost states') runs on
+// Tangent numbers carrying the traces of v, and the derivative parts of its results are
+// d/du [w~^T F'(u) v], mapped back through the transposed traces.  Same output factors and
+// scratch layout as the adjoint kernels.
+//
+// Bound by the FP64 pipe (2 FMA per clock and SM).  One sweep serves both sides of a face; on
+// hyper-dual numbers every operation carried 2 (D + 2) + 2 components and each side took a pass
+// of its own.  Bump channel, 6,144 triangles at p = 2, m = 30: the reverse step 48.2 -> 27.0 ms,
+// 61 launches of each kernel (faces 311, elements 67 and the separate free-stream pass 78 us per
+// launch before).
+//
+// theta (nullable): per boundary-face point (faces f0..F) two sums that grow by
+// osc * (*osc_dev) * d/dtheta_k [gbar^T (dF~/dU_L) t_L], theta = (Mach number, flow angle), from the
+// far-field ghost state's adjoint of the free-stream velocity; dvel = {dvel/dMach (x, y),
+// dvel/dalpha (x, y)}.  Each entry belongs to one thread; theta_sum_kernel adds them up.
 template <class T, int D, int P>
 __global__ void __launch_bounds__(128) face_hess_kernel(DGData<T> d, const T* __restrict__ u,
                                                         const T* __restrict__ v, const T* __restrict__ w,
-                                                        T* __restrict__ GT, const T* __restrict__ escale, T osc) {
+                                                        T* __restrict__ GT, const T* __restrict__ escale, T osc,
+                                                        ThetaSums<T> th) {
   using O = Ord<D, P>;
   constexpr int NB = O::NB, NFQ = O::NFQ, NV = O::NV, NPERM = O::NPERM, GEO = O::GEO;
-  using H = HD<T, NV>;
+  using S = Tangent<T>;
   const int64_t n = d.F * NFQ;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n) return;
@@ -1228,13 +1241,13 @@ __global__ void __launch_bounds__(128) face_hess_kernel(DGData<T> d, const T* __
 #pragma unroll
   for (int k = 0; k < D; ++k) nr[k] = d.fgeo[4 * f + k];
   const T wq = d.fgeo[4 * f + D] * d.Wf[q];
-  const T sdL = d.geo[GEO * (int64_t)eL + O::SD];
-  const T sdR = eR >= 0 ? d.geo[GEO * (int64_t)eR + O::SD] : T(1);
+  const T isdL = d.geo[GEO * (int64_t)eL + O::ISD];
+  const T isdR = eR >= 0 ? d.geo[GEO * (int64_t)eR + O::ISD] : T(0);
   const T* bL = d.Bf + ((fL * NPERM) * NFQ + q) * NB;
   const T* bR = d.Bf + ((fR * NPERM + (eR >= 0 ? pR : 0)) * NFQ + q) * NB;
-  T uL[NV], tL[NV], uR[NV], tR[NV], gb[NV];
-  const T scL = -osc * (escale ? escale[eL] : T(1)) / sdL;
-  const T scR = osc * (eR >= 0 && escale ? escale[eR] : T(1)) / sdR;
+  S L[NV], R[NV];
+  T gb[NV];
+  const T scL = -osc * (escale ? escale[eL] : T(1)) * isdL;
 #pragma unroll
   for (int c = 0; c < NV; ++c) {
     T a = 0, b = 0, g = 0;
@@ -1246,12 +1259,11 @@ __global__ void __launch_bounds__(128) face_hess_kernel(DGData<T> d, const T* __
       b += bj * v[o];
       g += bj * w[o];
     }
-    uL[c] = a / sdL;
-    tL[c] = b / sdL;
+    L[c] = S{a * isdL, b * isdL};
     gb[c] = scL * g;
-    uR[c] = tR[c] = T(0);
   }
   if (eR >= 0) {
+    const T scR = osc * (escale ? escale[eR] : T(1)) * isdR;
 #pragma unroll
     for (int c = 0; c < NV; ++c) {
       T a = 0, b = 0, g = 0;
@@ -1263,55 +1275,39 @@ __global__ void __launch_bounds__(128) face_hess_kernel(DGData<T> d, const T* __
         b += bj * v[o];
         g += bj * w[o];
       }
-      uR[c] = a / sdR;
-      tR[c] = b / sdR;
+      R[c] = S{a * isdR, b * isdR};
       gb[c] += scR * g;
+    }
+  } else if (mirror_bc(eR)) {
+    ghost_slip_wall<D, S, T>(L, nr, R);
+  } else {
+    ghost_farfield<D, S, T>(L, nr, d.fs, R);
+  }
+  S Lb[NV], Rb[NV];
+#pragma unroll
+  for (int c = 0; c < NV; ++c) Lb[c] = Rb[c] = S{T(0), T(0)};
+  roe_flux_vjp<D, S, T>(L, R, nr, d.fs.gamma, gb, Lb, Rb);
+  if (eR < 0) {
+    if (mirror_bc(eR)) {
+      ghost_slip_wall_vjp<D, S, T>(nr, Rb, Lb);
+    } else {
+      S vib[D];
+#pragma unroll
+      for (int k = 0; k < D; ++k) vib[k] = S{T(0), T(0)};
+      ghost_farfield_vjp<D, S, T>(L, nr, d.fs, Rb, Lb, vib);
+      if (th.sums && eL < d.E_loc) {  // a halo element's faces count in their own partition
+        const T sc = th.osc * (th.osc_dev ? *th.osc_dev : T(1)) * wq;
+        T* o = th.sums + ((f - th.f0) * NFQ + q) * 2;
+        o[0] += sc * (th.dvel[0] * vib[0].d + th.dvel[1] * vib[1].d);
+        o[1] += sc * (th.dvel[2] * vib[0].d + th.dvel[3] * vib[1].d);
+      }
     }
   }
   T* o = GT + idx * 2 * NV;
-#pragma unroll 1
-  for (int side = 0; side < 2; ++side) {
-    if (side == 1 && eR < 0) {
 #pragma unroll
-      for (int c = 0; c < NV; ++c) o[NV + c] = T(0);
-      break;
-    }
-    H L[NV], R[NV], F[NV];
-#pragma unroll
-    for (int c = 0; c < NV; ++c) {
-      L[c].v = uL[c];
-      L[c].t = tL[c];
-#pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        L[c].d[k] = (side == 0 && k == c) ? T(1) : T(0);
-        L[c].dt[k] = T(0);
-      }
-    }
-    if (eR >= 0) {
-#pragma unroll
-      for (int c = 0; c < NV; ++c) {
-        R[c].v = uR[c];
-        R[c].t = tR[c];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-          R[c].d[k] = (side == 1 && k == c) ? T(1) : T(0);
-          R[c].dt[k] = T(0);
-        }
-      }
-    } else if (mirror_bc(eR)) {
-      ghost_slip_wall<D, H, T>(L, nr, R);
-    } else {
-      ghost_farfield<D, H, T>(L, nr, d.fs, R);
-    }
-    roe_flux<D, H, T>(L, R, nr, d.fs.gamma, F);
-    const T sc = wq / (side == 0 ? sdL : sdR);
-#pragma unroll
-    for (int c = 0; c < NV; ++c) {
-      T a = 0;
-#pragma unroll
-      for (int vv = 0; vv < NV; ++vv) a += gb[vv] * F[vv].dt[c];
-      o[side * NV + c] = sc * a;
-    }
+  for (int c = 0; c < NV; ++c) {
+    o[c] = wq * isdL * Lb[c].d;
+    o[NV + c] = eR >= 0 ? wq * isdR * Rb[c].d : T(0);
   }
 }
 
@@ -1322,7 +1318,7 @@ __global__ void __launch_bounds__(256) elem_hess_kernel(DGData<T> d, const T* __
   using O = Ord<D, P>;
   constexpr int NB = O::NB, NQ = O::NQ, ET = O::ET, NVB = O::NVB, NV = O::NV, GEO = O::GEO;
   constexpr bool SM = O::SMEM_BF;
-  using H = HD<T, NV>;
+  using S = Tangent<T>;
   __shared__ T sBv[NQ * NB];
   __shared__ T sDv[D * NQ * NB];
   __shared__ T sBf[SM ? O::NBF : 1];
@@ -1348,8 +1344,9 @@ __global__ void __launch_bounds__(256) elem_hess_kernel(DGData<T> d, const T* __
   const int el1 = threadIdx.x / NQ, q1 = threadIdx.x - (threadIdx.x / NQ) * NQ;
   if (threadIdx.x < ne * NQ) {
     const T* ge = sgeo + el1 * GEO;
-    const T sd = ge[O::SD];
-    H U[NV];
+    const T isd = ge[O::ISD];
+    S U[NV], Ub[NV];
+    T fb[D][NV];
 #pragma unroll
     for (int c = 0; c < NV; ++c) {
       T a = 0, b = 0;
@@ -1358,40 +1355,28 @@ __global__ void __launch_bounds__(256) elem_hess_kernel(DGData<T> d, const T* __
         a += sBv[q1 * NB + j] * su[el1 * NVB + c * NB + j];
         b += sBv[q1 * NB + j] * sv[el1 * NVB + c * NB + j];
       }
-      U[c].v = a / sd;
-      U[c].t = b;  // the sqrt(det) factors of trace and test cancel
+      U[c] = S{a * isd, b};  // the sqrt(det) factors of trace and test cancel
+      Ub[c] = S{T(0), T(0)};
+      // adjoint of the flux along the Cartesian axes: the transposed test, mapped by A^-1
+      T t[D];
 #pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        U[c].d[k] = (k == c) ? T(1) : T(0);
-        U[c].dt[k] = T(0);
-      }
-    }
-    H F[D][NV];
-    euler_flux<D, H, T>(U, d.fs.gamma, F);
-    T fb[D * NV];
+      for (int dd = 0; dd < D; ++dd) {
+        T h = 0;
 #pragma unroll
-    for (int dd = 0; dd < D; ++dd)
-#pragma unroll
-      for (int vv = 0; vv < NV; ++vv) {
-        T a = 0;
-#pragma unroll
-        for (int i = 0; i < NB; ++i) a += sDv[(dd * NQ + q1) * NB + i] * sw[el1 * NVB + vv * NB + i];
-        fb[dd * NV + vv] = a;
+        for (int i = 0; i < NB; ++i) h += sDv[(dd * NQ + q1) * NB + i] * sw[el1 * NVB + c * NB + i];
+        t[dd] = h;
       }
 #pragma unroll
-    for (int c = 0; c < NV; ++c) {
-      T a = 0;
+      for (int k = 0; k < D; ++k) {
+        T h = ge[k] * t[0];
 #pragma unroll
-      for (int vv = 0; vv < NV; ++vv)
-#pragma unroll
-        for (int dd = 0; dd < D; ++dd) {
-          T fm = ge[dd * D] * F[0][vv].dt[c];
-#pragma unroll
-          for (int k = 1; k < D; ++k) fm += ge[dd * D + k] * F[k][vv].dt[c];
-          a += fb[dd * NV + vv] * fm;
-        }
-      sU[(el1 * NQ + q1) * NV + c] = a / sd;
+        for (int dd = 1; dd < D; ++dd) h += ge[dd * D + k] * t[dd];
+        fb[k][c] = h;
+      }
     }
+    euler_flux_vjp<D, S, T>(U, d.fs.gamma, fb, Ub);
+#pragma unroll
+    for (int c = 0; c < NV; ++c) sU[(el1 * NQ + q1) * NV + c] = Ub[c].d * isd;
   }
   __syncthreads();
   const T* Bf = SM ? sBf : d.Bf;
@@ -1408,10 +1393,10 @@ __global__ void __launch_bounds__(256) elem_hess_kernel(DGData<T> d, const T* __
 
 template <class T, int D, int P>
 cudaError_t jvp_state_adjoint_p(const DGData<T>& d, const T* u, const T* v, const T* w, T* out, T* GT,
-                                const T* escale, T osc, cudaStream_t st) {
+                                const T* escale, T osc, cudaStream_t st, const ThetaSums<T>& th) {
   using O = Ord<D, P>;
   const int64_t nf = d.F * O::NFQ;
-  if (nf > 0) face_hess_kernel<T, D, P><<<(unsigned)((nf + 127) / 128), 128, 0, st>>>(d, u, v, w, GT, escale, osc);
+  if (nf > 0) face_hess_kernel<T, D, P><<<(unsigned)((nf + 127) / 128), 128, 0, st>>>(d, u, v, w, GT, escale, osc, th);
   const int64_t eb = (d.E + O::ET - 1) / O::ET;
   elem_hess_kernel<T, D, P><<<(unsigned)eb, 256, 0, st>>>(d, u, v, w, GT, out, escale, osc);
   return cudaGetLastError();
@@ -1421,18 +1406,15 @@ cudaError_t jvp_state_adjoint_p(const DGData<T>& d, const T* u, const T* v, cons
 // theta = (Mach number, flow angle in degrees) enters the operator only through the
 // free-stream velocity of the far-field ghost state.  For the far-field faces (indices >= f0)
 // this kernel adds to acc[0..1]
-//   order 1:  sum_q sum_v gbar_q[v] dF~_v/dtheta_k                       ((dR/dtheta)^T w)
-//   order 2:  sum_q sum_v gbar_q[v] d/dtheta_k (dF~_v/dU_L . t_L)          ((d(J t)/dtheta)^T w)
-// with gbar_q[v] = -osc |f| w_q / sqrt|det A_L| sum_i phi_i(x_q) w[e_L][v][i] (the transposed lift
-// of w, the face term of R at the L element) and t_L the trace of t.  Jet numbers seeded on
-// the velocity give the first derivatives, hyper-dual numbers (velocity seeds, tangent t_L)
-// the mixed second ones.  dvel = {dvel/dMach (D), dvel/dalpha (D)}.  osc_dev (nullable)
-// multiplies osc.  Fixed-order sum: per-block partials, the last block adds them to acc.
-template <class T, int D, int P, int ORDER>
+//   osc sum_q sum_v gbar_q[v] dF~_v/dtheta_k                       (osc (dR/dtheta)^T w)
+// with gbar_q[v] = -|f| w_q / sqrt|det A_L| sum_i phi_i(x_q) w[e_L][v][i] (the transposed lift
+// of w, the face term of R at the L element).  Jet numbers seeded on the velocity give the
+// derivatives.  dvel = {dvel/dMach (D), dvel/dalpha (D)}.  Fixed-order sum: per-block partials,
+// the last block adds them to acc.
+template <class T, int D, int P>
 __global__ void __launch_bounds__(128) param_adjoint_kernel(DGData<T> d, int64_t f0, const T* __restrict__ u,
-                                                            const T* __restrict__ t, const T* __restrict__ w,
-                                                            double osc, const double* __restrict__ osc_dev,
-                                                            double dvm0, double dvm1, double dva0, double dva1,
+                                                            const T* __restrict__ w, double osc, double dvm0,
+                                                            double dvm1, double dva0, double dva1,
                                                             double* __restrict__ acc, double* __restrict__ partials,
                                                             unsigned* counter) {
   using O = Ord<D, P>;
@@ -1440,7 +1422,6 @@ __global__ void __launch_bounds__(128) param_adjoint_kernel(DGData<T> d, int64_t
   __shared__ double red[2][4];
   __shared__ bool last;
   double a0 = 0.0, a1 = 0.0;
-  const double os = osc * (osc_dev ? *osc_dev : 1.0);
   const int64_t n = (d.F - f0) * NFQ;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += (int64_t)gridDim.x * blockDim.x) {
     const int64_t f = f0 + idx / NFQ;
@@ -1454,62 +1435,37 @@ __global__ void __launch_bounds__(128) param_adjoint_kernel(DGData<T> d, int64_t
     const T isd = d.geo[GEO * (int64_t)eL + O::ISD];
     const T* be = d.Bf + ((fL * NPERM) * NFQ + q) * NB;
     const T wl = d.fgeo[4 * f + D] * d.Wf[q];
-    T uL[NV], tL[NV], gb[NV];
+    T uL[NV], gb[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      T a = 0, b = 0, c = 0;
+      T a = 0, c = 0;
 #pragma unroll
       for (int j = 0; j < NB; ++j) {
         const T bj = __ldg(be + j);
         const int64_t o = (int64_t)eL * NV * NB + v * NB + j;
         a += bj * u[o];
-        if (ORDER == 2) b += bj * t[o];
         c += bj * w[o];
       }
       uL[v] = a * isd;
-      tL[v] = b * isd;
-      gb[v] = (T)(-os) * wl * isd * c;
+      gb[v] = (T)(-osc) * wl * isd * c;
     }
     const double dm[3] = {dvm0, dvm1, 0.0}, da[3] = {dva0, dva1, 0.0};
-    if constexpr (ORDER == 1) {
-      using J = Jet<T, 2>;
-      J L[NV], R[NV], F[NV], vi[3];
+    using J = Jet<T, 2>;
+    J L[NV], R[NV], F[NV], vi[3];
 #pragma unroll
-      for (int v = 0; v < NV; ++v) L[v] = Lift<J, T>::of(uL[v]);
+    for (int v = 0; v < NV; ++v) L[v] = Lift<J, T>::of(uL[v]);
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        vi[k].v = d.fs.vel[k];
-        vi[k].d[0] = (T)dm[k];
-        vi[k].d[1] = (T)da[k];
-      }
-      ghost_farfield_v<D, J, T>(L, nr, d.fs.gamma, d.fs.rho, d.fs.p, vi, R);
-      roe_flux<D, J, T>(L, R, nr, d.fs.gamma, F);
+    for (int k = 0; k < 3; ++k) {
+      vi[k].v = d.fs.vel[k];
+      vi[k].d[0] = (T)dm[k];
+      vi[k].d[1] = (T)da[k];
+    }
+    ghost_farfield_v<D, J, T>(L, nr, d.fs.gamma, d.fs.rho, d.fs.p, vi, R);
+    roe_flux<D, J, T>(L, R, nr, d.fs.gamma, F);
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        a0 += (double)gb[v] * (double)F[v].d[0];
-        a1 += (double)gb[v] * (double)F[v].d[1];
-      }
-    } else {
-      using H = HD<T, 2>;
-      H L[NV], R[NV], F[NV], vi[3];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        L[v] = Lift<H, T>::of(uL[v]);
-        L[v].t = tL[v];
-      }
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        vi[k] = Lift<H, T>::of(d.fs.vel[k]);
-        vi[k].d[0] = (T)dm[k];
-        vi[k].d[1] = (T)da[k];
-      }
-      ghost_farfield_v<D, H, T>(L, nr, d.fs.gamma, d.fs.rho, d.fs.p, vi, R);
-      roe_flux<D, H, T>(L, R, nr, d.fs.gamma, F);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        a0 += (double)gb[v] * (double)F[v].dt[0];
-        a1 += (double)gb[v] * (double)F[v].dt[1];
-      }
+    for (int v = 0; v < NV; ++v) {
+      a0 += (double)gb[v] * (double)F[v].d[0];
+      a1 += (double)gb[v] * (double)F[v].d[1];
     }
   }
   for (int o = 16; o > 0; o >>= 1) {
@@ -1546,19 +1502,14 @@ __global__ void __launch_bounds__(128) param_adjoint_kernel(DGData<T> d, int64_t
 }
 
 template <class T, int D, int P>
-cudaError_t param_adjoint_p(const DGData<T>& d, int64_t f0, int order, const T* u, const T* t, const T* w, double osc,
-                            const double* osc_dev, const double* dvel, double* acc, double* partials,
-                            unsigned* counter, cudaStream_t st) {
+cudaError_t param_adjoint_p(const DGData<T>& d, int64_t f0, const T* u, const T* w, double osc, const double* dvel,
+                            double* acc, double* partials, unsigned* counter, cudaStream_t st) {
   const int64_t n = (d.F - f0) * Ord<D, P>::NFQ;
   if (n <= 0) return cudaSuccess;
   int64_t g = (n + 127) / 128;
   if (g > RED_BLOCKS) g = RED_BLOCKS;
-  if (order == 1)
-    param_adjoint_kernel<T, D, P, 1><<<(unsigned)g, 128, 0, st>>>(d, f0, u, t, w, osc, osc_dev, dvel[0], dvel[1],
-                                                                   dvel[2], dvel[3], acc, partials, counter);
-  else
-    param_adjoint_kernel<T, D, P, 2><<<(unsigned)g, 128, 0, st>>>(d, f0, u, t, w, osc, osc_dev, dvel[0], dvel[1],
-                                                                   dvel[2], dvel[3], acc, partials, counter);
+  param_adjoint_kernel<T, D, P><<<(unsigned)g, 128, 0, st>>>(d, f0, u, w, osc, dvel[0], dvel[1], dvel[2], dvel[3], acc,
+                                                             partials, counter);
   return cudaGetLastError();
 }
 
@@ -1895,15 +1846,15 @@ cudaError_t launch_jac_adjoint_d(const DGData<T>& d, LinData<T> lin, const T* w,
 }
 template <class T, int D>
 cudaError_t launch_jvp_state_adjoint_d(const DGData<T>& d, const T* u, const T* v, const T* w, T* out, T* GT,
-                                       const T* escale, T osc, cudaStream_t st) {
-  PCEXP_PSWITCH(D, (jvp_state_adjoint_p<T, D, P_>(d, u, v, w, out, GT, escale, osc, st)))
+                                       const T* escale, T osc, cudaStream_t st, const ThetaSums<T>& th) {
+  PCEXP_PSWITCH(D, (jvp_state_adjoint_p<T, D, P_>(d, u, v, w, out, GT, escale, osc, st, th)))
 }
 
 template <class T, int D>
-cudaError_t launch_param_adjoint_d(const DGData<T>& d, int64_t f0, int order, const T* u, const T* t, const T* w,
-                                   double osc, const double* osc_dev, const double* dvel, double* acc,
-                                   double* partials, unsigned* counter, cudaStream_t st) {
-  PCEXP_PSWITCH(D, (param_adjoint_p<T, D, P_>(d, f0, order, u, t, w, osc, osc_dev, dvel, acc, partials, counter, st)))
+cudaError_t launch_param_adjoint_d(const DGData<T>& d, int64_t f0, const T* u, const T* w, double osc,
+                                   const double* dvel, double* acc, double* partials, unsigned* counter,
+                                   cudaStream_t st) {
+  PCEXP_PSWITCH(D, (param_adjoint_p<T, D, P_>(d, f0, u, w, osc, dvel, acc, partials, counter, st)))
 }
 
 template <class T, int D, int P>
@@ -1970,7 +1921,7 @@ cudaError_t launch_local_dt_d(const DGData<T>& d, const T* u, const double* cfl_
   template cudaError_t launch_jac_adjoint_d<T, D>(const DGData<T>&, LinData<T>, const T*, T*, T*, const T*, T,     \
                                                   cudaStream_t);                                                   \
   template cudaError_t launch_jvp_state_adjoint_d<T, D>(const DGData<T>&, const T*, const T*, const T*, T*, T*,    \
-                                                        const T*, T, cudaStream_t);                                \
+                                                        const T*, T, cudaStream_t, const ThetaSums<T>&);           \
   template cudaError_t launch_wall_force_d<T, D>(const DGData<T>&, int64_t, const T*, double, double, double,      \
                                                  double*, double*, double*, unsigned*, cudaStream_t);              \
   template cudaError_t launch_vortex_error_d<T, D>(const DGData<T>&, const T*, const double*, const double*,       \
@@ -1979,8 +1930,7 @@ cudaError_t launch_local_dt_d(const DGData<T>& d, const T* u, const double* cfl_
                                                double*, unsigned*, cudaStream_t);                                  \
   template cudaError_t launch_vortex_param_grad_d<T, D>(const DGData<T>&, const T*, const double*, const double*,   \
                                                         const double*, double*, double*, unsigned*, cudaStream_t); \
-  template cudaError_t launch_param_adjoint_d<T, D>(const DGData<T>&, int64_t, int, const T*, const T*, const T*,  \
-                                                    double, const double*, const double*, double*, double*,        \
-                                                    unsigned*, cudaStream_t);
+  template cudaError_t launch_param_adjoint_d<T, D>(const DGData<T>&, int64_t, const T*, const T*, double,         \
+                                                    const double*, double*, double*, unsigned*, cudaStream_t);
 
 }  // namespace pcexp

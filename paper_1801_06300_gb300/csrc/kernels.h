@@ -118,6 +118,17 @@ struct LinData {
   T* Bface;
 };
 
+// Running sums of the free-stream adjoint of the second-order terms (face_hess_kernel): two
+// entries (Mach number, flow angle) per boundary-face point, face index >= f0; sums == nullptr: none.
+template <class T>
+struct ThetaSums {
+  T* sums = nullptr;
+  int64_t f0 = 0;
+  T osc = T(0);
+  const T* osc_dev = nullptr;
+  T dvel[4] = {T(0), T(0), T(0), T(0)};  // d(free-stream velocity)/dMach (x, y), then d/dalpha (x, y)
+};
+
 // ---- DG operator (dg_kernels.cuh, instantiated per dimension in dg2d.cu / dg3d.cu)
 template <class T, int D>
 cudaError_t launch_dg_operator_d(const DGData<T>& d, const T* u, const T* du, T* out, T* G, const T* escale,
@@ -135,7 +146,7 @@ cudaError_t launch_jac_adjoint_d(const DGData<T>& d, LinData<T> lin, const T* w,
                                  T osc, cudaStream_t st);
 template <class T, int D>
 cudaError_t launch_jvp_state_adjoint_d(const DGData<T>& d, const T* u, const T* v, const T* w, T* out, T* GT,
-                                       const T* escale, T osc, cudaStream_t st);
+                                       const T* escale, T osc, cudaStream_t st, const ThetaSums<T>& th);
 template <class T, int D>
 cudaError_t launch_wall_force_d(const DGData<T>& d, int64_t f0, const T* u, double ax, double ay, double az,
                                 double* grad, double* value, double* partials, unsigned* counter, cudaStream_t st);
@@ -143,9 +154,9 @@ template <class T, int D>
 cudaError_t launch_vortex_error_d(const DGData<T>& d, const T* u, const double* xq, const double* prm, double* grad,
                                   double* value, double* partials, unsigned* counter, cudaStream_t st);
 template <class T, int D>
-cudaError_t launch_param_adjoint_d(const DGData<T>& d, int64_t f0, int order, const T* u, const T* t, const T* w,
-                                   double osc, const double* osc_dev, const double* dvel, double* acc,
-                                   double* partials, unsigned* counter, cudaStream_t st);
+cudaError_t launch_param_adjoint_d(const DGData<T>& d, int64_t f0, const T* u, const T* w, double osc,
+                                   const double* dvel, double* acc, double* partials, unsigned* counter,
+                                   cudaStream_t st);
 template <class T, int D>
 cudaError_t launch_vortex_param_grad_d(const DGData<T>& d, const T* u, const double* xq, const double* prm,
                                        const double* dvel, double* out, double* partials, unsigned* counter,
@@ -202,9 +213,9 @@ cudaError_t launch_jac_adjoint(const DGData<T>& d, LinData<T> lin, const T* w, T
 // out = (d/du [ (osc diag(escale) J(u) v)^T w ])^T, the second-order adjoint; GT scratch [F][nfq][2 NV].
 template <class T>
 cudaError_t launch_jvp_state_adjoint(const DGData<T>& d, const T* u, const T* v, const T* w, T* out, T* GT,
-                                     const T* escale, T osc, cudaStream_t st) {
-  return d.dim == 3 ? launch_jvp_state_adjoint_d<T, 3>(d, u, v, w, out, GT, escale, osc, st)
-                    : launch_jvp_state_adjoint_d<T, 2>(d, u, v, w, out, GT, escale, osc, st);
+                                     const T* escale, T osc, cudaStream_t st, const ThetaSums<T>& th = {}) {
+  return d.dim == 3 ? launch_jvp_state_adjoint_d<T, 3>(d, u, v, w, out, GT, escale, osc, st, th)
+                    : launch_jvp_state_adjoint_d<T, 2>(d, u, v, w, out, GT, escale, osc, st, th);
 }
 // Pressure force on the slip walls along (ax, ay, az) -> *value, gradient added into grad
 // (nullable); boundary faces are those with index >= f0.
@@ -229,16 +240,17 @@ cudaError_t launch_local_dt(const DGData<T>& d, const T* u, const double* cfl_de
   return d.dim == 3 ? launch_local_dt_d<T, 3>(d, u, cfl_dev, cfl, dte, dtmin, partials, counter, st)
                     : launch_local_dt_d<T, 2>(d, u, cfl_dev, cfl, dte, dtmin, partials, counter, st);
 }
-// acc[0..1] += adjoint with respect to (Mach, alpha in degrees) of the far-field faces (index >= f0):
-// order 1: (dR(u)/dtheta)^T w; order 2: (d(J(u) t)/dtheta)^T w; both times osc (and *osc_dev).
-// dvel: d(free-stream velocity)/dMach (x, y), then d/dalpha (x, y).
+// acc[0..1] += osc (dR(u)/dtheta)^T w, theta = (Mach, alpha in degrees), of the far-field faces
+// (index >= f0).  dvel: d(free-stream velocity)/dMach (x, y), then d/dalpha (x, y).
 template <class T>
-cudaError_t launch_param_adjoint(const DGData<T>& d, int64_t f0, int order, const T* u, const T* t, const T* w,
-                                 double osc, const double* osc_dev, const double* dvel, double* acc, double* partials,
-                                 unsigned* counter, cudaStream_t st) {
-  return d.dim == 3 ? launch_param_adjoint_d<T, 3>(d, f0, order, u, t, w, osc, osc_dev, dvel, acc, partials, counter, st)
-                    : launch_param_adjoint_d<T, 2>(d, f0, order, u, t, w, osc, osc_dev, dvel, acc, partials, counter, st);
+cudaError_t launch_param_adjoint(const DGData<T>& d, int64_t f0, const T* u, const T* w, double osc,
+                                 const double* dvel, double* acc, double* partials, unsigned* counter,
+                                 cudaStream_t st) {
+  return d.dim == 3 ? launch_param_adjoint_d<T, 3>(d, f0, u, w, osc, dvel, acc, partials, counter, st)
+                    : launch_param_adjoint_d<T, 2>(d, f0, u, w, osc, dvel, acc, partials, counter, st);
 }
+// acc[0..1] += the sums of ThetaSums over its n boundary-face points (fixed order)
+cudaError_t launch_theta_sum(const double* sums, int64_t n, double* acc, cudaStream_t st);
 // out[0] = sum w |U_h - U_ex|^2, out[1..3] = sum w (U_h - U_ex) . dU_ex/d(Mach, alpha, eps) for the
 // vortex-error functional (prm: eps, x_c, y_c, period, t; dvel as for launch_param_adjoint)
 template <class T>

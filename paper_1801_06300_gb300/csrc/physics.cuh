@@ -1,7 +1,7 @@
 // Euler physics for the DG kernels (Sec. 4.1, 4.4 of the paper), written once
 // over the dimension D (2 or 3; D + 2 conservative variables) and over a scalar
 // type S that is a real type (the residual), Tangent<T> (value + directional
-// derivative: J v), Jet<T, N> (point Jacobians) or HD<T, N> (second order).
+// derivative: J v; through the reverse sweeps, second order) or Jet<T, N> (point Jacobians).
 //
 // Riemann flux: Roe's solver with square-root-density averages and no entropy
 // fix, F~ = 1/2 (F_n(U_L) + F_n(U_R)) - 1/2 sum_k |lambda_k| alpha_k r_k.
@@ -175,111 +175,6 @@ template <class T, int N> struct Lift<Jet<T, N>, T> {
     r.v = x;
 #pragma unroll
     for (int k = 0; k < N; ++k) r.d[k] = T(0);
-    return r;
-  }
-};
-
-// ------------------------------------------------------- hyper-dual (second order)
-// HD<T, N>: value v, partials d[c] along N seeded directions, the directional
-// derivative t along one more direction, and the partials dt[c] of t.  Running a
-// flux on HD gives d/dU_c (dF/dU . t): the second-order term needed by the adjoint of
-// a Jacobian-vector product with respect to the linearisation state.
-template <class T, int N>
-struct HD {
-  T v;
-  T d[N];
-  T t;
-  T dt[N];
-};
-template <class T, int N> PCEXP_DEV T val(const HD<T, N>& x) { return x.v; }
-template <class T, int N> PCEXP_DEV HD<T, N> operator+(const HD<T, N>& a, const HD<T, N>& b) {
-  HD<T, N> r;
-  r.v = a.v + b.v;
-  r.t = a.t + b.t;
-#pragma unroll
-  for (int c = 0; c < N; ++c) {
-    r.d[c] = a.d[c] + b.d[c];
-    r.dt[c] = a.dt[c] + b.dt[c];
-  }
-  return r;
-}
-template <class T, int N> PCEXP_DEV HD<T, N> operator-(const HD<T, N>& a) {
-  HD<T, N> r;
-  r.v = -a.v;
-  r.t = -a.t;
-#pragma unroll
-  for (int c = 0; c < N; ++c) {
-    r.d[c] = -a.d[c];
-    r.dt[c] = -a.dt[c];
-  }
-  return r;
-}
-template <class T, int N> PCEXP_DEV HD<T, N> operator-(const HD<T, N>& a, const HD<T, N>& b) { return a + (-b); }
-template <class T, int N> PCEXP_DEV HD<T, N> operator*(const HD<T, N>& a, const HD<T, N>& b) {
-  HD<T, N> r;
-  r.v = a.v * b.v;
-  r.t = a.t * b.v + a.v * b.t;
-#pragma unroll
-  for (int c = 0; c < N; ++c) {
-    r.d[c] = a.d[c] * b.v + a.v * b.d[c];
-    r.dt[c] = a.dt[c] * b.v + a.t * b.d[c] + a.d[c] * b.t + a.v * b.dt[c];
-  }
-  return r;
-}
-template <class T, int N> PCEXP_DEV HD<T, N> operator*(const HD<T, N>& a, T b) {
-  HD<T, N> r;
-  r.v = a.v * b;
-  r.t = a.t * b;
-#pragma unroll
-  for (int c = 0; c < N; ++c) {
-    r.d[c] = a.d[c] * b;
-    r.dt[c] = a.dt[c] * b;
-  }
-  return r;
-}
-template <class T, int N> PCEXP_DEV HD<T, N> operator*(T a, const HD<T, N>& b) { return b * a; }
-template <class T, int N> PCEXP_DEV HD<T, N> operator+(const HD<T, N>& a, T b) { HD<T, N> r = a; r.v += b; return r; }
-template <class T, int N> PCEXP_DEV HD<T, N> operator+(T a, const HD<T, N>& b) { HD<T, N> r = b; r.v += a; return r; }
-template <class T, int N> PCEXP_DEV HD<T, N> operator-(const HD<T, N>& a, T b) { HD<T, N> r = a; r.v -= b; return r; }
-template <class T, int N> PCEXP_DEV HD<T, N> operator-(T a, const HD<T, N>& b) { return (-b) + a; }
-// f(a) from f, f', f'' at a.v
-template <class T, int N> PCEXP_DEV HD<T, N> hd_apply(const HD<T, N>& a, T f0, T f1, T f2) {
-  HD<T, N> r;
-  r.v = f0;
-  r.t = f1 * a.t;
-#pragma unroll
-  for (int c = 0; c < N; ++c) {
-    r.d[c] = f1 * a.d[c];
-    r.dt[c] = f1 * a.dt[c] + f2 * a.d[c] * a.t;
-  }
-  return r;
-}
-template <class T, int N> PCEXP_DEV HD<T, N> hd_inv(const HD<T, N>& a) {
-  const T i = T(1) / a.v;
-  return hd_apply(a, i, -i * i, T(2) * i * i * i);
-}
-template <class T, int N> PCEXP_DEV HD<T, N> operator/(const HD<T, N>& a, const HD<T, N>& b) { return a * hd_inv(b); }
-template <class T, int N> PCEXP_DEV HD<T, N> operator/(const HD<T, N>& a, T b) { return a * (T(1) / b); }
-template <class T, int N> PCEXP_DEV HD<T, N> operator/(T a, const HD<T, N>& b) { return hd_inv(b) * a; }
-template <class T, int N> PCEXP_DEV HD<T, N> sqrt_s(const HD<T, N>& a) {
-  const T s = sqrt_s(a.v);
-  return hd_apply(a, s, T(0.5) / s, T(-0.25) / (s * a.v));
-}
-template <class T, int N> PCEXP_DEV HD<T, N> abs_s(const HD<T, N>& a) {
-  const T sg = a.v > T(0) ? T(1) : (a.v < T(0) ? T(-1) : T(0));
-  return hd_apply(a, sg * a.v, sg, T(0));
-}
-template <class T, int N> PCEXP_DEV HD<T, N> pow_s(const HD<T, N>& a, T e) {
-  const T p = pow_s(a.v, e);
-  return hd_apply(a, p, e * p / a.v, e * (e - T(1)) * p / (a.v * a.v));
-}
-template <class T, int N> struct Lift<HD<T, N>, T> {
-  PCEXP_DEV static HD<T, N> of(T x) {
-    HD<T, N> r;
-    r.v = x;
-    r.t = T(0);
-#pragma unroll
-    for (int c = 0; c < N; ++c) r.d[c] = r.dt[c] = T(0);
     return r;
   }
 };
@@ -502,6 +397,306 @@ PCEXP_DEV void ghost_farfield_v(const S (&U)[D + 2], const T (&n)[D], T g, T rho
     kb = kb + vb * vb;
   }
   G[NV - 1] = pb / gm + T(0.5) * rb * kb;
+}
+
+// ------------------------------------------------------------ reverse mode of the fluxes
+// Each *_vjp takes the adjoint of an output and adds the adjoints of the inputs, the exact
+// transpose of the forward function (sign(0) = 0 for |x|).  One evaluation costs two to three
+// forward ones, whatever the number of inputs.  On S = Tangent<T> with the inputs' tangents t, the
+// derivative parts of the results are d/dU [ybar^T F'(U) t]: the second-order term of the reverse
+// step, without seeding a direction per input (hyper-dual numbers carry 2 (D + 2) + 2 components
+// through every operation and need a pass per side).
+template <class T> PCEXP_DEV T sign_of(T x) { return x > T(0) ? T(1) : (x < T(0) ? T(-1) : T(0)); }
+
+// Fb[d][v]: adjoint of the flux along axis d (no state in it); Ub += dF^T Fb
+template <int D, class S, class T>
+PCEXP_DEV void euler_flux_vjp(const S (&U)[D + 2], T g, const T (&Fb)[D][D + 2], S (&Ub)[D + 2]) {
+  constexpr int NV = D + 2;
+  const T gm = g - T(1);
+  const S ir = T(1) / U[0];
+  S vel[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) vel[d] = U[1 + d] * ir;
+  S ke = U[1] * vel[0];
+#pragma unroll
+  for (int d = 1; d < D; ++d) ke = ke + U[1 + d] * vel[d];
+  const S e = U[NV - 1] + gm * (U[NV - 1] - T(0.5) * ke);
+  T trace = Fb[0][1];
+#pragma unroll
+  for (int d = 1; d < D; ++d) trace += Fb[d][1 + d];
+  S eb = Fb[0][NV - 1] * vel[0];
+#pragma unroll
+  for (int d = 1; d < D; ++d) eb = eb + Fb[d][NV - 1] * vel[d];
+  const S pb = eb + trace;
+  const S keb = (T(-0.5) * gm) * pb;
+  S irb = Lift<S, T>::of(T(0));
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    S vb = keb * U[1 + d] + Fb[d][NV - 1] * e;
+    S mb = keb * vel[d] + Fb[d][0];
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+      vb = vb + Fb[d][1 + k] * U[1 + k];
+      mb = mb + Fb[k][1 + d] * vel[k];
+    }
+    Ub[1 + d] = Ub[1 + d] + mb + vb * ir;
+    irb = irb + vb * U[1 + d];
+  }
+  Ub[NV - 1] = Ub[NV - 1] + eb + gm * pb;
+  Ub[0] = Ub[0] - ir * ir * irb;
+}
+
+// adjoints of one side's state from those of its Roe-flux intermediates: rho, velocity, pressure,
+// total enthalpy H, energy E (mass row and momenta already in Ub)
+template <int D, class S, class T>
+PCEXP_DEV void primitives_vjp(const S (&U)[D + 2], const S& ir, const S (&v)[D], const S& p, T gm, const S (&vb)[D],
+                              S pb, const S& Hb, S (&Ub)[D + 2]) {
+  constexpr int NV = D + 2;
+  const S Hi = Hb * ir;  // H = (E + p) / rho
+  pb = pb + Hi;
+  const S keb = (T(-0.5) * gm) * pb;
+  S irb = Hb * (U[NV - 1] + p);
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    const S w = vb[d] + keb * U[1 + d];
+    Ub[1 + d] = Ub[1 + d] + keb * v[d] + w * ir;
+    irb = irb + w * U[1 + d];
+  }
+  Ub[NV - 1] = Ub[NV - 1] + Hi + gm * pb;
+  Ub[0] = Ub[0] - ir * ir * irb;
+}
+
+// Lb, Rb += (dF~/dL)^T Fb, (dF~/dR)^T Fb for the Roe flux of roe_flux (same intermediates)
+template <int D, class S, class T>
+PCEXP_DEV void roe_flux_vjp(const S (&L)[D + 2], const S (&R)[D + 2], const T (&n)[D], T g, const T (&Fb)[D + 2],
+                            S (&Lb)[D + 2], S (&Rb)[D + 2], T vrn = T(0)) {
+  constexpr int NV = D + 2;
+  const T gm = g - T(1);
+  const S rL = L[0], irL = T(1) / rL, rR = R[0], irR = T(1) / rR;
+  S vL[D], vR[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    vL[d] = L[1 + d] * irL;
+    vR[d] = R[1 + d] * irR;
+  }
+  S keL = L[1] * vL[0], keR = R[1] * vR[0];
+#pragma unroll
+  for (int d = 1; d < D; ++d) {
+    keL = keL + L[1 + d] * vL[d];
+    keR = keR + R[1 + d] * vR[d];
+  }
+  const S pL = gm * (L[NV - 1] - T(0.5) * keL), pR = gm * (R[NV - 1] - T(0.5) * keR);
+  const S qL = dot_n<D>(vL, n), qR = dot_n<D>(vR, n);
+  const S hL = L[NV - 1] + pL, hR = R[NV - 1] + pR;
+  const S HL = hL * irL, HR = hR * irR;
+  const S sL = sqrt_s(rL), sR = sqrt_s(rR), is = T(1) / (sL + sR);
+  const S wL = sL * is, wR = sR * is, rh = sL * sR;
+  S vh[D], dv[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    vh[d] = wL * vL[d] + wR * vR[d];
+    dv[d] = vR[d] - vL[d];
+  }
+  const S Hh = wL * HL + wR * HR;
+  S q2 = vh[0] * vh[0], vdv = vh[0] * dv[0];
+#pragma unroll
+  for (int d = 1; d < D; ++d) {
+    q2 = q2 + vh[d] * vh[d];
+    vdv = vdv + vh[d] * dv[d];
+  }
+  const S cc = gm * (Hh - T(0.5) * q2), cs = sqrt_s(cc), i2c = T(0.5) / cc;
+  const S qh = dot_n<D>(vh, n), dq = dot_n<D>(dv, n), dp = pR - pL, dr = rR - rL;
+  const S qs = vrn != T(0) ? qh - vrn : qh;
+  const T s1 = sign_of(val(qs) - val(cs)), s2 = sign_of(val(qs)), s4 = sign_of(val(qs) + val(cs));
+  const S l1 = s1 * (qs - cs), l2 = s2 * qs, l4 = s4 * (qs + cs);
+  const S w = rh * cs * dq;
+  const S a1 = (dp - w) * i2c, a4 = (dp + w) * i2c, a2 = dr - T(2) * dp * i2c;
+  const S t1 = l1 * a1, t4 = l4 * a4, t2 = l2 * a2, ts = l2 * rh;
+  // F~ = (c - dd) / 2: the dissipation's adjoint is -Fb / 2
+  const T d0 = T(-0.5) * Fb[0], dE = T(-0.5) * Fb[NV - 1];
+  T dm[D], dmn = T(0);
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    dm[d] = T(-0.5) * Fb[1 + d];
+    dmn += dm[d] * n[d];
+  }
+  // dd_0 = t1 + t2 + t4, dd_m = (t1 + t2 + t4) vh + (t4 - t1) cs n + ts (dv - dq n),
+  // dd_E = (t1 + t4) Hh + (t4 - t1) cs qh + t2 q2 / 2 + ts (vdv - qh dq)
+  S dmvh = dm[0] * vh[0], dmdv = dm[0] * dv[0];
+#pragma unroll
+  for (int d = 1; d < D; ++d) {
+    dmvh = dmvh + dm[d] * vh[d];
+    dmdv = dmdv + dm[d] * dv[d];
+  }
+  const S mc = t4 - t1;
+  const S base = dmvh + d0, sb = base + dE * Hh, t2b = base + (T(0.5) * dE) * q2;
+  const S mcb = dE * qh + dmn, mb = mcb * cs;
+  const S tsb = dmdv - dmn * dq + dE * (vdv - qh * dq);
+  S csb = mcb * mc;
+  S qhb = dE * (mc * cs - ts * dq);
+  S dqb = -(ts * mcb);
+  S q2b = (T(0.5) * dE) * t2;
+  const S sum = t1 + t2 + t4;
+  S Hhb = dE * (t1 + t4);
+  const S t1b = sb - mb, t4b = sb + mb;
+  const S l1b = s1 * (t1b * a1), l4b = s4 * (t4b * a4), l2b = s2 * (t2b * a2 + tsb * rh);
+  qhb = qhb + l1b + l2b + l4b;
+  csb = csb - l1b + l4b;
+  const S a1b = t1b * l1, a4b = t4b * l4, a2b = t2b * l2;
+  S rhb = tsb * l2;
+  const S ab = a1b + a4b, wb = (a4b - a1b) * i2c;
+  const S dpb = (ab - T(2) * a2b) * i2c;
+  const S i2cb = (ab - T(2) * a2b) * dp + (a4b - a1b) * w;
+  const S wrc = wb * rh, wcd = wb * dq;
+  rhb = rhb + wcd * cs;
+  csb = csb + wcd * rh;
+  dqb = dqb + wrc * cs;
+  const S ccb = csb * cs * i2c - T(2) * (i2c * i2c) * i2cb;  // cs = sqrt(cc), i2c = 1 / (2 cc)
+  Hhb = Hhb + gm * ccb;
+  q2b = q2b - (T(0.5) * gm) * ccb;
+  // central part: c_0 = rL qL + rR qR, c_m = m qL + m' qR + (pL + pR) n, c_E = hL qL + hR qR
+  const T c0 = -d0, cE = -dE, cmn = -dmn;
+  S qLb = c0 * rL + cE * hL, qRb = c0 * rR + cE * hR;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    qLb = qLb - dm[d] * L[1 + d];
+    qRb = qRb - dm[d] * R[1 + d];
+  }
+  const S eL = cE * qL, eR = cE * qR;  // adjoint of h = E + p of each side
+  S vLb[D], vRb[D], wd = Hhb * (HL - HR);
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    const S vhb = dm[d] * sum + (dE * ts) * dv[d] + qhb * n[d] + T(2) * q2b * vh[d];
+    const S dvb = dm[d] * ts + (dE * ts) * vh[d] + dqb * n[d];
+    vLb[d] = wL * vhb - dvb + qLb * n[d];
+    vRb[d] = wR * vhb + dvb + qRb * n[d];
+    wd = wd - vhb * dv[d];
+    Lb[1 + d] = Lb[1 + d] - dm[d] * qL;
+    Rb[1 + d] = Rb[1 + d] - dm[d] * qR;
+  }
+  // wL = sL / (sL + sR), wR = 1 - wL; rh = sL sR; s = sqrt(r)
+  const S wi = wd * is;
+  const S sLb = wi * wR + rhb * sR, sRb = rhb * sL - wi * wL;
+  Lb[0] = Lb[0] + c0 * qL - a2b + T(0.5) * sLb / sL;
+  Rb[0] = Rb[0] + c0 * qR + a2b + T(0.5) * sRb / sR;
+  Lb[NV - 1] = Lb[NV - 1] + eL;
+  Rb[NV - 1] = Rb[NV - 1] + eR;
+  primitives_vjp<D, S, T>(L, irL, vL, pL, gm, vLb, eL - dpb + cmn, wL * Hhb, Lb);
+  primitives_vjp<D, S, T>(R, irR, vR, pR, gm, vRb, eR + dpb + cmn, wR * Hhb, Rb);
+  if (vrn != T(0)) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      Lb[v] = Lb[v] - (T(0.5) * vrn) * Fb[v];
+      Rb[v] = Rb[v] - (T(0.5) * vrn) * Fb[v];
+    }
+  }
+}
+
+// Ub += (dG/dU)^T Gb for ghost_slip_wall (linear in U)
+template <int D, class S, class T>
+PCEXP_DEV void ghost_slip_wall_vjp(const T (&n)[D], const S (&Gb)[D + 2], S (&Ub)[D + 2], T vrn = T(0)) {
+  constexpr int NV = D + 2;
+  S a = Gb[1] * n[0];
+#pragma unroll
+  for (int d = 1; d < D; ++d) a = a + Gb[1 + d] * n[d];
+  S b = T(2) * a;
+  Ub[0] = Ub[0] + Gb[0];
+  if (vrn != T(0)) {
+    b = b + (T(2) * vrn) * Gb[NV - 1];
+    Ub[0] = Ub[0] + vrn * b;
+  }
+#pragma unroll
+  for (int d = 0; d < D; ++d) Ub[1 + d] = Ub[1 + d] + Gb[1 + d] - b * n[d];
+  Ub[NV - 1] = Ub[NV - 1] + Gb[NV - 1];
+}
+
+// Ub += (dG/dU)^T Gb and vib += (dG/dv_inf)^T Gb for ghost_farfield (same intermediates)
+template <int D, class S, class T>
+PCEXP_DEV void ghost_farfield_vjp(const S (&U)[D + 2], const T (&n)[D], const Free<T>& fs, const S (&Gb)[D + 2],
+                                  S (&Ub)[D + 2], S (&vib)[D]) {
+  constexpr int NV = D + 2;
+  const T g = fs.gamma, gm = g - T(1);
+  const S ir = T(1) / U[0];
+  S vel[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) vel[d] = U[1 + d] * ir;
+  S ke = U[1] * vel[0];
+#pragma unroll
+  for (int d = 1; d < D; ++d) ke = ke + U[1 + d] * vel[d];
+  const S p = gm * (U[NV - 1] - T(0.5) * ke);
+  const S c = sqrt_s(g * p * ir);
+  const S qn = dot_n<D>(vel, n);
+  const T cinf = sqrt_s(g * fs.p / fs.rho);
+  T qinf = fs.vel[0] * n[0];
+#pragma unroll
+  for (int d = 1; d < D; ++d) qinf += fs.vel[d] * n[d];
+  const T mn = val(qn) / val(c);
+  const bool in_p = mn > T(-1), in_m = !(mn < T(1));  // invariants taken from the interior
+  const S rp = select_s(in_p, qn + T(2) * c / gm, Lift<S, T>::of(qinf + T(2) * cinf / gm));
+  const S rm = select_s(!in_m, Lift<S, T>::of(qinf - T(2) * cinf / gm), qn - T(2) * c / gm);
+  const S qb = T(0.5) * (rp + rm);
+  const S cb = T(0.25) * gm * (rp - rm);
+  const bool out = val(qb) >= T(0);
+  const S s_in = p / pow_s(U[0], g);
+  const T s_inf = fs.p / pow_s(fs.rho, g);
+  const S sb = select_s(out, s_in, Lift<S, T>::of(s_inf));
+  const S rb = pow_s(cb * cb / (g * sb), T(1) / gm);
+  S vb[D], kb = Lift<S, T>::of(T(0)), rbb = Gb[0], qbb = Lift<S, T>::of(T(0)), vbb[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    const S vt = select_s(out, vel[d] - qn * n[d], Lift<S, T>::of(fs.vel[d] - qinf * n[d]));
+    vb[d] = vt + qb * n[d];
+    kb = kb + vb[d] * vb[d];
+    rbb = rbb + Gb[1 + d] * vb[d];
+  }
+  rbb = rbb + T(0.5) * Gb[NV - 1] * kb;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    vbb[d] = rb * (Gb[1 + d] + Gb[NV - 1] * vb[d]);
+    qbb = qbb + vbb[d] * n[d];
+  }
+  const S pbb = Gb[NV - 1] / gm;  // G_E = p_b / gm + rho_b |v_b|^2 / 2, p_b = rho_b c_b^2 / g
+  rbb = rbb + pbb * cb * cb / g;
+  S cbb = T(2) / g * pbb * rb * cb;
+  const S lr = rbb * rb / gm;  // rho_b = (c_b^2 / (g s_b))^(1 / gm)
+  cbb = cbb + T(2) * lr / cb;
+  S qnb = Lift<S, T>::of(T(0)), qib = qnb, cib = qnb, pb = qnb;
+  const S rpb = T(0.5) * qbb + (T(0.25) * gm) * cbb, rmb = T(0.5) * qbb - (T(0.25) * gm) * cbb;
+  if (in_p) {
+    qnb = qnb + rpb;
+    cib = cib + rpb;
+  } else {
+    qib = qib + rpb;
+  }
+  if (in_m) {
+    qnb = qnb + rmb;
+    cib = cib - rmb;
+  } else {
+    qib = qib + rmb;
+  }
+  if (out) {
+    qnb = qnb - qbb;
+    pb = pb - lr / p;         // s_in = p rho^-g
+    Ub[0] = Ub[0] + g * lr * ir;
+  } else {
+    qib = qib - qbb;
+  }
+  const S ch = (T(1) / gm) * cib * c;  // (2 / gm) cib * dc, dc = c / 2 (dp / p - drho / rho)
+  pb = pb + ch / p;
+  Ub[0] = Ub[0] - ch * ir;
+  const S keb = (T(-0.5) * gm) * pb;
+  S irb = Lift<S, T>::of(T(0));
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    S w = keb * U[1 + d] + qnb * n[d];
+    if (out) w = w + vbb[d];
+    else vib[d] = vib[d] + vbb[d];
+    vib[d] = vib[d] + qib * n[d];
+    Ub[1 + d] = Ub[1 + d] + keb * vel[d] + w * ir;
+    irb = irb + w * U[1 + d];
+  }
+  Ub[NV - 1] = Ub[NV - 1] + gm * pb;
+  Ub[0] = Ub[0] - ir * ir * irb;
 }
 
 }  // namespace pcexp
