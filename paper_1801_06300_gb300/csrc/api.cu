@@ -418,13 +418,12 @@ template <class T> LinData<T> lindata(pcexp_ctx* c) {
 // Linearise the operator at u for the J v products that follow.  FP64 contexts build the
 // face and volume point Jacobians once; FP32-mixed contexts build the face blocks only and
 // recompute the volume flux tangents at u in every J v (reading u and dv instead of
-// D nv^2 values per volume point).  blocks = true builds both (the transpose needs them).
+// D nv^2 values per volume point).
 template <class T>
-int linearize(pcexp_ctx* c, const DGData<T>& d, const T* u, bool blocks = false) {
+int linearize(pcexp_ctx* c, const DGData<T>& d, const T* u) {
   c->lin_state = u;
-  if (c->face_tangent && !blocks) return PCEXP_OK;  // every J v recomputes its tangents at u
-  const bool faces_only = c->jv_tangent && !blocks;
-  PCEXP_LAUNCH(c, PCEXP_KC_LINEARIZE, launch_linearize<T>(d, u, lindata<T>(c), c->st, faces_only));
+  if (c->face_tangent) return PCEXP_OK;  // every J v recomputes its tangents at u
+  PCEXP_LAUNCH(c, PCEXP_KC_LINEARIZE, launch_linearize<T>(d, u, lindata<T>(c), c->st, c->jv_tangent));
   return PCEXP_OK;
 }
 
@@ -1210,7 +1209,7 @@ int create_impl(pcexp_ctx* c, const pcexp_mesh* mesh, int p, const pcexp_physics
   const size_t nfp = (size_t)(c->F > 0 ? c->F : 1) * c->nfq, nv = (size_t)c->nv;
   PCEXP_TRY(valloc(&c->G, nfp * nv));
   PCEXP_TRY(valloc(&c->dte, c->E));
-  PCEXP_TRY(valloc(&c->Avol, (size_t)c->dim * nv * nv * c->E * c->nq));
+  if (!c->jv_tangent) PCEXP_TRY(valloc(&c->Avol, (size_t)c->dim * nv * nv * c->E * c->nq));
   PCEXP_TRY(valloc(&c->GT, 2 * nv * nfp));
   PCEXP_TRY(valloc(&c->Bface, 2 * nv * nv * nfp));
   PCEXP_TRY(dalloc(c, &c->io64a, Kp));
@@ -1239,8 +1238,7 @@ int vjp_impl(pcexp_ctx* c, const double* U, const double* w, double* JTw, int on
   const DGData<T> d = dgdata<T>(c);
   PCEXP_TRY(import_vec<T>(c, U, on_device, a));
   PCEXP_TRY(import_vec<T>(c, w, on_device, b));
-  PCEXP_TRY(linearize<T>(c, d, a, true));
-  PCEXP_CK(launch_jac_adjoint<T>(d, lindata<T>(c), b, o, reinterpret_cast<T*>(c->GT), nullptr, T(1), c->st));
+  PCEXP_CK(launch_vjp<T>(d, a, b, o, reinterpret_cast<T*>(c->GT), c->st));
   PCEXP_TRY(export_vec<T>(c, o, JTw, on_device));
   if (on_device) PCEXP_CK(cudaStreamSynchronize(c->st));
   return PCEXP_OK;
@@ -1436,10 +1434,11 @@ int step_backward_impl(pcexp_ctx* c, const double* U, double dt, int m, const do
     PCEXP_CK(launch_axpy(c->b_rb, c->b_bb, nullptr, -1.0, Kp, c->st));
     // theta_bar += (dR(u_*; theta)/dtheta)^T bbar_2
     PCEXP_TRY(param_adjoint(c, d, c->b_us, c->b_bb, 1.0));
-    PCEXP_TRY(linearize<double>(c, d, c->b_us));
-    PCEXP_TRY(adj_jt(c, d, c->b_bb, c->b_t1));
+    // one product at u_*: without point Jacobians, so those at u_n stay
+    PCEXP_TRY(group_exchange<double>(c, c->b_bb));
+    PCEXP_CK(launch_vjp<double>(d, c->b_us, c->b_bb, c->b_t1, reinterpret_cast<double*>(c->GT), c->st));
+    PCEXP_TRY(group_zero_halo<double>(c, c->b_t1));
     PCEXP_CK(launch_axpy(c->b_ubs, c->b_t1, nullptr, 1.0, Kp, c->st));
-    PCEXP_TRY(linearize<double>(c, d, c->b_un));
   }
   // u_* = u_n + delta
   PCEXP_CK(launch_axpy(c->b_ubn, c->b_ubs, nullptr, 1.0, Kp, c->st));
@@ -2105,8 +2104,7 @@ int group_adjoint_part(pcexp_ctx* c, int adj, const std::vector<double>& u, cons
   PCEXP_TRY(group_exchange<T>(c, a));
   PCEXP_TRY(group_exchange<T>(c, ww));
   if (adj == 1) {
-    PCEXP_TRY(linearize<T>(c, d, a, true));
-    PCEXP_CK(launch_jac_adjoint<T>(d, lindata<T>(c), ww, o, reinterpret_cast<T*>(c->GT), nullptr, T(1), c->st));
+    PCEXP_CK(launch_vjp<T>(d, a, ww, o, reinterpret_cast<T*>(c->GT), c->st));
   } else {
     if constexpr (std::is_same<T, double>::value) {
       PCEXP_TRY(import_vec<T>(c, v->data(), 0, b));

@@ -678,11 +678,42 @@ cudaError_t tan_tables_p(const DGData<float>& d, cudaStream_t st) {
                                  cudaMemcpyDeviceToDevice, st);
 }
 
+// U[v] = isd sum_j b[j] ue[v][j]: the trace of an element's coefficients at a point, table row b
+// in global memory
+template <class T, int D, int P>
+PCEXP_DEV void point_trace(const T* b, const T* __restrict__ ue, T isd, T (&U)[D + 2]) {
+  constexpr int NB = Ord<D, P>::NB, NV = D + 2;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    T a = 0;
+#pragma unroll
+    for (int j = 0; j < NB; ++j) a += __ldg(b + j) * ue[v * NB + j];
+    U[v] = a * isd;
+  }
+}
+
+// Reverse sweep of a face's Riemann flux: Lb, Rb += its adjoints; on boundary faces (eR < 0, R the
+// ghost state of L) the ghost's adjoint is folded into Lb.
+template <class T, int D>
+PCEXP_DEV void face_flux_vjp(const DGData<T>& d, int eR, const T (&L)[D + 2], const T (&R)[D + 2], const T (&n)[D],
+                             T vrn, const T (&gb)[D + 2], T (&Lb)[D + 2], T (&Rb)[D + 2]) {
+  roe_flux_vjp<D, T, T>(L, R, n, d.fs.gamma, gb, Lb, Rb, vrn);
+  if (eR >= 0) return;
+  if (mirror_bc(eR)) {
+    ghost_slip_wall_vjp<D, T, T>(n, Rb, Lb, vrn);
+  } else {
+    T vib[D];
+#pragma unroll
+    for (int k = 0; k < D; ++k) vib[k] = T(0);
+    ghost_farfield_vjp<D, T, T>(L, n, d.fs, Rb, Lb, vib);
+  }
+}
+
 // ------------------------------------------------------- point Jacobians (linearisation)
 // The exact Jacobian of the scheme (Eq. jac1, jac2) is assembled point by point: the
 // volume flux Jacobians dF_d/dU and the Riemann-flux Jacobians dF~/dU_L, dF~/dU_R are
-// evaluated exactly by running the flux code on Jet<T, D+2> numbers seeded with unit
-// directions (the paper obtains the Riemann-flux Jacobians by AD as well).  Every J v
+// evaluated exactly, the former on Jet<T, D+2> numbers seeded with unit directions, the latter
+// by reverse sweeps (the paper obtains the Riemann-flux Jacobians by AD as well).  Every J v
 // of a PCEXP step is taken at u_n, so the Jacobians are built once per step and each
 // of the 2m+1 products reduces to traces, small mat-vecs and the test/lift contractions.
 template <class T, int D, int P>
@@ -730,12 +761,15 @@ __global__ void __launch_bounds__(256) linearize_vol_kernel(DGData<T> d, const T
       }
 }
 
+// The face blocks come row by row from reverse sweeps of the Roe flux: with the adjoint e_v one
+// sweep gives row v of both dF~/dU_L and dF~/dU_R (the flux's own intermediates are hoisted out of
+// the loop), where a forward sweep per side carries D + 2 directions through every operation.
+// FP64 at p = 2, 20^3 Kuhn cubes (96,000 faces): 3.5 -> 1.6 ms; bound by the FP64 pipe.
 template <class T, int D, int P>
 __global__ void __launch_bounds__(128) linearize_face_kernel(DGData<T> d, const T* __restrict__ u,
                                                              T* __restrict__ Bface) {
   using O = Ord<D, P>;
   constexpr int NB = O::NB, NFQ = O::NFQ, NV = O::NV, NPERM = O::NPERM, GEO = O::GEO, NN = NV * NV;
-  using J = Jet<T, NV>;
   const int64_t n = d.F * NFQ;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n) return;
@@ -748,62 +782,33 @@ __global__ void __launch_bounds__(128) linearize_face_kernel(DGData<T> d, const 
 #pragma unroll
   for (int k = 0; k < D; ++k) nr[k] = d.fgeo[4 * f + k];
   const T wq = d.fgeo[4 * f + D] * d.Wf[q];
-  T uL[NV], uR[NV];
+  const T vrn = d.rot ? d.vrn[idx] : T(0);
+  T L[NV], R[NV];
   const T isdL = d.geo[GEO * (int64_t)eL + O::ISD];
   T isdR = T(0);
-  {
-    const T* be = d.Bf + ((fL * NPERM) * NFQ + q) * NB;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      T a = 0;
-#pragma unroll
-      for (int j = 0; j < NB; ++j) a += __ldg(be + j) * u[(int64_t)eL * NV * NB + v * NB + j];
-      uL[v] = a * isdL;
-    }
-  }
+  point_trace<T, D, P>(d.Bf + ((fL * NPERM) * NFQ + q) * NB, u + (int64_t)eL * NV * NB, isdL, L);
   if (eR >= 0) {
     isdR = d.geo[GEO * (int64_t)eR + O::ISD];
-    const T* be = d.Bf + ((fR * NPERM + pR) * NFQ + q) * NB;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      T a = 0;
-#pragma unroll
-      for (int j = 0; j < NB; ++j) a += __ldg(be + j) * u[(int64_t)eR * NV * NB + v * NB + j];
-      uR[v] = a * isdR;
-    }
+    point_trace<T, D, P>(d.Bf + ((fR * NPERM + pR) * NFQ + q) * NB, u + (int64_t)eR * NV * NB, isdR, R);
+  } else if (mirror_bc(eR)) {
+    ghost_slip_wall<D, T, T>(L, nr, R, vrn);
+  } else {
+    ghost_farfield<D, T, T>(L, nr, d.fs, R);
   }
 #pragma unroll 1
-  for (int side = 0; side < 2; ++side) {
-    J L[NV], R[NV], F[NV];
-    if (side == 1 && eR < 0) {
+  for (int v = 0; v < NV; ++v) {
+    T gb[NV], Lb[NV], Rb[NV];
 #pragma unroll
-      for (int k = 0; k < NN; ++k) Bface[bface_at<T, 2 * NN>(NN + k, idx, n)] = T(0);
-      break;
+    for (int c = 0; c < NV; ++c) {
+      gb[c] = c == v ? T(1) : T(0);
+      Lb[c] = Rb[c] = T(0);
     }
+    face_flux_vjp<T, D>(d, eR, L, R, nr, vrn, gb, Lb, Rb);
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      L[v].v = uL[v];
-#pragma unroll
-      for (int c = 0; c < NV; ++c) L[v].d[c] = (side == 0 && v == c) ? T(1) : T(0);
+    for (int c = 0; c < NV; ++c) {
+      Bface[bface_at<T, 2 * NN>(v * NV + c, idx, n)] = wq * isdL * Lb[c];
+      Bface[bface_at<T, 2 * NN>(NN + v * NV + c, idx, n)] = eR >= 0 ? wq * isdR * Rb[c] : T(0);
     }
-    if (eR >= 0) {
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        R[v].v = uR[v];
-#pragma unroll
-        for (int c = 0; c < NV; ++c) R[v].d[c] = (side == 1 && v == c) ? T(1) : T(0);
-      }
-    } else if (mirror_bc(eR)) {
-      ghost_slip_wall<D, J, T>(L, nr, R, d.rot ? d.vrn[idx] : T(0));
-    } else {
-      ghost_farfield<D, J, T>(L, nr, d.fs, R);
-    }
-    roe_flux<D, J, T>(L, R, nr, d.fs.gamma, F, d.rot ? d.vrn[idx] : T(0));
-    const T sc = wq * (side == 0 ? isdL : isdR);
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int c = 0; c < NV; ++c) Bface[bface_at<T, 2 * NN>(side * NN + v * NV + c, idx, n)] = sc * F[v].d[c];
   }
 }
 
@@ -1311,19 +1316,20 @@ __global__ void __launch_bounds__(128) face_hess_kernel(DGData<T> d, const T* __
   }
 }
 
-template <class T, int D, int P>
+// Element part of the second-order adjoint (HESS) or of J(u)^T w without stored Jacobians.
+template <class T, int D, int P, bool HESS>
 __global__ void __launch_bounds__(256) elem_hess_kernel(DGData<T> d, const T* __restrict__ u, const T* __restrict__ v,
                                                         const T* __restrict__ w, const T* __restrict__ GT,
                                                         T* __restrict__ out, const T* __restrict__ escale, T osc) {
   using O = Ord<D, P>;
   constexpr int NB = O::NB, NQ = O::NQ, ET = O::ET, NVB = O::NVB, NV = O::NV, GEO = O::GEO;
   constexpr bool SM = O::SMEM_BF;
-  using S = Tangent<T>;
+  using S = typename std::conditional<HESS, Tangent<T>, T>::type;
   __shared__ T sBv[NQ * NB];
   __shared__ T sDv[D * NQ * NB];
   __shared__ T sBf[SM ? O::NBF : 1];
   __shared__ T su[ET * NVB];
-  __shared__ T sv[ET * NVB];
+  __shared__ T sv[HESS ? ET * NVB : 1];
   __shared__ T sw[ET * NVB];
   __shared__ T sU[ET * NQ * NV];
   __shared__ T sgeo[ET * GEO];
@@ -1336,7 +1342,7 @@ __global__ void __launch_bounds__(256) elem_hess_kernel(DGData<T> d, const T* __
     for (int i = threadIdx.x; i < O::NBF; i += blockDim.x) sBf[i] = d.Bf[i];
   for (int i = threadIdx.x; i < ne * NVB; i += blockDim.x) {
     su[i] = u[e0 * NVB + i];
-    sv[i] = v[e0 * NVB + i];
+    if constexpr (HESS) sv[i] = v[e0 * NVB + i];
     sw[i] = w[e0 * NVB + i] * osc * (escale ? escale[e0 + i / NVB] : T(1));
   }
   for (int i = threadIdx.x; i < ne * GEO; i += blockDim.x) sgeo[i] = d.geo[e0 * GEO + i];
@@ -1353,10 +1359,11 @@ __global__ void __launch_bounds__(256) elem_hess_kernel(DGData<T> d, const T* __
 #pragma unroll
       for (int j = 0; j < NB; ++j) {
         a += sBv[q1 * NB + j] * su[el1 * NVB + c * NB + j];
-        b += sBv[q1 * NB + j] * sv[el1 * NVB + c * NB + j];
+        if constexpr (HESS) b += sBv[q1 * NB + j] * sv[el1 * NVB + c * NB + j];
       }
-      U[c] = S{a * isd, b};  // the sqrt(det) factors of trace and test cancel
-      Ub[c] = S{T(0), T(0)};
+      if constexpr (HESS) U[c] = S{a * isd, b};  // the sqrt(det) factors of trace and test cancel
+      else U[c] = a * isd;
+      Ub[c] = Lift<S, T>::of(T(0));
       // adjoint of the flux along the Cartesian axes: the transposed test, mapped by A^-1
       T t[D];
 #pragma unroll
@@ -1376,7 +1383,20 @@ __global__ void __launch_bounds__(256) elem_hess_kernel(DGData<T> d, const T* __
     }
     euler_flux_vjp<D, S, T>(U, d.fs.gamma, fb, Ub);
 #pragma unroll
-    for (int c = 0; c < NV; ++c) sU[(el1 * NQ + q1) * NV + c] = Ub[c].d * isd;
+    for (int c = 0; c < NV; ++c) {
+      T o;
+      if constexpr (HESS) {
+        o = Ub[c].d * isd;
+      } else {
+        o = Ub[c];
+        if (d.rot) {  // rotating frame: the flux is F - U v_r^T
+          const T* vr = d.vrq + ((e0 + el1) * NQ + q1) * D;
+#pragma unroll
+          for (int k = 0; k < D; ++k) o -= fb[k][c] * vr[k];
+        }
+      }
+      sU[(el1 * NQ + q1) * NV + c] = o;
+    }
   }
   __syncthreads();
   const T* Bf = SM ? sBf : d.Bf;
@@ -1387,6 +1407,14 @@ __global__ void __launch_bounds__(256) elem_hess_kernel(DGData<T> d, const T* __
 #pragma unroll
     for (int q = 0; q < NQ; ++q) acc += sBv[q * NB + j] * sU[(el * NQ + q) * NV + c];
     acc += gather_faces_T<T, D, P, SM>(d, Bf, GT, e0 + el, c, j);
+    if constexpr (!HESS) {
+      if (d.rot && c >= 1 && c <= D) {  // transpose of the source -omega x: +omega x w~ (antisymmetric)
+        T m[D];
+#pragma unroll
+        for (int k = 0; k < D; ++k) m[k] = sw[el * NVB + (1 + k) * NB + j];
+        acc -= rot_source<T, D>(d.om, m, c - 1);
+      }
+    }
     out[e0 * NVB + it] = acc;
   }
 }
@@ -1398,7 +1426,70 @@ cudaError_t jvp_state_adjoint_p(const DGData<T>& d, const T* u, const T* v, cons
   const int64_t nf = d.F * O::NFQ;
   if (nf > 0) face_hess_kernel<T, D, P><<<(unsigned)((nf + 127) / 128), 128, 0, st>>>(d, u, v, w, GT, escale, osc, th);
   const int64_t eb = (d.E + O::ET - 1) / O::ET;
-  elem_hess_kernel<T, D, P><<<(unsigned)eb, 256, 0, st>>>(d, u, v, w, GT, out, escale, osc);
+  elem_hess_kernel<T, D, P, true><<<(unsigned)eb, 256, 0, st>>>(d, u, v, w, GT, out, escale, osc);
+  return cudaGetLastError();
+}
+
+// ------------------------------------------- J(u)^T w for a single product
+// Reverse sweeps of the fluxes at u with the transposed lift and test of w as adjoints: no point
+// Jacobians are formed (building them for one product took 72% of pcexp_vjp).  Scratch layout of
+// the adjoint kernels.  Vortex, 20,402 triangles at p = 3, FP64: a call takes 334 us against 842
+// with the Jacobians (503 + 117 us of building them).
+template <class T, int D, int P>
+__global__ void __launch_bounds__(128) face_vjp_kernel(DGData<T> d, const T* __restrict__ u, const T* __restrict__ w,
+                                                       T* __restrict__ GT) {
+  using O = Ord<D, P>;
+  constexpr int NB = O::NB, NFQ = O::NFQ, NV = O::NV, NPERM = O::NPERM, GEO = O::GEO;
+  const int64_t n = d.F * NFQ;
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= n) return;
+  const int64_t f = idx / NFQ;
+  const int q = (int)(idx - f * NFQ);
+  const int eL = d.fel[2 * f], eR = d.fel[2 * f + 1];
+  const int loc = d.floc[f];
+  const int fL = loc & 0xff, fR = (loc >> 8) & 0xff, pR = loc >> 16;
+  T nr[D];
+#pragma unroll
+  for (int k = 0; k < D; ++k) nr[k] = d.fgeo[4 * f + k];
+  const T wq = d.fgeo[4 * f + D] * d.Wf[q];
+  const T vrn = d.rot ? d.vrn[idx] : T(0);
+  const T isdL = d.geo[GEO * (int64_t)eL + O::ISD];
+  T isdR = T(0), L[NV], R[NV], gb[NV];
+  const T* bL = d.Bf + ((fL * NPERM) * NFQ + q) * NB;
+  point_trace<T, D, P>(bL, u + (int64_t)eL * NV * NB, isdL, L);
+  point_trace<T, D, P>(bL, w + (int64_t)eL * NV * NB, -isdL, gb);
+  if (eR >= 0) {
+    isdR = d.geo[GEO * (int64_t)eR + O::ISD];
+    const T* bR = d.Bf + ((fR * NPERM + pR) * NFQ + q) * NB;
+    T g[NV];
+    point_trace<T, D, P>(bR, u + (int64_t)eR * NV * NB, isdR, R);
+    point_trace<T, D, P>(bR, w + (int64_t)eR * NV * NB, isdR, g);
+#pragma unroll
+    for (int c = 0; c < NV; ++c) gb[c] += g[c];
+  } else if (mirror_bc(eR)) {
+    ghost_slip_wall<D, T, T>(L, nr, R, vrn);
+  } else {
+    ghost_farfield<D, T, T>(L, nr, d.fs, R);
+  }
+  T Lb[NV], Rb[NV];
+#pragma unroll
+  for (int c = 0; c < NV; ++c) Lb[c] = Rb[c] = T(0);
+  face_flux_vjp<T, D>(d, eR, L, R, nr, vrn, gb, Lb, Rb);
+  T* o = GT + idx * 2 * NV;
+#pragma unroll
+  for (int c = 0; c < NV; ++c) {
+    o[c] = wq * isdL * Lb[c];
+    o[NV + c] = eR >= 0 ? wq * isdR * Rb[c] : T(0);
+  }
+}
+
+template <class T, int D, int P>
+cudaError_t vjp_p(const DGData<T>& d, const T* u, const T* w, T* out, T* GT, cudaStream_t st) {
+  using O = Ord<D, P>;
+  const int64_t nf = d.F * O::NFQ;
+  if (nf > 0) face_vjp_kernel<T, D, P><<<(unsigned)((nf + 127) / 128), 128, 0, st>>>(d, u, w, GT);
+  const int64_t eb = (d.E + O::ET - 1) / O::ET;
+  elem_hess_kernel<T, D, P, false><<<(unsigned)eb, 256, 0, st>>>(d, u, nullptr, w, GT, out, nullptr, T(1));
   return cudaGetLastError();
 }
 
@@ -1851,6 +1942,11 @@ cudaError_t launch_jvp_state_adjoint_d(const DGData<T>& d, const T* u, const T* 
 }
 
 template <class T, int D>
+cudaError_t launch_vjp_d(const DGData<T>& d, const T* u, const T* w, T* out, T* GT, cudaStream_t st) {
+  PCEXP_PSWITCH(D, (vjp_p<T, D, P_>(d, u, w, out, GT, st)))
+}
+
+template <class T, int D>
 cudaError_t launch_param_adjoint_d(const DGData<T>& d, int64_t f0, const T* u, const T* w, double osc,
                                    const double* dvel, double* acc, double* partials, unsigned* counter,
                                    cudaStream_t st) {
@@ -1922,6 +2018,7 @@ cudaError_t launch_local_dt_d(const DGData<T>& d, const T* u, const double* cfl_
                                                   cudaStream_t);                                                   \
   template cudaError_t launch_jvp_state_adjoint_d<T, D>(const DGData<T>&, const T*, const T*, const T*, T*, T*,    \
                                                         const T*, T, cudaStream_t, const ThetaSums<T>&);           \
+  template cudaError_t launch_vjp_d<T, D>(const DGData<T>&, const T*, const T*, T*, T*, cudaStream_t);             \
   template cudaError_t launch_wall_force_d<T, D>(const DGData<T>&, int64_t, const T*, double, double, double,      \
                                                  double*, double*, double*, unsigned*, cudaStream_t);              \
   template cudaError_t launch_vortex_error_d<T, D>(const DGData<T>&, const T*, const double*, const double*,       \

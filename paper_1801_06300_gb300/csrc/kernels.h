@@ -148,6 +148,8 @@ template <class T, int D>
 cudaError_t launch_jvp_state_adjoint_d(const DGData<T>& d, const T* u, const T* v, const T* w, T* out, T* GT,
                                        const T* escale, T osc, cudaStream_t st, const ThetaSums<T>& th);
 template <class T, int D>
+cudaError_t launch_vjp_d(const DGData<T>& d, const T* u, const T* w, T* out, T* GT, cudaStream_t st);
+template <class T, int D>
 cudaError_t launch_wall_force_d(const DGData<T>& d, int64_t f0, const T* u, double ax, double ay, double az,
                                 double* grad, double* value, double* partials, unsigned* counter, cudaStream_t st);
 template <class T, int D>
@@ -209,6 +211,11 @@ cudaError_t launch_jac_adjoint(const DGData<T>& d, LinData<T> lin, const T* w, T
                                cudaStream_t st) {
   return d.dim == 3 ? launch_jac_adjoint_d<T, 3>(d, lin, w, out, GT, escale, osc, st)
                     : launch_jac_adjoint_d<T, 2>(d, lin, w, out, GT, escale, osc, st);
+}
+// out = J(u)^T w without point Jacobians (a single product at u); GT is scratch [F][nfq][2 NV].
+template <class T>
+cudaError_t launch_vjp(const DGData<T>& d, const T* u, const T* w, T* out, T* GT, cudaStream_t st) {
+  return d.dim == 3 ? launch_vjp_d<T, 3>(d, u, w, out, GT, st) : launch_vjp_d<T, 2>(d, u, w, out, GT, st);
 }
 // out = (d/du [ (osc diag(escale) J(u) v)^T w ])^T, the second-order adjoint; GT scratch [F][nfq][2 NV].
 template <class T>
