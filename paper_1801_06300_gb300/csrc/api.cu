@@ -48,10 +48,7 @@ struct pcexp_ctx {
   void* S32[2] = {nullptr, nullptr};  // FP32 shadows (mixed form only)
   void *V = nullptr, *w = nullptr, *tmp = nullptr, *delta = nullptr, *G = nullptr, *dte = nullptr;
   double *io64a = nullptr, *io64b = nullptr;
-  void *Avol = nullptr, *Bface = nullptr;  // point Jacobians at the linearisation state
-  const void* lin_state = nullptr;         // state the last linearize() recorded
-  bool jv_tangent = false;                 // volume part of J v by flux tangents (FP32-mixed)
-  bool face_tangent = false;               // face part of J v by Riemann-flux tangents (no face blocks)
+  void *pts = nullptr, *Bface = nullptr;  // linearisation: volume points, face blocks (LinData)
   void* GT = nullptr;                      // adjoint face scratch [F][nfq][2 nv]
   double* xq = nullptr;                    // physical volume points [E][nq][dim] (first vortex functional)
   double* diag = nullptr;                  // FP64 [Bv (nq nb) | Wv (nq) | sqrt|det A| (E)] (first entropy output)
@@ -412,18 +409,13 @@ int dg_apply(pcexp_ctx* c, const DGData<T>& d, const T* u, const T* du, T* out, 
 }
 
 template <class T> LinData<T> lindata(pcexp_ctx* c) {
-  return LinData<T>{reinterpret_cast<T*>(c->Avol), reinterpret_cast<T*>(c->Bface)};
+  return LinData<T>{reinterpret_cast<T*>(c->pts), reinterpret_cast<T*>(c->Bface)};
 }
 
-// Linearise the operator at u for the J v products that follow.  FP64 contexts build the
-// face and volume point Jacobians once; FP32-mixed contexts build the face blocks only and
-// recompute the volume flux tangents at u in every J v (reading u and dv instead of
-// D nv^2 values per volume point).
+// Linearise the operator at u for the J v products that follow.
 template <class T>
 int linearize(pcexp_ctx* c, const DGData<T>& d, const T* u) {
-  c->lin_state = u;
-  if (c->face_tangent) return PCEXP_OK;  // every J v recomputes its tangents at u
-  PCEXP_LAUNCH(c, PCEXP_KC_LINEARIZE, launch_linearize<T>(d, u, lindata<T>(c), c->st, c->jv_tangent));
+  PCEXP_LAUNCH(c, PCEXP_KC_LINEARIZE, launch_linearize<T>(d, u, lindata<T>(c), c->st));
   return PCEXP_OK;
 }
 
@@ -433,9 +425,8 @@ int jac_apply(pcexp_ctx* c, const DGData<T>& d, const T* dv, T* out, const T* es
               const double* oscale) {
   PCEXP_TRY(group_exchange<T>(c, dv));
   cudaEvent_t* ev = prof_events(c, 3);
-  const T* u_elem = c->jv_tangent ? reinterpret_cast<const T*>(c->lin_state) : nullptr;
   cudaError_t e = launch_jac_apply<T>(d, lindata<T>(c), dv, out, reinterpret_cast<T*>(c->G), escale, skip, oscale,
-                                      c->st, ev, u_elem, c->face_tangent);
+                                      c->st, ev);
   if (ev) {
     prof_note(c, PCEXP_KC_JVP_FACE, ev, 0);
     prof_note(c, PCEXP_KC_JVP_ELEM, ev, 1);
@@ -1136,11 +1127,6 @@ int create_impl(pcexp_ctx* c, const pcexp_mesh* mesh, int p, const pcexp_physics
   c->volume = s.volume;
   c->phys = *phys;
   c->fp32 = opt->precision == PCEXP_FP32_MIXED;
-  c->jv_tangent = c->fp32;
-  // the face part of J v applies the stored face point Jacobians: recomputing the Roe-flux
-  // tangents per face point in every J v measured slower on GB300 (48^3 tetrahedra, P2:
-  // 37.6 against 33.9 + 2.0 ms per step with the blocks and their linearisation)
-  c->face_tangent = false;
   c->m_max = opt->m_max;
   c->eta = opt->breakdown_eta > 0 ? opt->breakdown_eta : (c->fp32 ? 1e-6 : 1e-12);
   c->ktol = opt->krylov_tol > 0 ? opt->krylov_tol : 0.0;
@@ -1168,11 +1154,12 @@ int create_impl(pcexp_ctx* c, const pcexp_mesh* mesh, int p, const pcexp_physics
     PCEXP_TRY(upload<float>(c, &c->tabs, tabs));
     PCEXP_TRY(upload<float>(c, &c->geo, s.geo));
     PCEXP_TRY(upload<float>(c, &c->fgeo, s.fgeo));
-    if (c->jv_tangent) PCEXP_CK(launch_tan_tables(dgdata<float>(c), c->st));
+    PCEXP_CK(upload_tables<float>(dgdata<float>(c), s.Bv.data(), s.Dv.data(), s.Wv.data(), s.Bf.data(), c->st));
   } else {
     PCEXP_TRY(upload<double>(c, &c->tabs, tabs));
     PCEXP_TRY(upload<double>(c, &c->geo, s.geo));
     PCEXP_TRY(upload<double>(c, &c->fgeo, s.fgeo));
+    PCEXP_CK(upload_tables<double>(dgdata<double>(c), s.Bv.data(), s.Dv.data(), s.Wv.data(), s.Bf.data(), c->st));
   }
   void* q = nullptr;
   PCEXP_TRY(upload<double>(c, &q, pack_basis_change(s.Q, s.E, s.nb, s.dim)));
@@ -1207,9 +1194,9 @@ int create_impl(pcexp_ctx* c, const pcexp_mesh* mesh, int p, const pcexp_physics
   PCEXP_TRY(valloc(&c->tmp, Kp));
   PCEXP_TRY(valloc(&c->delta, Kp));
   const size_t nfp = (size_t)(c->F > 0 ? c->F : 1) * c->nfq, nv = (size_t)c->nv;
-  PCEXP_TRY(valloc(&c->G, nfp * nv));
+  PCEXP_TRY(valloc(&c->G, (size_t)(c->fp32 ? face_flux_size(dgdata<float>(c)) : face_flux_size(dgdata<double>(c)))));
   PCEXP_TRY(valloc(&c->dte, c->E));
-  if (!c->jv_tangent) PCEXP_TRY(valloc(&c->Avol, (size_t)c->dim * nv * nv * c->E * c->nq));
+  PCEXP_TRY(valloc(&c->pts, (size_t)4 * c->E * c->nq));
   PCEXP_TRY(valloc(&c->GT, 2 * nv * nfp));
   PCEXP_TRY(valloc(&c->Bface, 2 * nv * nv * nfp));
   PCEXP_TRY(dalloc(c, &c->io64a, Kp));

@@ -12,9 +12,8 @@
 //                   with Fhat_d' = sum_d (A^-1)_{d' d} F_d(U(x_q))
 //   face term     = -|det A|^-1/2 sum_q w_q |f| phi^_i(x_q) F~_n(x_q)
 // Two launches per operator: a face kernel (one thread per face point) writes
-// |f| w_q F~_n into the face-flux buffer G; an element kernel (a tile of elements
-// per block, staged in shared memory) adds the volume term and lifts the face
-// fluxes of its D+1 faces.  Every face flux is computed once and every output is
+// |f| w_q F~_n into the face-flux buffer G; an element kernel (a tile of 32 elements
+// per block) adds the volume term and lifts the face fluxes of its D+1 faces.  Every face flux is computed once and every output is
 // written once, in a fixed order (deterministic).
 //
 // Face points are those of the face's L element (its local face-vertex order).
@@ -47,7 +46,6 @@ template <int D, int P> struct Ord {
   // elements per block (tetrahedra: at most 16, which keeps the FP64 tile within 48 KB)
   static constexpr int ET0 = (256 / NQ) > 128 ? 128 : (256 / NQ);
   static constexpr int ET = (D == 3 && ET0 > 16) ? 16 : ET0;
-  static constexpr int NJV = D * NV * NV;           // volume point-Jacobian entries
   static constexpr int NJF = 2 * NV * NV;           // face point-Jacobian entries
   static constexpr int NBF = NF * NPERM * NFQ * NB;  // trace-table entries
   static constexpr bool SMEM_BF = D == 2;            // stage the trace tables in shared memory
@@ -81,8 +79,76 @@ template <class O> PCEXP_DEV int slot_face(int fs) { return fs >> 4; }
 PCEXP_DEV int slot_side(int fs) { return (fs >> 3) & 1; }
 PCEXP_DEV int slot_perm(int fs) { return fs & 7; }
 
+// Table rows and face-flux records are padded to whole 16-byte vectors where they are read with
+// 16-byte loads.
+template <class T> constexpr int VECW = 16 / (int)sizeof(T);
+template <class T, int N> constexpr int PADV = (N + VECW<T> - 1) / VECW<T> * VECW<T>;
+
+// r[0..N) = p[0..N) from a 16-byte-aligned row (shared memory, or global through the
+// read-only cache), N a multiple of VECW<T>
+template <class T, int N, bool GLOBAL = false>
+PCEXP_DEV void load_row(const T* p, T (&r)[N]) {
+  if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int k = 0; k < N / 4; ++k) {
+      const float4 a = GLOBAL ? __ldg(reinterpret_cast<const float4*>(p) + k) : reinterpret_cast<const float4*>(p)[k];
+      r[4 * k] = a.x;
+      r[4 * k + 1] = a.y;
+      r[4 * k + 2] = a.z;
+      r[4 * k + 3] = a.w;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) {
+      const double2 a = GLOBAL ? __ldg(reinterpret_cast<const double2*>(p) + k) : reinterpret_cast<const double2*>(p)[k];
+      r[2 * k] = a.x;
+      r[2 * k + 1] = a.y;
+    }
+  }
+}
+
+// c[0..N) = p[0..N), coefficients of one variable of an element (read-only in the kernel):
+// 8-byte loads of FP32 pairs when N is even (rows then start on 8-byte boundaries)
+template <class T, int N>
+PCEXP_DEV void load_coeffs(const T* __restrict__ p, T (&c)[N]) {
+  if constexpr (sizeof(T) == 4 && N % 2 == 0) {
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) {
+      const float2 a = __ldg(reinterpret_cast<const float2*>(p) + k);
+      c[2 * k] = a.x;
+      c[2 * k + 1] = a.y;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; ++k) c[k] = __ldg(p + k);
+  }
+}
+
+// Face fluxes G: [F][nv][GS] with GS = nfq rounded up to whole 16-byte vectors, or [F][nv][nfq]
+// (PADG false: the fixed scratch of the no-allocation entry point).
+template <class T, int D, int P, bool PADG = true> constexpr int GSTRIDE = PADG ? PADV<T, Ord<D, P>::NFQ> : Ord<D, P>::NFQ;
+
+// One face point's fluxes into G.  The last point also writes the records' padding: a sector that is
+// never completely written costs a read when it leaves the L2 (face J v on 48^3 cubes: 392 -> 470
+// us without this).
+template <class T, int D, int P, bool PADG>
+PCEXP_DEV void store_face_flux(T* __restrict__ G, int64_t f, int q, const T (&x)[D + 2]) {
+  constexpr int NFQ = Ord<D, P>::NFQ, NV = D + 2, GS = GSTRIDE<T, D, P, PADG>;
+  T* g = G + f * NV * GS + q;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) g[v * GS] = x[v];
+  if constexpr (GS > NFQ) {
+    if (q == NFQ - 1) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int k = 1; k <= GS - NFQ; ++k) g[v * GS + k] = T(0);
+    }
+  }
+}
+
 // ------------------------------------------------------------------ face kernel
-template <class T, int D, int P, bool TAN>
+template <class T, int D, int P, bool TAN, bool PADG>
 __global__ void __launch_bounds__(256) face_kernel(DGData<T> d, const T* __restrict__ u,
                                                    const T* __restrict__ du, T* __restrict__ G,
                                                    const int* __restrict__ skip) {
@@ -151,271 +217,88 @@ __global__ void __launch_bounds__(256) face_kernel(DGData<T> d, const T* __restr
   S Fn[NV];
   roe_flux<D, S, T>(UL, UR, n, d.fs.gamma, Fn, d.rot ? d.vrn[idx] : T(0));
   const T wl = meas * sWf[q];
-  T* g = G + idx * NV;
+  T fx[NV];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) g[v] = wl * PartOf<S>::get(Fn[v]);
-}
-
-// Rows of the element kernel's tables and coefficient tiles are padded to whole 16-byte
-// vectors so that a row is read with 16-byte loads.
-template <class T> constexpr int VECW = 16 / (int)sizeof(T);
-template <class T, int N> constexpr int PADV = (N + VECW<T> - 1) / VECW<T> * VECW<T>;
-
-// r[0..N) = p[0..N) from a 16-byte-aligned row (shared memory, or global through the
-// read-only cache), N a multiple of VECW<T>
-template <class T, int N, bool GLOBAL = false>
-PCEXP_DEV void load_row(const T* p, T (&r)[N]) {
-  if constexpr (sizeof(T) == 4) {
-#pragma unroll
-    for (int k = 0; k < N / 4; ++k) {
-      const float4 a = GLOBAL ? __ldg(reinterpret_cast<const float4*>(p) + k) : reinterpret_cast<const float4*>(p)[k];
-      r[4 * k] = a.x;
-      r[4 * k + 1] = a.y;
-      r[4 * k + 2] = a.z;
-      r[4 * k + 3] = a.w;
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < N / 2; ++k) {
-      const double2 a = GLOBAL ? __ldg(reinterpret_cast<const double2*>(p) + k) : reinterpret_cast<const double2*>(p)[k];
-      r[2 * k] = a.x;
-      r[2 * k + 1] = a.y;
-    }
-  }
-}
-
-// c[0..N) = p[0..N), coefficients of one variable of an element (read-only in the kernel):
-// 8-byte loads of FP32 pairs when N is even (rows then start on 8-byte boundaries)
-template <class T, int N>
-PCEXP_DEV void load_coeffs(const T* __restrict__ p, T (&c)[N]) {
-  if constexpr (sizeof(T) == 4 && N % 2 == 0) {
-#pragma unroll
-    for (int k = 0; k < N / 2; ++k) {
-      const float2 a = __ldg(reinterpret_cast<const float2*>(p) + k);
-      c[2 * k] = a.x;
-      c[2 * k + 1] = a.y;
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < N; ++k) c[k] = __ldg(p + k);
-  }
-}
-
-// lift of the D+1 face fluxes onto test function i of variable v of element e
-template <class T, int D, int P, bool SM>
-PCEXP_DEV T lift_faces(const DGData<T>& d, const T* Bf, const T* __restrict__ G, int64_t e, int v, int i) {
-  using O = Ord<D, P>;
-  constexpr int NB = O::NB, NFQ = O::NFQ, NV = O::NV, NPERM = O::NPERM, NF = O::NF;
-  T lift = 0;
-#pragma unroll
-  for (int k = 0; k < NF; ++k) {
-    const int fs = d.ef[NF * e + k];
-    const T* gf = G + (int64_t)slot_face<O>(fs) * NFQ * NV;
-    const T* tb = Bf + ((k * NPERM + slot_perm(fs)) * NFQ) * NB + i;
-    T a = 0;
-#pragma unroll
-    for (int q = 0; q < NFQ; ++q) a += tab<SM>(tb + q * NB) * gf[q * NV + v];
-    lift = slot_side(fs) ? lift + a : lift - a;
-  }
-  return lift;
+  for (int v = 0; v < NV; ++v) fx[v] = wl * PartOf<S>::get(Fn[v]);
+  store_face_flux<T, D, P, PADG>(G, f, q, fx);
 }
 
 // --------------------------------------------------------------- element kernel
-// Phase 1: one thread per volume point forms the trace (and tangent) of u, the Euler flux
-// and its mapping to reference directions.  Phase 2: a group of S lanes owns one (element,
-// variable) pair and accumulates all nb test functions at once over a strided share of the
-// (point, direction) sum and of the element's faces (the lift pre-scaled by 1/|det A| so it
-// shares the accumulator); a shuffle tree combines the S shares.  Every operand row is read
-// with 16-byte loads and serves all nb accumulators.  (Staging the block's face fluxes and
-// the 3D trace tables in shared memory was measured slower on GB300: the larger footprint
-// costs more occupancy than the L1 traffic it saves.)
-template <class T, int D, int P, bool TAN>
-__global__ void __launch_bounds__(256) elem_kernel(DGData<T> d, const T* __restrict__ u,
-                                                   const T* __restrict__ du, const T* __restrict__ G,
-                                                   T* __restrict__ out, const T* __restrict__ escale,
-                                                   const int* __restrict__ skip, const double* __restrict__ oscale) {
+// The reference tables of one (D, p) in constant memory, read at warp-uniform addresses as operands
+// of the FMAs (outside the load/store pipe).  They depend on the reference simplex alone, so
+// every context of that order uploads the same bytes (upload_tables).
+//   Bv [nq][nb]        phi_j at the volume points
+//   Wm [nq][nb1]       w_q phi_k at the volume points, k < nb1 (the basis of order p - 1)
+//   Cm [D][nb][nb1]    <d phi_i / d xi_d, phi_k>: the gradients of the basis in the basis of order p - 1
+//   Bf [nf][nfq][nb]   phi_j at the face points, the element's own face-vertex order
+template <int D, int P> struct TabLayout {
   using O = Ord<D, P>;
-  constexpr int NB = O::NB, NQ = O::NQ, NFQ = O::NFQ, ET = O::ET, NVB = O::NVB, NV = O::NV, GEO = O::GEO;
-  constexpr int DV = D * NV, NF = O::NF, NPERM = O::NPERM;
-  constexpr int NBP = PADV<T, NB>;
-  constexpr bool SM = O::SMEM_BF;
-  constexpr int NPAIR = ET * NV;
-  constexpr int S = (NPAIR * 8 <= 256) ? 8 : (NPAIR * 4 <= 256) ? 4 : (NPAIR * 2 <= 256) ? 2 : 1;
-  constexpr int ROUNDS = (NPAIR * S + 255) / 256;
-  using Sc = typename std::conditional<TAN, Tangent<T>, T>::type;
-  __shared__ __align__(16) T sBv[NQ * NBP];
-  __shared__ __align__(16) T sDv[D * NQ * NBP];
-  __shared__ __align__(16) T sBf[SM ? NF * NPERM * NFQ * NBP : 1];
-  __shared__ __align__(16) T su[ET * NV * NBP];
-  __shared__ __align__(16) T sdu[TAN ? ET * NV * NBP : 1];
-  __shared__ T sF[ET * NQ * DV];
-  __shared__ T sgeo[ET * GEO];
-  if (skip && *skip) return;
-  const int64_t e0 = (int64_t)blockIdx.x * ET;
-  const int ne = (int)((d.E - e0) < ET ? (d.E - e0) : ET);
-  for (int i = threadIdx.x; i < NQ * NBP; i += blockDim.x) {
-    const int r = i / NBP, j = i - r * NBP;
-    sBv[i] = j < NB ? d.Bv[r * NB + j] : T(0);
+  static constexpr int NB1 = P == 0 ? 0 : Ord<D, P == 0 ? 0 : P - 1>::NB;
+  static constexpr int BV = 0, WM = BV + O::NQ * O::NB, CM = WM + O::NQ * NB1, BF = CM + D * O::NB * NB1;
+  static constexpr int N = BF + O::NF * O::NFQ * O::NB;
+};
+template <class T, int D, int P> __constant__ T c_tab[TabLayout<D, P>::N];
+
+// Degree of basis function i (the basis is graded)
+template <int D> __host__ __device__ constexpr int degree_of(int i) {
+  int deg = 0, n = 1;
+  while (i >= n) {
+    ++deg;
+    n += D == 2 ? deg + 1 : (deg + 1) * (deg + 2) / 2;
   }
-  for (int i = threadIdx.x; i < D * NQ * NBP; i += blockDim.x) {
-    const int r = i / NBP, j = i - r * NBP;
-    sDv[i] = j < NB ? d.Dv[r * NB + j] : T(0);
+  return deg;
+}
+template <int D> __host__ __device__ constexpr int basis_size(int p) {
+  return p < 0 ? 0 : D == 2 ? (p + 1) * (p + 2) / 2 : (p + 1) * (p + 2) * (p + 3) / 6;
+}
+
+// What the volume term is the flux of: the state u (residual), or the flux's derivative along du at
+// u, from the traces of u (TANGENT) or from the point values stored by the linearisation (STORED).
+enum ElemMode { ELEM_FLUX = 0, ELEM_TANGENT = 1, ELEM_STORED = 2 };
+
+// The NFQ fluxes of one face and variable in the order of the element's own face points: the L
+// element's as stored; on the R side the points of a symmetric rule are permuted with the face
+// vertices (2D: reversed; the 7-point rule: the centroid, then two orbits of three points whose
+// distinguished vertices are 0, 2, 1).
+template <class T, int D, int P, int GS>
+PCEXP_DEV void face_fluxes(const T (&r)[GS], int fs, T (&x)[Ord<D, P>::NFQ]) {
+  constexpr int NFQ = Ord<D, P>::NFQ;
+  const int side = slot_side(fs);
+  if constexpr (D == 2) {
+#pragma unroll
+    for (int q = 0; q < NFQ; ++q) x[q] = side ? r[NFQ - 1 - q] : r[q];
+  } else if constexpr (NFQ == 7) {
+    // entry s' of an orbit comes from the L vertex s with perm(s) = s'
+    constexpr unsigned long long INV = 36ull | 24ull << 6 | 33ull << 12 | 18ull << 18 | 9ull << 24 | 6ull << 30;
+    const int code = (int)(INV >> (6 * slot_perm(fs))) & 63;
+    constexpr int AT[3] = {0, 2, 1};  // position in the orbit of the point distinguished by vertex s
+    x[0] = r[0];
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+      const int from = (code >> (2 * s)) & 3;
+#pragma unroll
+      for (int o = 1; o <= 4; o += 3) x[o + AT[s]] = from == 0 ? r[o + AT[0]] : from == 1 ? r[o + AT[1]] : r[o + AT[2]];
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < NFQ; ++q) x[q] = r[q];
   }
-  if constexpr (SM)
-    for (int i = threadIdx.x; i < NF * NPERM * NFQ * NBP; i += blockDim.x) sBf[i] = d.BfP[i];
-  for (int i = threadIdx.x; i < ne * NV * NBP; i += blockDim.x) {
-    const int r = i / NBP, j = i - r * NBP;
-    su[i] = j < NB ? u[e0 * NVB + r * NB + j] : T(0);
-    if constexpr (TAN) sdu[i] = j < NB ? du[e0 * NVB + r * NB + j] : T(0);
-  }
-  for (int i = threadIdx.x; i < ne * GEO; i += blockDim.x) sgeo[i] = d.geo[e0 * GEO + i];
-  __syncthreads();
-  const T g = d.fs.gamma;
-  const T osc = oscale ? (T)*oscale : T(1);
-  // phase 1: flux at each volume point, mapped to reference directions
-  for (int it = threadIdx.x; it < ne * NQ; it += blockDim.x) {
-    const int el = it / NQ, q = it - el * NQ;
-    const T* ge = sgeo + el * GEO;
-    const T isd = ge[O::ISD];
-    T b[NBP];
-    load_row<T, NBP>(sBv + q * NBP, b);
-    Sc U[NV];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      T c[NBP];
-      load_row<T, NBP>(su + (el * NV + v) * NBP, c);
-      T a = 0;
+  for (int q = 0; q < NFQ; ++q) x[q] = side ? x[q] : -x[q];
+}
+
+// acc[i] += sum_k C[i][k] m[k] for i >= I: the gradient of a function of degree g lies in degrees < g
+template <class T, int D, int P, int I, int N>
+PCEXP_DEV void combine_modes(const T* C, const T (&m)[N], T (&acc)[Ord<D, P>::NB]) {
+  if constexpr (I < Ord<D, P>::NB) {
+    constexpr int n = basis_size<D>(degree_of<D>(I) - 1);
 #pragma unroll
-      for (int j = 0; j < NB; ++j) a = fma(b[j], c[j], a);
-      if constexpr (TAN) {
-        load_row<T, NBP>(sdu + (el * NV + v) * NBP, c);
-        T t = 0;
-#pragma unroll
-        for (int j = 0; j < NB; ++j) t = fma(b[j], c[j], t);
-        U[v] = Sc{a * isd, t * isd};
-      } else {
-        U[v] = a * isd;
-      }
-    }
-    Sc F[D][NV];
-    euler_flux<D, Sc, T>(U, g, F);
-    if (d.rot) {  // rotating frame: F - U v_r^T at the point
-      const T* vr = d.vrq + ((e0 + el) * NQ + q) * D;
-#pragma unroll
-      for (int k = 0; k < D; ++k)
-#pragma unroll
-        for (int v = 0; v < NV; ++v) F[k][v] = F[k][v] - U[v] * vr[k];
-    }
-    T* fo = sF + (el * NQ + q) * DV;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      T fk[D];
-#pragma unroll
-      for (int k = 0; k < D; ++k) fk[k] = PartOf<Sc>::get(F[k][v]);
-#pragma unroll
-      for (int dd = 0; dd < D; ++dd) {
-        T a = ge[dd * D] * fk[0];
-#pragma unroll
-        for (int k = 1; k < D; ++k) a += ge[dd * D + k] * fk[k];
-        fo[dd * NV + v] = a;
-      }
-    }
-  }
-  __syncthreads();
-  const T* Bf = SM ? sBf : d.BfP;
-  // phase 2: S lanes per (element, variable): test against grad phi and lift the faces
-  const int ls = threadIdx.x % S;
-#pragma unroll 1
-  for (int round = 0; round < ROUNDS; ++round) {
-    const int pr = round * (256 / S) + (int)threadIdx.x / S;
-    const bool act = pr < ne * NV;
-    const int prc = act ? pr : 0;
-    const int el = prc / NV, v = prc - (prc / NV) * NV;
-    T acc[NB];
-#pragma unroll
-    for (int i = 0; i < NB; ++i) acc[i] = T(0);
-    for (int k = ls; k < NQ * D; k += S) {
-      const int q = k / D, dd = k - (k / D) * D;
-      const T f = sF[(el * NQ + q) * DV + dd * NV + v];
-      T row[NBP];
-      load_row<T, NBP>(sDv + (dd * NQ + q) * NBP, row);
-#pragma unroll
-      for (int i = 0; i < NB; ++i) acc[i] = fma(row[i], f, acc[i]);
-    }
-    const int64_t e = e0 + el;
-    const T isd = sgeo[el * GEO + O::ISD];
-    const T rdet = isd * isd;  // the lift carries 1/sqrt|det|, the volume term sqrt|det|
-    for (int kf = ls; kf < NF; kf += S) {
-      const int fs = d.ef[NF * e + kf];
-      const T* gf = G + (int64_t)slot_face<O>(fs) * NFQ * NV;
-      const T* tb = Bf + ((kf * NPERM + slot_perm(fs)) * NFQ) * NBP;
-      const T sg = slot_side(fs) ? rdet : -rdet;
-#pragma unroll
-      for (int q = 0; q < NFQ; ++q) {
-        const T gq = sg * gf[q * NV + v];
-        T row[NBP];
-        load_row<T, NBP, !SM>(tb + q * NBP, row);
-#pragma unroll
-        for (int i = 0; i < NB; ++i) acc[i] = fma(row[i], gq, acc[i]);
-      }
-    }
-#pragma unroll
-    for (int off = S / 2; off >= 1; off /= 2)
-#pragma unroll
-      for (int i = 0; i < NB; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
-    if (act) {
-      const T es = escale ? escale[e] : T(1);
-      const T sc = sgeo[el * GEO + O::SD] * osc * es;
-      const bool src = d.rot && v >= 1 && v <= D;
-#pragma unroll
-      for (int i = 0; i < NB; ++i)
-        if (i % S == ls) {
-          T o = acc[i] * sc;
-          if (src) {  // the rotating frame's source, on the coefficients of u (R) or du (J v)
-            const T* xr = (TAN ? sdu : su) + el * NV * NBP + i;
-            T m[D];
-#pragma unroll
-            for (int k = 0; k < D; ++k) m[k] = xr[(1 + k) * NBP];
-            o += rot_source<T, D>(d.om, m, v - 1) * osc * es;
-          }
-          out[e * NVB + v * NB + i] = o;
-        }
-    }
+    for (int k = 0; k < n; ++k) acc[I] = fma(C[I * TabLayout<D, P>::NB1 + k], m[k], acc[I]);
+    combine_modes<T, D, P, I + 1>(C, m, acc);
   }
 }
 
-template <class T, int D, int P>
-cudaError_t dg_op_p(const DGData<T>& d, const T* u, const T* du, T* out, T* G, const T* escale, const int* skip,
-                    const double* oscale, cudaStream_t st, const cudaEvent_t* ev) {
-  using O = Ord<D, P>;
-  const int64_t nfp = d.F * O::NFQ;
-  if (ev) cudaEventRecord(ev[0], st);
-  if (nfp > 0) {
-    const int64_t nb = (nfp + 255) / 256;
-    if (du) face_kernel<T, D, P, true><<<(unsigned)nb, 256, 0, st>>>(d, u, du, G, skip);
-    else face_kernel<T, D, P, false><<<(unsigned)nb, 256, 0, st>>>(d, u, du, G, skip);
-  }
-  if (ev) cudaEventRecord(ev[1], st);
-  const int64_t eb = (d.E + O::ET - 1) / O::ET;
-  if (du) elem_kernel<T, D, P, true><<<(unsigned)eb, 256, 0, st>>>(d, u, du, G, out, escale, skip, oscale);
-  else elem_kernel<T, D, P, false><<<(unsigned)eb, 256, 0, st>>>(d, u, du, G, out, escale, skip, oscale);
-  if (ev) cudaEventRecord(ev[2], st);
-  return cudaGetLastError();
-}
-
-// ------------------------------------- FP32 volume J v by flux tangents, one element per lane
-// The reference tables [Bv (nq x nb) | Dv (D x nq x nb)] of one (D, p) in constant memory.
-// They depend on the reference simplex alone, so every context of that order uploads the
-// same bytes (tan_tables_p); the kernel below reads them at warp-uniform addresses, which
-// the constant cache serves as broadcasts outside the load/store pipe.
-template <int D, int P> __constant__ float c_tan[(D + 1) * Ord<D, P>::NQ * Ord<D, P>::NB];
-
-// ---------------------------------- the same J v volume part as a pipelined persistent kernel
-// cp.async copies (global -> shared, no register staging), 4 or 16 bytes
-PCEXP_DEV void cp_async4(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
+// cp.async copies (global -> shared, no register staging)
 PCEXP_DEV void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
                "l"(src)
@@ -424,258 +307,388 @@ PCEXP_DEV void cp_async16(void* dst, const void* src) {
 PCEXP_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 PCEXP_DEV void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Shared-memory words of one stage of elem_tan_pipe_kernel<D, P>: u, u' rows, face fluxes,
-// geometry records and face slots of 32 elements.
-template <int D, int P> struct TanPipe {
-  using O = Ord<D, P>;
-  static constexpr int NBP = PADV<float, O::NB>;
-  static constexpr int UR0 = 2 * O::NV * NBP;
-  static constexpr int UROW = UR0 + (36 - UR0 % 32) % 32;
-  static constexpr int GREC = O::NF * O::NFQ * O::NV;
-  static constexpr int GROW = GREC | 1;
-  static constexpr int PST = O::NVB | 1;
-  static constexpr int SU = 32 * UROW, SG = 32 * GROW, SGEO = 32 * O::GEO, SEF = 32 * O::NF;
-  // warps per block: with two 41 KB stages two blocks fit an SM (P2); six warps each keep the
-  // registers of 2 x 192 threads within the SM's file and split the 14 points 3/3/2/2/2/2
-  static constexpr int WARPS = D == 3 ? 6 : O::NF;
-  static constexpr int PART = WARPS * 32 * PST;
-  // the partial sums reuse the consumed rows and face fluxes (not the geometry records)
-  static constexpr int SROWS = ((SU + SG > PART ? SU + SG : PART) + 3) / 4 * 4;
-  static constexpr int STAGE = SROWS + SGEO + SEF;  // words (SGEO and SU keep 16-byte alignment)
-  static_assert(SU % 4 == 0, "16-byte alignment of the face fluxes");
-  static constexpr size_t BYTES = 2 * (size_t)STAGE * 4;
-};
-
-// Persistent element kernel of the FP32 J v on tetrahedra: a block of six warps loops over
-// tiles of 32 elements (one element per lane; the warps split the volume points and the
-// faces, so every reference-table index is warp-uniform and the tables are read from constant
-// memory).  While tile t is computed, tile t + gridDim.x is copied into the other
-// shared-memory stage by cp.async: its u, u' rows and geometry records at the start of the
-// tile, its face fluxes (gathered through its face slots, which are loaded into a register at
-// the start and are needed only then) after the volume loop.  The staging latency is hidden
-// behind a tile of compute.
-template <int D, int P>
-__global__ void __launch_bounds__(32 * TanPipe<D, P>::WARPS, 2) elem_tan_pipe_kernel(DGData<float> d, const float* __restrict__ u,
-                                                                     const float* __restrict__ du,
-                                                                     const float* __restrict__ G, float* __restrict__ out,
-                                                                     const float* __restrict__ escale,
-                                                                     const int* __restrict__ skip,
-                                                                     const double* __restrict__ oscale, int64_t ntiles) {
-  using O = Ord<D, P>;
-  using L = TanPipe<D, P>;
-  constexpr int NB = O::NB, NQ = O::NQ, NFQ = O::NFQ, NV = O::NV, NF = O::NF, NPERM = O::NPERM, GEO = O::GEO;
-  constexpr int NVB = O::NVB, QW = L::WARPS, NT = 32 * QW;
-  static_assert(NT >= 32 * NF, "one thread per (element, face) slot of a tile");
-  constexpr int NBP = L::NBP, UROW = L::UROW, GROW = L::GROW, PST = L::PST;
-  static_assert(!O::SMEM_BF, "tetrahedra read the trace tables through the read-only cache");
-  extern __shared__ __align__(16) float dsm[];
-  if (skip && *skip) return;
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  int64_t t = blockIdx.x;
-  if (t >= ntiles) return;
-  const float g = d.fs.gamma;
-  const float osc = oscale ? (float)*oscale : 1.f;
-
-  // copies of tile tt into stage S: u, u' rows (4-byte copies into padded rows), geometry
-  // records (16-byte copies); the face fluxes follow once the face slots are known
-  auto stage_rows = [&](int64_t tt, float* S) {
-    const int64_t e0 = tt * 32;
-    const int ne = (int)((d.E - e0) < 32 ? (d.E - e0) : 32);
-    float* su = S;
-    float* sgeo = S + L::SROWS;
-    for (int i = tid; i < ne * NVB; i += NT) {
-      const int el = i / NVB, r = i - el * NVB, v = r / NB, j = r - v * NB;
-      cp_async4(su + el * UROW + v * NBP + j, u + e0 * NVB + i);
-      cp_async4(su + el * UROW + (NV + v) * NBP + j, du + e0 * NVB + i);
-    }
-    for (int i = tid; i < ne * (GEO / 4); i += NT) cp_async16(sgeo + 4 * i, d.geo + e0 * GEO + 4 * i);
-  };
-  auto stage_faces = [&](int64_t tt, float* S, int fs) {
-    const int64_t e0 = tt * 32;
-    const int ne = (int)((d.E - e0) < 32 ? (d.E - e0) : 32);
-    if (tid < ne * NF) {
-      int* sef = reinterpret_cast<int*>(S + L::SROWS + L::SGEO);
-      sef[tid] = fs;
-      const int el = tid / NF, kf = tid - el * NF;
-      float* dst = S + L::SU + el * GROW + kf * NFQ * NV;
-      const float* src = G + (int64_t)slot_face<O>(fs) * NFQ * NV;
-#pragma unroll 5
-      for (int k = 0; k < NFQ * NV; ++k) cp_async4(dst + k, src + k);
-    }
-  };
-
-  // prologue: tile t into stage 0
-  {
-    stage_rows(t, dsm);
-    const int64_t e0 = t * 32;
-    const int ne = (int)((d.E - e0) < 32 ? (d.E - e0) : 32);
-    const int fs = tid < ne * NF ? d.ef[e0 * NF + tid] : 0;
-    stage_faces(t, dsm, fs);
-    cp_async_commit();
-    cp_async_wait_all();
-    __syncthreads();
-  }
-  for (int it = 0; t < ntiles; ++it, t += gridDim.x) {
-    float* S = dsm + (it & 1) * L::STAGE;
-    float* N = dsm + ((it & 1) ^ 1) * L::STAGE;
-    const int64_t e0 = t * 32;
-    const int ne = (int)((d.E - e0) < 32 ? (d.E - e0) : 32);
-    const int64_t tn = t + gridDim.x;
-    const bool has_next = tn < ntiles;
-    int fs_next = 0;
-    if (has_next) {
-      stage_rows(tn, N);
-      const int64_t en0 = tn * 32;
-      const int nen = (int)((d.E - en0) < 32 ? (d.E - en0) : 32);
-      if (tid < nen * NF) fs_next = d.ef[en0 * NF + tid];
-    }
-    const float* su = S;
-    const float* sg = S + L::SU;
-    const float* sgeo = S + L::SROWS;
-    const int* sef = reinterpret_cast<const int*>(S + L::SROWS + L::SGEO);
-    const int el = lane < ne ? lane : 0;  // lanes past the last element repeat element 0; discarded
-    const float* ge = sgeo + el * GEO;
-    float Ai[D * D];
-#pragma unroll
-    for (int k = 0; k < D * D; ++k) Ai[k] = ge[k];
-    const float isd = ge[O::ISD];
-    float acc[NV][NB];
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int i = 0; i < NB; ++i) acc[v][i] = 0.f;
-    const float* ur = su + el * UROW;
-    // flux tangent at volume point q mapped to reference directions, tested (accumulated)
-    auto point = [&](int q, const Tangent<float>(&U)[NV]) {
-      Tangent<float> F[D][NV];
-      euler_flux<D, Tangent<float>, float>(U, g, F);
-      const float* dq = c_tan<D, P> + NQ * NB + q * NB;
-#pragma unroll
-      for (int dd = 0; dd < D; ++dd) {
-        float fh[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          float a = Ai[dd * D] * F[0][v].d;
-#pragma unroll
-          for (int k = 1; k < D; ++k) a += Ai[dd * D + k] * F[k][v].d;
-          fh[v] = a;
-        }
-#pragma unroll
-        for (int i = 0; i < NB; ++i) {
-          const float tq = dq[dd * NQ * NB + i];
-#pragma unroll
-          for (int v = 0; v < NV; ++v) acc[v][i] = fmaf(tq, fh[v], acc[v][i]);
-        }
-      }
-    };
-    // two of the warp's points per pass: each u, u' row read from shared memory serves both
-    // traces (the rows are the kernel's main shared-memory traffic)
-#pragma unroll 1
-    for (int q0 = w; q0 < NQ; q0 += 2 * QW) {
-      const int q1 = q0 + QW;
-      const bool two = q1 < NQ;  // warp-uniform
-      const float* b0 = c_tan<D, P> + q0 * NB;
-      const float* b1 = c_tan<D, P> + (two ? q1 : q0) * NB;
-      Tangent<float> U0[NV], U1[NV];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        float c[NBP];
-        load_row<float, NBP>(ur + v * NBP, c);
-        float a0 = 0.f, a1 = 0.f;
-#pragma unroll
-        for (int j = 0; j < NB; ++j) {
-          a0 = fmaf(b0[j], c[j], a0);
-          a1 = fmaf(b1[j], c[j], a1);
-        }
-        load_row<float, NBP>(ur + (NV + v) * NBP, c);
-        float t0 = 0.f, t1 = 0.f;
-#pragma unroll
-        for (int j = 0; j < NB; ++j) {
-          t0 = fmaf(b0[j], c[j], t0);
-          t1 = fmaf(b1[j], c[j], t1);
-        }
-        U0[v] = Tangent<float>{a0 * isd, t0 * isd};
-        U1[v] = Tangent<float>{a1 * isd, t1 * isd};
-        asm volatile("" ::: "memory");  // one variable's rows in flight at a time (registers)
-      }
-      point(q0, U0);
-      if (two) point(q1, U1);
-    }
-    // the next tile's face fluxes, now that its face slots have arrived
-    if (has_next) stage_faces(tn, N, fs_next);
-    cp_async_commit();
-    // faces: lift of the staged face fluxes, pre-scaled by 1/|det A| to share the accumulators;
-    // faces 0..NF-2 go whole to the last warps (warp QW - 1 - kf, which have fewer volume
-    // points); the points of face NF-1 are split between warps 0 and 1, so that no warp waits
-    // at the tile's barriers for one that has a whole face more
-    // (with 14 points, 3/3/2/2/2/2 over six warps, the four warps of two points take one whole
-    // face each instead)
-    static_assert(QW - (NF - 1) >= 2, "two warps share the last face");
-    constexpr bool FACE_PER_LIGHT_WARP = QW - NQ % QW == NF;
-    const float rdet = isd * isd;
-    int kf = -1, qa = 0, qb = NFQ;
-    if constexpr (FACE_PER_LIGHT_WARP) {
-      if (w >= QW - NF) kf = QW - 1 - w;
-    } else {
-      if (w >= QW - (NF - 1)) {
-        kf = QW - 1 - w;
-      } else if (w < 2) {
-        kf = NF - 1;
-        qa = w == 0 ? 0 : (NFQ + 1) / 2;
-        qb = w == 0 ? (NFQ + 1) / 2 : NFQ;
-      }
-    }
-    if (kf >= 0) {  // warp-uniform
-      const int fs = sef[el * NF + kf];
-      const float sgn = slot_side(fs) ? rdet : -rdet;
-      const float* tb = d.BfP + ((kf * NPERM + slot_perm(fs)) * NFQ) * NBP;
-      const float* gr = sg + el * GROW + kf * NFQ * NV;
-#pragma unroll
-      for (int q = 0; q < NFQ; ++q) {
-        if (q < qa || q >= qb) continue;  // warp-uniform
-        float row[NBP];
-        load_row<float, NBP, true>(tb + q * NBP, row);
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          const float gq = sgn * gr[q * NV + v];
-#pragma unroll
-          for (int i = 0; i < NB; ++i) acc[v][i] = fmaf(row[i], gq, acc[v][i]);
-        }
-      }
-    }
-    __syncthreads();  // the stage is consumed; the partial sums reuse it
-    float* part = S;
-    float* pr = part + (w * 32 + lane) * PST;
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int i = 0; i < NB; ++i) pr[v * NB + i] = acc[v][i];
-    __syncthreads();
-    for (int o = tid; o < ne * NVB; o += NT) {
-      const int el2 = o / NVB, r = o - el2 * NVB;
-      float s = part[el2 * PST + r];
-#pragma unroll
-      for (int ww = 1; ww < QW; ++ww) s += part[(ww * 32 + el2) * PST + r];
-      float sc = sgeo[el2 * GEO + O::SD] * osc;
-      if (escale) sc *= escale[e0 + el2];
-      out[e0 * NVB + o] = s * sc;
-    }
-    cp_async_wait_all();
-    __syncthreads();  // next stage landed; this stage's partial sums are read
-  }
+// Four values from a 16-byte boundary, issued where it stands (volatile: not sunk past a barrier
+// to the first use)
+PCEXP_DEV void load_early(const float* p, float (&x)[4]) {
+  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3])
+               : "l"(p));
+}
+PCEXP_DEV void load_early(const double* p, double (&x)[4]) {
+  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(x[0]), "=d"(x[1]) : "l"(p));
+  asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(x[2]), "=d"(x[3]) : "l"(p + 2));
 }
 
-template <int D, int P>
-cudaError_t tan_tables_p(const DGData<float>& d, cudaStream_t st) {
+template <class T, int D, int P, int MODE> struct ElemTile {
   using O = Ord<D, P>;
-  cudaError_t e = cudaSuccess;
-  if constexpr (D == 3) {
-    e = cudaFuncSetAttribute(elem_tan_pipe_kernel<D, P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)TanPipe<D, P>::BYTES);
-    if (e != cudaSuccess) return e;
+  static constexpr int ET = 32, NT = ET * O::NV;
+  static constexpr int RS = O::NVB | 1;  // odd row stride: lanes (elements) hit distinct banks
+  static constexpr int ROWS = ET * RS * (MODE == ELEM_TANGENT ? 2 : 1);
+  static constexpr int FLUX = P == 0 ? 0 : O::NQ * D * O::NV * ET;
+  // FP32: the threads' own face-flux records, copied in while the volume part is computed
+  static constexpr bool AHEAD = sizeof(T) == 4;
+  static constexpr int GV = GSTRIDE<T, D, P> / VECW<T>;  // 16-byte vectors of a record
+  static constexpr int ROWS4 = (ROWS + 3) / 4 * 4;       // the records start on a 16-byte boundary
+  static constexpr int RECS = AHEAD ? O::NF * GV * NT * VECW<T> : 0;
+  static constexpr size_t BYTES = sizeof(T) * (size_t)(ROWS4 + RECS + FLUX);
+  // blocks per SM the registers are bounded for (the shared memory allows as many or more)
+  static constexpr int MINB = sizeof(T) == 4 ? (D == 3 ? 4 : 5) : (D == 3 ? 2 : 3);
+};
+
+// A block owns 32 elements and has a warp per variable.
+//   Phase 1: lane = element, the warps share the volume points.  Each lane reads its element's rows
+//   from shared memory once for all its warp's points, forms the traces, the flux (or its
+//   derivative) in the element's reference directions (contravariant form: q_d = A^-1_d . v, no
+//   Cartesian flux is formed and mapped) and stores it as [point][direction][variable][element].
+//   Phase 2: lane = element, warp = variable.  Each thread tests its variable's flux against the
+//   gradients and lifts its face fluxes, nb accumulators in registers.  The gradients of P^p lie
+//   in P^(p-1): the fluxes are first projected on that basis (Wm), then combined (Cm), e.g. 249
+//   instead of 420 FMAs per variable on tetrahedra at p = 2.
+// Every table index is warp-uniform, every shared-memory access conflict-free, and no partial
+// sums cross warps; both forms (FP32 and FP64) run the same code.  FP32 is bound by instruction
+// issue and, on meshes whose face fluxes leave the L2, by the latency of their gather: each thread
+// copies its records into shared memory by cp.async before the volume part (48^3 cubes at p = 2:
+// 509 us without that).  FP64 is bound by its pipe.
+// Measured against the kernels this one replaces, per launch of the Krylov J v: FP32 48^3 cubes at
+// p = 2 449 -> 277 us (a persistent kernel whose six warps each kept 50 partial sums and recomputed
+// the flux derivative from u), FP32 131,072 triangles at p = 3 111 -> 32 us (lanes sharing an
+// element's test functions), FP64 20^3 cubes at p = 2 485 -> 427 us (stored D nv x nv Jacobians);
+// the residual's: FP64 24^3 cubes at p = 2 1117 -> 717 us.
+template <class T, int D, int P, int MODE, bool PADG>
+__global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P, MODE>::MINB)
+    elem_op_kernel(DGData<T> d, const T* __restrict__ u, const T* __restrict__ du, const T* __restrict__ pts,
+                   const T* __restrict__ G, T* __restrict__ out, const T* __restrict__ escale,
+                   const int* __restrict__ skip, const double* __restrict__ oscale) {
+  using O = Ord<D, P>;
+  using L = ElemTile<T, D, P, MODE>;
+  using X = TabLayout<D, P>;
+  constexpr int NB = O::NB, NQ = O::NQ, NFQ = O::NFQ, NV = O::NV, NVB = O::NVB, GEO = O::GEO, NF = O::NF;
+  constexpr int NPERM = O::NPERM, ET = L::ET, RS = L::RS, NB1 = X::NB1;
+  constexpr int GS = GSTRIDE<T, D, P, PADG>;
+  extern __shared__ __align__(16) unsigned char elem_dyn[];
+  T* rows = reinterpret_cast<T*>(elem_dyn);
+  T* sG = rows + L::ROWS4;  // [face][vector][thread][16 bytes]
+  T* sF = sG + L::RECS;
+  if (skip && *skip) return;
+  const T* tab = c_tab<T, D, P>;
+  const int64_t e0 = (int64_t)blockIdx.x * ET;
+  const int ne = (int)((d.E - e0) < ET ? (d.E - e0) : ET);
+  // the warp's index through a shuffle, so that it is known to be uniform (table loads by it)
+  const int lane = threadIdx.x & 31, w = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
+  const int64_t e = e0 + (lane < ne ? lane : 0);  // lanes past the last element repeat element e0; discarded
+  int slots[NF];
+  if constexpr (NF == 4) {
+    const int4 s4 = __ldg(reinterpret_cast<const int4*>(d.ef) + e);
+    slots[0] = s4.x;
+    slots[1] = s4.y;
+    slots[2] = s4.z;
+    slots[NF - 1] = s4.w;
+  } else {
+#pragma unroll
+    for (int k = 0; k < NF; ++k) slots[k] = __ldg(d.ef + NF * e + k);
   }
-  return cudaMemcpyToSymbolAsync(c_tan<D, P>, d.Bv, sizeof(float) * (D + 1) * O::NQ * O::NB, 0,
-                                 cudaMemcpyDeviceToDevice, st);
+  // the tile's rows: ET * NVB = NT * NB values, all loads issued before the first store
+  {
+    const T* src = (MODE == ELEM_FLUX ? u : du) + e0 * NVB;
+    T x[NB], y[MODE == ELEM_TANGENT ? NB : 1];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+      const int i = threadIdx.x + k * L::NT;
+      x[k] = i < ne * NVB ? src[i] : T(0);
+      if constexpr (MODE == ELEM_TANGENT) y[k] = i < ne * NVB ? u[e0 * NVB + i] : T(0);
+    }
+    if constexpr (L::AHEAD) {
+#pragma unroll
+      for (int k = 0; k < NF; ++k) {
+        const T* g = G + ((int64_t)slot_face<O>(slots[k]) * NV + w) * GS;
+#pragma unroll
+        for (int h = 0; h < L::GV; ++h)
+          cp_async16(sG + ((k * L::GV + h) * L::NT + threadIdx.x) * VECW<T>, g + h * VECW<T>);
+      }
+      cp_async_commit();
+    }
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+      const int i = threadIdx.x + k * L::NT, r = i / NVB * RS + i % NVB;
+      if (i < ne * NVB) {
+        rows[r] = x[k];
+        if constexpr (MODE == ELEM_TANGENT) rows[ET * RS + r] = y[k];
+      }
+    }
+  }
+  T ge[GEO];
+  load_row<T, GEO, true>(d.geo + GEO * e, ge);
+  const T isd = ge[O::ISD];
+  constexpr int PP = P == 0 ? 1 : (NQ + NV - 1) / NV;  // points per warp
+  T pv[MODE == ELEM_STORED ? PP : 1][4];
+  if constexpr (MODE == ELEM_STORED && P > 0) {
+#pragma unroll
+    for (int i = 0; i < PP; ++i) load_early(pts + ((int64_t)(w + i * NV < NQ ? w + i * NV : w) * d.E + e) * 4, pv[i]);
+  }
+  __syncthreads();
+  const int el = lane < ne ? lane : 0;
+  if constexpr (P > 0) {
+    const T gm = d.fs.gamma - T(1);
+    T Ai[D][D];
+#pragma unroll
+    for (int k = 0; k < D * D; ++k) Ai[k / D][k % D] = ge[k];
+    // traces of this lane's element at the warp's points q = w, w + NV, ... (the last may be past NQ:
+    // it repeats the warp's first point and is not stored)
+    T t[PP][NV], s[MODE == ELEM_TANGENT ? PP : 1][NV];
+    const T* ra = rows + el * RS;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+#pragma unroll
+      for (int i = 0; i < PP; ++i) {
+        t[i][v] = T(0);
+        if constexpr (MODE == ELEM_TANGENT) s[i][v] = T(0);
+      }
+#pragma unroll
+      for (int j = 0; j < NB; ++j) {
+        const T c = ra[v * NB + j];
+        T c2 = T(0);
+        if constexpr (MODE == ELEM_TANGENT) c2 = ra[ET * RS + v * NB + j];
+#pragma unroll
+        for (int i = 0; i < PP; ++i) {
+          const int q = w + i * NV < NQ ? w + i * NV : w;
+          const T b = tab[X::BV + q * NB + j];
+          t[i][v] = fma(b, c, t[i][v]);
+          if constexpr (MODE == ELEM_TANGENT) s[i][v] = fma(b, c2, s[i][v]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < PP; ++i) {
+      const int q = w + i * NV;
+      if (q >= NQ) break;  // warp-uniform
+      T vel[D], H, k2 = T(0);
+      T F[D][NV];
+      if constexpr (MODE == ELEM_STORED) {
+#pragma unroll
+        for (int k = 0; k < D; ++k) vel[k] = pv[MODE == ELEM_STORED ? i : 0][k];
+        H = pv[MODE == ELEM_STORED ? i : 0][D];
+#pragma unroll
+        for (int k = 0; k < D; ++k) k2 = fma(T(0.5) * vel[k], vel[k], k2);
+      } else {
+        T U[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) U[v] = (MODE == ELEM_TANGENT ? s[MODE == ELEM_TANGENT ? i : 0][v] : t[i][v]) * isd;
+        const T ir = T(1) / U[0];
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+          vel[k] = U[1 + k] * ir;
+          k2 = fma(T(0.5) * vel[k], vel[k], k2);
+        }
+        const T p = gm * (U[NV - 1] - k2 * U[0]);
+        if constexpr (MODE == ELEM_FLUX) {
+#pragma unroll
+          for (int dd = 0; dd < D; ++dd) {
+            T qd = Ai[dd][0] * vel[0];
+#pragma unroll
+            for (int k = 1; k < D; ++k) qd = fma(Ai[dd][k], vel[k], qd);
+            F[dd][0] = U[0] * qd;
+#pragma unroll
+            for (int k = 0; k < D; ++k) F[dd][1 + k] = fma(U[1 + k], qd, Ai[dd][k] * p);
+            F[dd][NV - 1] = (U[NV - 1] + p) * qd;
+          }
+          if (d.rot) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) t[i][v] = U[v];
+          }
+        }
+        H = (U[NV - 1] + p) * ir;
+      }
+      if constexpr (MODE != ELEM_FLUX) {
+        // derivative along the trace t: with w_d = rho dq_d = A^-1_d . dm - q_d drho,
+        // dF_d = (A^-1_d . dm, v w_d + q_d dm + A^-1_d dp, H w_d + q_d (dE + dp))
+        T dp = fma(k2, t[i][0], t[i][NV - 1]);
+#pragma unroll
+        for (int k = 0; k < D; ++k) dp = fma(-vel[k], t[i][1 + k], dp);
+        dp *= gm;
+        const T de = t[i][NV - 1] + dp;
+#pragma unroll
+        for (int dd = 0; dd < D; ++dd) {
+          T qd = Ai[dd][0] * vel[0], f0 = Ai[dd][0] * t[i][1];
+#pragma unroll
+          for (int k = 1; k < D; ++k) {
+            qd = fma(Ai[dd][k], vel[k], qd);
+            f0 = fma(Ai[dd][k], t[i][1 + k], f0);
+          }
+          const T wd = fma(-qd, t[i][0], f0);
+          F[dd][0] = f0;
+#pragma unroll
+          for (int k = 0; k < D; ++k) F[dd][1 + k] = fma(vel[k], wd, fma(qd, t[i][1 + k], Ai[dd][k] * dp));
+          F[dd][NV - 1] = fma(H, wd, qd * de);
+        }
+      }
+      if (d.rot) {  // rotating frame: the flux is F - U v_r^T
+        const T* vr = d.vrq + (e * NQ + q) * D;
+#pragma unroll
+        for (int dd = 0; dd < D; ++dd) {
+          T vd = Ai[dd][0] * vr[0];
+#pragma unroll
+          for (int k = 1; k < D; ++k) vd = fma(Ai[dd][k], vr[k], vd);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) F[dd][v] = fma(-vd, t[i][v], F[dd][v]);
+        }
+      }
+#pragma unroll
+      for (int dd = 0; dd < D; ++dd)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) sF[((q * D + dd) * NV + v) * ET + lane] = F[dd][v];
+    }
+    __syncthreads();
+  }
+  // phase 2: variable w of this lane's element
+  if constexpr (L::AHEAD) cp_async_wait_all();  // a thread reads its own copies only
+  T acc[NB];
+#pragma unroll
+  for (int i = 0; i < NB; ++i) acc[i] = T(0);
+#pragma unroll
+  for (int k = 0; k < NF; ++k) {
+    const int fs = slots[k];
+    T r[GS], x[NFQ];
+    if constexpr (L::AHEAD) {
+#pragma unroll
+      for (int h = 0; h < L::GV; ++h) {
+        T y[VECW<T>];
+        load_row<T, VECW<T>>(sG + ((k * L::GV + h) * L::NT + threadIdx.x) * VECW<T>, y);
+#pragma unroll
+        for (int i = 0; i < VECW<T>; ++i) r[h * VECW<T> + i] = y[i];
+      }
+    } else {
+      const T* g = G + ((int64_t)slot_face<O>(fs) * NV + w) * GS;
+      if constexpr (PADG) {
+        load_row<T, GS, true>(g, r);
+      } else {
+#pragma unroll
+        for (int q = 0; q < NFQ; ++q) r[q] = __ldg(g + q);
+      }
+    }
+    face_fluxes<T, D, P, GS>(r, fs, x);
+    if constexpr (D == 3 && P == 1) {
+      // the collapsed face rule is not symmetric: the table of the side's vertex permutation
+      const T* tb = d.BfP + ((k * NPERM + slot_perm(fs)) * NFQ) * PADV<T, NB>;
+#pragma unroll
+      for (int q = 0; q < NFQ; ++q) {
+        T row[PADV<T, NB>];
+        load_row<T, PADV<T, NB>, true>(tb + q * PADV<T, NB>, row);
+#pragma unroll
+        for (int i = 0; i < NB; ++i) acc[i] = fma(row[i], x[q], acc[i]);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < NFQ; ++q)
+#pragma unroll
+        for (int i = 0; i < NB; ++i) acc[i] = fma(tab[X::BF + (k * NFQ + q) * NB + i], x[q], acc[i]);
+    }
+  }
+  // the lift carries 1/sqrt|det|; the volume term sqrt|det| (flux) or nothing (the factors of the
+  // trace and the test cancel in the derivative)
+  const T ls = MODE == ELEM_FLUX ? isd * isd : isd;
+#pragma unroll
+  for (int i = 0; i < NB; ++i) acc[i] *= ls;
+  if constexpr (P > 0) {
+#pragma unroll
+    for (int dd = 0; dd < D; ++dd) {
+      T m[NB1 > 0 ? NB1 : 1];
+#pragma unroll
+      for (int k = 0; k < NB1; ++k) m[k] = T(0);
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        const T f = sF[((q * D + dd) * NV + w) * ET + lane];
+#pragma unroll
+        for (int k = 0; k < NB1; ++k) m[k] = fma(tab[X::WM + q * NB1 + k], f, m[k]);
+      }
+      combine_modes<T, D, P, 1>(tab + X::CM + dd * NB * NB1, m, acc);
+    }
+  }
+  T sc = oscale ? (T)*oscale : T(1);
+  if (escale) sc *= escale[e];
+  if (d.rot && w >= 1 && w <= D) {  // the frame's source, on the coefficients of u (R) or du (J v)
+    const T so = MODE == ELEM_FLUX ? isd : T(1);
+    const T* ra = rows + el * RS;
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      T m[D];
+#pragma unroll
+      for (int k = 0; k < D; ++k) m[k] = ra[(1 + k) * NB + i];
+      acc[i] += rot_source<T, D>(d.om, m, w - 1) * so;
+    }
+  }
+  if (d.rot) __syncthreads();  // the rows have been read before they are overwritten
+  if constexpr (MODE == ELEM_FLUX) sc *= ge[O::SD];
+#pragma unroll
+  for (int i = 0; i < NB; ++i) rows[lane * RS + w * NB + i] = acc[i] * sc;
+  __syncthreads();
+  for (int i = threadIdx.x; i < ne * NVB; i += L::NT) out[e0 * NVB + i] = rows[i / NVB * RS + i % NVB];
+}
+
+template <class T, int D, int P, int MODE, bool PADG>
+static void elem_op_launch(const DGData<T>& d, const T* u, const T* du, const T* pts, const T* G, T* out,
+                           const T* escale, const int* skip, const double* oscale, cudaStream_t st) {
+  using L = ElemTile<T, D, P, MODE>;
+  elem_op_kernel<T, D, P, MODE, PADG><<<(unsigned)((d.E + L::ET - 1) / L::ET), L::NT, L::BYTES, st>>>(
+      d, u, du, pts, G, out, escale, skip, oscale);
+}
+
+template <class T, int D, int P>
+cudaError_t dg_op_p(const DGData<T>& d, const T* u, const T* du, T* out, T* G, const T* escale, const int* skip,
+                    const double* oscale, cudaStream_t st, const cudaEvent_t* ev, bool tight) {
+  using O = Ord<D, P>;
+  const int64_t nfp = d.F * O::NFQ;
+  const unsigned nb = (unsigned)((nfp + 255) / 256);
+  if (tight) {
+    if constexpr (std::is_same<T, double>::value) {
+      if (du) return cudaErrorInvalidValue;
+      if (nfp > 0) face_kernel<T, D, P, false, false><<<nb, 256, 0, st>>>(d, u, du, G, skip);
+      elem_op_launch<T, D, P, ELEM_FLUX, false>(d, u, nullptr, nullptr, G, out, escale, skip, oscale, st);
+      return cudaGetLastError();
+    }
+    return cudaErrorInvalidValue;
+  }
+  if (ev) cudaEventRecord(ev[0], st);
+  if (nfp > 0) {
+    if (du) face_kernel<T, D, P, true, true><<<nb, 256, 0, st>>>(d, u, du, G, skip);
+    else face_kernel<T, D, P, false, true><<<nb, 256, 0, st>>>(d, u, du, G, skip);
+  }
+  if (ev) cudaEventRecord(ev[1], st);
+  if (du) elem_op_launch<T, D, P, ELEM_TANGENT, true>(d, u, du, nullptr, G, out, escale, skip, oscale, st);
+  else elem_op_launch<T, D, P, ELEM_FLUX, true>(d, u, nullptr, nullptr, G, out, escale, skip, oscale, st);
+  if (ev) cudaEventRecord(ev[2], st);
+  return cudaGetLastError();
+}
+
+// Uploads c_tab and raises the shared-memory limits of the element kernels (current device).
+template <class T, int D, int P>
+cudaError_t upload_tables_p(const double* Bv, const double* Dv, const double* Wv, const double* Bf, cudaStream_t st) {
+  using O = Ord<D, P>;
+  using X = TabLayout<D, P>;
+  constexpr int NB = O::NB, NQ = O::NQ, NB1 = X::NB1;
+  T tab[X::N];
+  for (int i = 0; i < NQ * NB; ++i) tab[X::BV + i] = (T)Bv[i];
+  for (int q = 0; q < NQ; ++q)
+    for (int k = 0; k < NB1; ++k) tab[X::WM + q * NB1 + k] = (T)(Wv[q] * Bv[q * NB + k]);
+  for (int dd = 0; dd < D; ++dd)
+    for (int i = 0; i < NB; ++i)
+      for (int k = 0; k < NB1; ++k) {
+        double a = 0;  // sum_q w_q d phi_i / d xi_d phi_k (Dv carries w_q)
+        for (int q = 0; q < NQ; ++q) a += Dv[(dd * NQ + q) * NB + i] * Bv[q * NB + k];
+        tab[X::CM + (dd * NB + i) * NB1 + k] = (T)a;
+      }
+  for (int f = 0; f < O::NF; ++f)
+    for (int i = 0; i < O::NFQ * NB; ++i) tab[X::BF + f * O::NFQ * NB + i] = (T)Bf[(f * O::NPERM) * O::NFQ * NB + i];
+  cudaError_t e = cudaMemcpyToSymbolAsync(c_tab<T, D, P>, tab, sizeof(tab), 0, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  auto allow = [&](auto kernel, size_t bytes) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  };
+  allow(elem_op_kernel<T, D, P, ELEM_FLUX, true>, ElemTile<T, D, P, ELEM_FLUX>::BYTES);
+  allow(elem_op_kernel<T, D, P, ELEM_TANGENT, true>, ElemTile<T, D, P, ELEM_TANGENT>::BYTES);
+  allow(elem_op_kernel<T, D, P, ELEM_STORED, true>, ElemTile<T, D, P, ELEM_STORED>::BYTES);
+  if constexpr (std::is_same<T, double>::value)
+    allow(elem_op_kernel<T, D, P, ELEM_FLUX, false>, ElemTile<T, D, P, ELEM_FLUX>::BYTES);
+  return e;
 }
 
 // U[v] = isd sum_j b[j] ue[v][j]: the trace of an element's coefficients at a point, table row b
@@ -709,56 +722,36 @@ PCEXP_DEV void face_flux_vjp(const DGData<T>& d, int eR, const T (&L)[D + 2], co
   }
 }
 
-// ------------------------------------------------------- point Jacobians (linearisation)
-// The exact Jacobian of the scheme (Eq. jac1, jac2) is assembled point by point: the
-// volume flux Jacobians dF_d/dU and the Riemann-flux Jacobians dF~/dU_L, dF~/dU_R are
-// evaluated exactly, the former on Jet<T, D+2> numbers seeded with unit directions, the latter
-// by reverse sweeps (the paper obtains the Riemann-flux Jacobians by AD as well).  Every J v
-// of a PCEXP step is taken at u_n, so the Jacobians are built once per step and each
-// of the 2m+1 products reduces to traces, small mat-vecs and the test/lift contractions.
+// ------------------------------------------------------- linearisation
+// The exact Jacobian of the scheme (Eq. jac1, jac2) point by point.  Faces: the Riemann-flux
+// Jacobians dF~/dU_L, dF~/dU_R, evaluated exactly by reverse sweeps (the paper obtains them by AD as
+// well).  Volume: the velocity and the total enthalpy, from which the derivative of the Euler flux
+// along any direction costs fewer operations than a product with its stored D nv x nv Jacobian
+// (51 against 75 FMAs per point on tetrahedra), and 4 values per point instead of D nv^2.
+// Every J v of a PCEXP step is taken at u_n, so both are built once per step.
+//   pts [nq][E][4]: velocity (D), H = (E + p) / rho; in 2D the fourth entry is unused
 template <class T, int D, int P>
 __global__ void __launch_bounds__(256) linearize_vol_kernel(DGData<T> d, const T* __restrict__ u,
-                                                            T* __restrict__ Avol) {
+                                                            T* __restrict__ pts) {
   using O = Ord<D, P>;
   constexpr int NB = O::NB, NQ = O::NQ, NV = O::NV, GEO = O::GEO;
-  using J = Jet<T, NV>;
-  const int64_t n = d.E * NQ;
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n) return;
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // points of an element together
+  if (idx >= d.E * NQ) return;
   const int64_t e = idx / NQ;
   const int q = (int)(idx - e * NQ);
-  const T* ge = d.geo + GEO * e;
-  const T isd = ge[O::ISD];
-  J U[NV];
+  T U[NV];
+  point_trace<T, D, P>(d.Bv + q * NB, u + e * NV * NB, d.geo[GEO * e + O::ISD], U);
+  const T ir = T(1) / U[0];
+  T x[4] = {T(0), T(0), T(0), T(0)}, k2 = T(0);
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    T a = 0;
-#pragma unroll
-    for (int j = 0; j < NB; ++j) a += __ldg(d.Bv + q * NB + j) * u[e * NV * NB + v * NB + j];
-    U[v].v = a * isd;
-#pragma unroll
-    for (int c = 0; c < NV; ++c) U[v].d[c] = (v == c) ? T(1) : T(0);
+  for (int k = 0; k < D; ++k) {
+    x[k] = U[1 + k] * ir;
+    k2 = fma(T(0.5) * x[k], x[k], k2);
   }
-  J F[D][NV];
-  euler_flux<D, J, T>(U, d.fs.gamma, F);
-  if (d.rot) {
-    const T* vr = d.vrq + idx * D;
+  x[D] = (U[NV - 1] + (d.fs.gamma - T(1)) * (U[NV - 1] - k2 * U[0])) * ir;
+  T* o = pts + ((int64_t)q * d.E + e) * 4;
 #pragma unroll
-    for (int k = 0; k < D; ++k)
-#pragma unroll
-      for (int v = 0; v < NV; ++v) F[k][v] = F[k][v] - U[v] * vr[k];
-  }
-#pragma unroll
-  for (int dd = 0; dd < D; ++dd)
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-#pragma unroll
-      for (int c = 0; c < NV; ++c) {
-        T a = ge[dd * D] * F[0][v].d[c];
-#pragma unroll
-        for (int k = 1; k < D; ++k) a += ge[dd * D + k] * F[k][v].d[c];
-        Avol[(int64_t)(dd * NV * NV + v * NV + c) * n + idx] = a;
-      }
+  for (int k = 0; k < 4; ++k) o[k] = x[k];
 }
 
 // The face blocks come row by row from reverse sweeps of the Roe flux: with the adjoint e_v one
@@ -886,7 +879,7 @@ __global__ void __launch_bounds__(256) face_apply_kernel(DGData<T> d, const T* _
   T tL[NV], tR[NV];
   trace(eL, fL, 0, tL);
   if (eR >= 0) trace(eR, fR, pR, tR);
-  T* g = G + idx * NV;
+  T g[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     T a = 0;
@@ -898,151 +891,28 @@ __global__ void __launch_bounds__(256) face_apply_kernel(DGData<T> d, const T* _
     }
     g[v] = a;
   }
+  store_face_flux<T, D, P, true>(G, f, q, g);
 }
 
 template <class T, int D, int P>
-__global__ void __launch_bounds__(256) elem_apply_kernel(DGData<T> d, const T* __restrict__ Avol,
-                                                         const T* __restrict__ dv, const T* __restrict__ G,
-                                                         T* __restrict__ out, const T* __restrict__ escale,
-                                                         const int* __restrict__ skip,
-                                                         const double* __restrict__ oscale) {
-  using O = Ord<D, P>;
-  constexpr int NB = O::NB, NQ = O::NQ, ET = O::ET, NVB = O::NVB, NV = O::NV, GEO = O::GEO, DV = D * NV;
-  constexpr int NN = NV * NV;
-  constexpr int NPRE = D == 2 ? O::NJV : NN;  // point-Jacobian entries loaded before the staging
-  constexpr bool SM = O::SMEM_BF;
-  __shared__ T sBv[NQ * NB];
-  __shared__ T sDv[D * NQ * NB];
-  __shared__ T sBf[SM ? O::NBF : 1];
-  __shared__ T sdu[ET * NVB];
-  __shared__ T sF[ET * NQ * DV];
-  __shared__ T ssd[ET];
-  static_assert(ET * NQ <= 256, "one volume point per thread");
-  if (skip && *skip) return;
-  const int64_t e0 = (int64_t)blockIdx.x * ET;
-  const int ne = (int)((d.E - e0) < ET ? (d.E - e0) : ET);
-  const int64_t n = d.E * NQ;
-  // issue this thread's point-Jacobian loads first, so they are in flight while the
-  // block stages its tile of dv in shared memory
-  const int el1 = threadIdx.x / NQ, q1 = threadIdx.x - (threadIdx.x / NQ) * NQ;
-  const bool has_pt = threadIdx.x < ne * NQ;
-  const int64_t pidx = (e0 + el1) * NQ + q1;
-  T A[NPRE];
-#pragma unroll
-  for (int k = 0; k < NPRE; ++k) A[k] = has_pt ? Avol[(int64_t)k * n + pidx] : T(0);
-  for (int i = threadIdx.x; i < NQ * NB; i += blockDim.x) sBv[i] = d.Bv[i];
-  for (int i = threadIdx.x; i < D * NQ * NB; i += blockDim.x) sDv[i] = d.Dv[i];
-  if constexpr (SM)
-    for (int i = threadIdx.x; i < O::NBF; i += blockDim.x) sBf[i] = d.Bf[i];
-  for (int i = threadIdx.x; i < ne * NVB; i += blockDim.x) sdu[i] = dv[e0 * NVB + i];
-  for (int i = threadIdx.x; i < ne; i += blockDim.x) ssd[i] = d.geo[(e0 + i) * GEO + O::ISD];
-  __syncthreads();
-  const T osc = oscale ? (T)*oscale : T(1);
-  // phase 1: trace of dv at this thread's volume point, times the mapped flux Jacobians
-  if (has_pt) {
-    T t[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      T a = 0;
-#pragma unroll
-      for (int j = 0; j < NB; ++j) a += sBv[q1 * NB + j] * sdu[el1 * NVB + v * NB + j];
-      t[v] = a;
-    }
-    T* fo = sF + (el1 * NQ + q1) * DV;
-#pragma unroll
-    for (int dd = 0; dd < D; ++dd)
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        T a = 0;
-#pragma unroll
-        for (int c = 0; c < NV; ++c) {
-          const int k = dd * NN + v * NV + c;
-          const T akc = k < NPRE ? A[k < NPRE ? k : 0] : Avol[(int64_t)k * n + pidx];
-          a += akc * t[c];
-        }
-        fo[dd * NV + v] = a;
-      }
-  }
-  __syncthreads();
-  const T* Bf = SM ? sBf : d.Bf;
-  // phase 2: test against grad phi (the sqrt(det) factors cancel), lift the face terms
-  for (int it = threadIdx.x; it < ne * NVB; it += blockDim.x) {
-    const int el = it / NVB, r = it - el * NVB;
-    const int v = r / NB, i = r - v * NB;
-    T acc = 0;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q)
-#pragma unroll
-      for (int dd = 0; dd < D; ++dd) acc += sDv[(dd * NQ + q) * NB + i] * sF[(el * NQ + q) * DV + dd * NV + v];
-    const int64_t e = e0 + el;
-    const T lift = lift_faces<T, D, P, SM>(d, Bf, G, e, v, i);
-    acc = acc + lift * ssd[el];
-    if (d.rot && v >= 1 && v <= D) {  // the rotating frame's source on the coefficients of dv
-      T m[D];
-#pragma unroll
-      for (int k = 0; k < D; ++k) m[k] = sdu[el * NVB + (1 + k) * NB + i];
-      acc += rot_source<T, D>(d.om, m, v - 1);
-    }
-    acc *= osc;
-    if (escale) acc *= escale[e];
-    out[e0 * NVB + it] = acc;
-  }
-}
-
-template <class T, int D, int P>
-cudaError_t linearize_p(const DGData<T>& d, const T* u, LinData<T> lin, bool faces_only, cudaStream_t st) {
+cudaError_t linearize_p(const DGData<T>& d, const T* u, LinData<T> lin, cudaStream_t st) {
   using O = Ord<D, P>;
   const int64_t nv = d.E * O::NQ, nf = d.F * O::NFQ;
-  if (!faces_only) linearize_vol_kernel<T, D, P><<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(d, u, lin.Avol);
+  linearize_vol_kernel<T, D, P><<<(unsigned)((nv + 255) / 256), 256, 0, st>>>(d, u, lin.pts);
   if (nf > 0) linearize_face_kernel<T, D, P><<<(unsigned)((nf + 127) / 128), 128, 0, st>>>(d, u, lin.Bface);
   return cudaGetLastError();
 }
 
-// J v from the face point Jacobians and either the volume point Jacobians (u_elem null)
-// or the volume flux tangents recomputed at u_elem (the elements then read u and dv
-// instead of D nv^2 values per volume point).
-//
-// face_tan: the face part recomputes the Riemann-flux tangent at every face point from the
-// traces of u_elem and dv (face_kernel<TAN>) instead of applying the stored face point
-// Jacobians (it then reads u_n and dv instead of 2 nv^2 values per face point).
+// J v from the face point Jacobians and the stored volume points.
 template <class T, int D, int P>
-cudaError_t jac_apply_p(const DGData<T>& d, LinData<T> lin, const T* u_elem, const T* dv, T* out, T* G,
-                        const T* escale, const int* skip, const double* oscale, cudaStream_t st,
-                        const cudaEvent_t* ev, bool face_tan) {
+cudaError_t jac_apply_p(const DGData<T>& d, LinData<T> lin, const T* dv, T* out, T* G, const T* escale,
+                        const int* skip, const double* oscale, cudaStream_t st, const cudaEvent_t* ev) {
   using O = Ord<D, P>;
   const int64_t nf = d.F * O::NFQ;
   if (ev) cudaEventRecord(ev[0], st);
-  if (nf > 0) {
-    if (face_tan && u_elem)
-      face_kernel<T, D, P, true><<<(unsigned)((nf + 255) / 256), 256, 0, st>>>(d, u_elem, dv, G, skip);
-    else
-      face_apply_kernel<T, D, P><<<(unsigned)((nf + 255) / 256), 256, 0, st>>>(d, lin.Bface, dv, G, skip);
-  }
+  if (nf > 0) face_apply_kernel<T, D, P><<<(unsigned)((nf + 255) / 256), 256, 0, st>>>(d, lin.Bface, dv, G, skip);
   if (ev) cudaEventRecord(ev[1], st);
-  const int64_t eb = (d.E + O::ET - 1) / O::ET;
-  if (u_elem) {
-    if constexpr (std::is_same<T, float>::value && D == 3) {
-      if (d.rot) {  // the frame terms live in the tile kernel
-        elem_kernel<T, D, P, true><<<(unsigned)eb, 256, 0, st>>>(d, u_elem, dv, G, out, escale, skip, oscale);
-      } else if (d.E > 0) {
-        // persistent: two blocks per SM (two 42 KB stages each), tiles of 32 elements
-        static int nsm = 0;
-        if (!nsm) {
-          int dev = 0;
-          cudaGetDevice(&dev);
-          if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1) nsm = 152;
-        }
-        const int64_t ntiles = (d.E + 31) / 32;
-        const int64_t grid = ntiles < 2 * (int64_t)nsm ? ntiles : 2 * (int64_t)nsm;
-        elem_tan_pipe_kernel<D, P><<<(unsigned)grid, 32 * TanPipe<D, P>::WARPS, TanPipe<D, P>::BYTES, st>>>(
-            d, u_elem, dv, G, out, escale, skip, oscale, ntiles);
-      }
-    } else {
-      elem_kernel<T, D, P, true><<<(unsigned)eb, 256, 0, st>>>(d, u_elem, dv, G, out, escale, skip, oscale);
-    }
-  } else {
-    elem_apply_kernel<T, D, P><<<(unsigned)eb, 256, 0, st>>>(d, lin.Avol, dv, G, out, escale, skip, oscale);
-  }
+  elem_op_launch<T, D, P, ELEM_STORED, true>(d, nullptr, dv, lin.pts, G, out, escale, skip, oscale, st);
   if (ev) cudaEventRecord(ev[2], st);
   return cudaGetLastError();
 }
@@ -1053,7 +923,7 @@ cudaError_t jac_apply_p(const DGData<T>& d, LinData<T> lin, const T* u_elem, con
 // adjoint of the lifted face flux at every face point,
 //   Gbar = -(1/sd_L) sum_i Bf_L[i] w~_L[i] + (1/sd_R) sum_i Bf_R[i] w~_R[i],
 // and stores B_L^T Gbar and B_R^T Gbar; the element kernel applies the transposed
-// volume Jacobians to the transposed test of w~ and gathers the transposed traces
+// flux derivatives to the transposed test of w~ and gathers the transposed traces
 // of its faces.  Deterministic (no atomics).
 template <class T, int D, int P>
 __global__ void __launch_bounds__(256) face_adjoint_kernel(DGData<T> d, const T* __restrict__ Bface,
@@ -1130,12 +1000,12 @@ PCEXP_DEV T gather_faces_T(const DGData<T>& d, const T* Bf, const T* __restrict_
 }
 
 template <class T, int D, int P>
-__global__ void __launch_bounds__(256) elem_adjoint_kernel(DGData<T> d, const T* __restrict__ Avol,
+__global__ void __launch_bounds__(256) elem_adjoint_kernel(DGData<T> d, const T* __restrict__ pts,
                                                            const T* __restrict__ w, const T* __restrict__ GT,
                                                            T* __restrict__ out, const T* __restrict__ escale,
                                                            T osc) {
   using O = Ord<D, P>;
-  constexpr int NB = O::NB, NQ = O::NQ, ET = O::ET, NVB = O::NVB, NV = O::NV, NN = NV * NV;
+  constexpr int NB = O::NB, NQ = O::NQ, ET = O::ET, NVB = O::NVB, NV = O::NV;
   constexpr bool SM = O::SMEM_BF;
   __shared__ T sBv[NQ * NB];
   __shared__ T sDv[D * NQ * NB];
@@ -1145,7 +1015,6 @@ __global__ void __launch_bounds__(256) elem_adjoint_kernel(DGData<T> d, const T*
   static_assert(ET * NQ <= 256, "one volume point per thread");
   const int64_t e0 = (int64_t)blockIdx.x * ET;
   const int ne = (int)((d.E - e0) < ET ? (d.E - e0) : ET);
-  const int64_t n = d.E * NQ;
   for (int i = threadIdx.x; i < NQ * NB; i += blockDim.x) sBv[i] = d.Bv[i];
   for (int i = threadIdx.x; i < D * NQ * NB; i += blockDim.x) sDv[i] = d.Dv[i];
   if constexpr (SM)
@@ -1153,11 +1022,11 @@ __global__ void __launch_bounds__(256) elem_adjoint_kernel(DGData<T> d, const T*
   for (int i = threadIdx.x; i < ne * NVB; i += blockDim.x)
     sw[i] = w[e0 * NVB + i] * osc * (escale ? escale[e0 + i / NVB] : T(1));
   __syncthreads();
-  // phase 1: transposed test, then transposed volume Jacobians, at this thread's point
+  // phase 1: transposed test, then the transposed flux derivative, at this thread's point
   const int el1 = threadIdx.x / NQ, q1 = threadIdx.x - (threadIdx.x / NQ) * NQ;
   if (threadIdx.x < ne * NQ) {
-    const int64_t pidx = (e0 + el1) * NQ + q1;
-    T fb[D * NV];
+    const int64_t e = e0 + el1;
+    T fb[D][NV];
 #pragma unroll
     for (int dd = 0; dd < D; ++dd)
 #pragma unroll
@@ -1165,17 +1034,50 @@ __global__ void __launch_bounds__(256) elem_adjoint_kernel(DGData<T> d, const T*
         T a = 0;
 #pragma unroll
         for (int i = 0; i < NB; ++i) a += sDv[(dd * NQ + q1) * NB + i] * sw[el1 * NVB + v * NB + i];
-        fb[dd * NV + v] = a;
+        fb[dd][v] = a;
       }
+    T pv[4], Ub[NV], k2 = T(0), dpb = T(0);
+    load_row<T, 4, true>(pts + ((int64_t)q1 * d.E + e) * 4, pv);
+    const T gm = d.fs.gamma - T(1);
 #pragma unroll
-    for (int c = 0; c < NV; ++c) {
-      T a = 0;
+    for (int c = 0; c < NV; ++c) Ub[c] = T(0);
 #pragma unroll
-      for (int dd = 0; dd < D; ++dd)
+    for (int k = 0; k < D; ++k) k2 = fma(T(0.5) * pv[k], pv[k], k2);
+    // transpose of the derivative of elem_op_kernel: w_d = A_d . dm - q_d drho,
+    // dF_d = (A_d . dm, v w_d + q_d dm + A_d dp, H w_d + q_d (dE + dp))
 #pragma unroll
-        for (int v = 0; v < NV; ++v) a += Avol[(int64_t)(dd * NN + v * NV + c) * n + pidx] * fb[dd * NV + v];
-      sU[(el1 * NQ + q1) * NV + c] = a;
+    for (int dd = 0; dd < D; ++dd) {
+      const T* A = d.geo + O::GEO * e + dd * D;
+      T qd = A[0] * pv[0], wb = fb[dd][NV - 1] * pv[D], pb = T(0);
+#pragma unroll
+      for (int k = 1; k < D; ++k) qd = fma(A[k], pv[k], qd);
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        wb = fma(fb[dd][1 + k], pv[k], wb);
+        pb = fma(fb[dd][1 + k], A[k], pb);
+      }
+      const T f0b = fb[dd][0] + wb, eb = fb[dd][NV - 1] * qd;
+      dpb += pb + eb;
+      Ub[NV - 1] += eb;
+      Ub[0] = fma(-qd, wb, Ub[0]);
+#pragma unroll
+      for (int k = 0; k < D; ++k) Ub[1 + k] = fma(A[k], f0b, fma(fb[dd][1 + k], qd, Ub[1 + k]));
+      if (d.rot) {  // rotating frame: the flux is F - U v_r^T
+        const T* vr = d.vrq + (e * NQ + q1) * D;
+        T vd = A[0] * vr[0];
+#pragma unroll
+        for (int k = 1; k < D; ++k) vd = fma(A[k], vr[k], vd);
+#pragma unroll
+        for (int c = 0; c < NV; ++c) Ub[c] = fma(-vd, fb[dd][c], Ub[c]);
+      }
     }
+    dpb *= gm;
+    Ub[0] = fma(k2, dpb, Ub[0]);
+    Ub[NV - 1] += dpb;
+#pragma unroll
+    for (int k = 0; k < D; ++k) Ub[1 + k] = fma(-pv[k], dpb, Ub[1 + k]);
+#pragma unroll
+    for (int c = 0; c < NV; ++c) sU[(el1 * NQ + q1) * NV + c] = Ub[c];
   }
   __syncthreads();
   const T* Bf = SM ? sBf : d.Bf;
@@ -1204,7 +1106,7 @@ cudaError_t jac_adjoint_p(const DGData<T>& d, LinData<T> lin, const T* w, T* out
   const int64_t nf = d.F * O::NFQ;
   if (nf > 0) face_adjoint_kernel<T, D, P><<<(unsigned)((nf + 255) / 256), 256, 0, st>>>(d, lin.Bface, w, GT, escale, osc);
   const int64_t eb = (d.E + O::ET - 1) / O::ET;
-  elem_adjoint_kernel<T, D, P><<<(unsigned)eb, 256, 0, st>>>(d, lin.Avol, w, GT, out, escale, osc);
+  elem_adjoint_kernel<T, D, P><<<(unsigned)eb, 256, 0, st>>>(d, lin.pts, w, GT, out, escale, osc);
   return cudaGetLastError();
 }
 
@@ -1913,22 +1815,33 @@ template <int D> constexpr int PMAX = D == 2 ? 3 : 2;
 
 template <class T, int D>
 cudaError_t launch_dg_operator_d(const DGData<T>& d, const T* u, const T* du, T* out, T* G, const T* escale,
-                                 const int* skip, cudaStream_t st, const cudaEvent_t* ev, const double* oscale) {
-  PCEXP_PSWITCH(D, (dg_op_p<T, D, P_>(d, u, du, out, G, escale, skip, oscale, st, ev)))
+                                 const int* skip, cudaStream_t st, const cudaEvent_t* ev, const double* oscale,
+                                 bool tight) {
+  PCEXP_PSWITCH(D, (dg_op_p<T, D, P_>(d, u, du, out, G, escale, skip, oscale, st, ev, tight)))
 }
 template <class T, int D>
-cudaError_t launch_linearize_d(const DGData<T>& d, const T* u, LinData<T> lin, bool faces_only, cudaStream_t st) {
-  PCEXP_PSWITCH(D, (linearize_p<T, D, P_>(d, u, lin, faces_only, st)))
+cudaError_t launch_linearize_d(const DGData<T>& d, const T* u, LinData<T> lin, cudaStream_t st) {
+  PCEXP_PSWITCH(D, (linearize_p<T, D, P_>(d, u, lin, st)))
 }
 template <class T, int D>
-cudaError_t launch_jac_apply_d(const DGData<T>& d, LinData<T> lin, const T* u_elem, const T* dv, T* out, T* G,
-                               const T* escale, const int* skip, const double* oscale, cudaStream_t st,
-                               const cudaEvent_t* ev, bool face_tan) {
-  PCEXP_PSWITCH(D, (jac_apply_p<T, D, P_>(d, lin, u_elem, dv, out, G, escale, skip, oscale, st, ev, face_tan)))
+cudaError_t launch_jac_apply_d(const DGData<T>& d, LinData<T> lin, const T* dv, T* out, T* G, const T* escale,
+                               const int* skip, const double* oscale, cudaStream_t st, const cudaEvent_t* ev) {
+  PCEXP_PSWITCH(D, (jac_apply_p<T, D, P_>(d, lin, dv, out, G, escale, skip, oscale, st, ev)))
 }
-template <int D>
-cudaError_t launch_tan_tables_d(const DGData<float>& d, cudaStream_t st) {
-  PCEXP_PSWITCH(D, (tan_tables_p<D, P_>(d, st)))
+template <class T, int D>
+cudaError_t upload_tables_d(const DGData<T>& d, const double* Bv, const double* Dv, const double* Wv, const double* Bf,
+                            cudaStream_t st) {
+  PCEXP_PSWITCH(D, (upload_tables_p<T, D, P_>(Bv, Dv, Wv, Bf, st)))
+}
+template <class T, int D>
+int64_t face_flux_size_d(const DGData<T>& d) {
+  const int nv = D + 2;
+  switch (d.p) {
+    case 0: return d.F * nv * GSTRIDE<T, D, 0>;
+    case 1: return d.F * nv * GSTRIDE<T, D, 1>;
+    case 2: return d.F * nv * GSTRIDE<T, D, 2>;
+    default: return d.F * nv * GSTRIDE<T, D, (PMAX<D> >= 3 ? 3 : 2)>;
+  }
 }
 template <class T, int D>
 cudaError_t launch_jac_adjoint_d(const DGData<T>& d, LinData<T> lin, const T* w, T* out, T* GT, const T* escale,
@@ -2009,11 +1922,14 @@ cudaError_t launch_local_dt_d(const DGData<T>& d, const T* u, const double* cfl_
 
 #define PCEXP_INST_D(T, D)                                                                                         \
   template cudaError_t launch_dg_operator_d<T, D>(const DGData<T>&, const T*, const T*, T*, T*, const T*,           \
-                                                  const int*, cudaStream_t, const cudaEvent_t*, const double*);    \
-  template cudaError_t launch_linearize_d<T, D>(const DGData<T>&, const T*, LinData<T>, bool, cudaStream_t);       \
-  template cudaError_t launch_jac_apply_d<T, D>(const DGData<T>&, LinData<T>, const T*, const T*, T*, T*,          \
-                                                const T*, const int*, const double*, cudaStream_t,                 \
-                                                const cudaEvent_t*, bool);                                         \
+                                                  const int*, cudaStream_t, const cudaEvent_t*, const double*,     \
+                                                  bool);                                                           \
+  template cudaError_t launch_linearize_d<T, D>(const DGData<T>&, const T*, LinData<T>, cudaStream_t);             \
+  template cudaError_t launch_jac_apply_d<T, D>(const DGData<T>&, LinData<T>, const T*, T*, T*, const T*,          \
+                                                const int*, const double*, cudaStream_t, const cudaEvent_t*);      \
+  template cudaError_t upload_tables_d<T, D>(const DGData<T>&, const double*, const double*, const double*,        \
+                                             const double*, cudaStream_t);                                         \
+  template int64_t face_flux_size_d<T, D>(const DGData<T>&);                                                       \
   template cudaError_t launch_jac_adjoint_d<T, D>(const DGData<T>&, LinData<T>, const T*, T*, T*, const T*, T,     \
                                                   cudaStream_t);                                                   \
   template cudaError_t launch_jvp_state_adjoint_d<T, D>(const DGData<T>&, const T*, const T*, const T*, T*, T*,    \

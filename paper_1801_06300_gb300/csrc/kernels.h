@@ -95,9 +95,8 @@ struct DGData {
   int dim;
 };
 
-// Point Jacobians of the DG operator at a linearisation state u, NV = D + 2.
-//   Avol [D NV NV][E*nq]:  k = d'*NV*NV + v*NV + c: sum_d (A^-1)_{d'd} dF_d[v]/dU[c] at volume points
-//                          (structure of arrays: entry k of every point is contiguous)
+// The DG operator's linearisation at a state u, NV = D + 2.
+//   pts [nq][E][4]:  velocity (D) and total enthalpy H at the volume points
 //   Bface, NJF = 2 NV NV entries per face point: k = s*NV*NV + v*NV + c: |f| w_q / sqrt(det_s)
 //                          dF~[v]/dU_s[c], s = L (0), R (1), the ghost-state chain rule folded into
 //                          s = L on boundary faces; in 16-byte chunks of VEC = 16 / sizeof(T)
@@ -114,7 +113,7 @@ __host__ __device__ __forceinline__ int64_t bface_at(int k, int64_t idx, int64_t
 
 template <class T>
 struct LinData {
-  T* Avol;
+  T* pts;
   T* Bface;
 };
 
@@ -132,15 +131,18 @@ struct ThetaSums {
 // ---- DG operator (dg_kernels.cuh, instantiated per dimension in dg2d.cu / dg3d.cu)
 template <class T, int D>
 cudaError_t launch_dg_operator_d(const DGData<T>& d, const T* u, const T* du, T* out, T* G, const T* escale,
-                                 const int* skip, cudaStream_t st, const cudaEvent_t* ev, const double* oscale);
+                                 const int* skip, cudaStream_t st, const cudaEvent_t* ev, const double* oscale,
+                                 bool tight);
 template <class T, int D>
-cudaError_t launch_linearize_d(const DGData<T>& d, const T* u, LinData<T> lin, bool faces_only, cudaStream_t st);
+cudaError_t launch_linearize_d(const DGData<T>& d, const T* u, LinData<T> lin, cudaStream_t st);
 template <class T, int D>
-cudaError_t launch_jac_apply_d(const DGData<T>& d, LinData<T> lin, const T* u_elem, const T* dv, T* out, T* G,
-                               const T* escale, const int* skip, const double* oscale, cudaStream_t st,
-                               const cudaEvent_t* ev, bool face_tan);
-template <int D>
-cudaError_t launch_tan_tables_d(const DGData<float>& d, cudaStream_t st);
+cudaError_t launch_jac_apply_d(const DGData<T>& d, LinData<T> lin, const T* dv, T* out, T* G, const T* escale,
+                               const int* skip, const double* oscale, cudaStream_t st, const cudaEvent_t* ev);
+template <class T, int D>
+cudaError_t upload_tables_d(const DGData<T>& d, const double* Bv, const double* Dv, const double* Wv, const double* Bf,
+                            cudaStream_t st);
+template <class T, int D>
+int64_t face_flux_size_d(const DGData<T>& d);
 template <class T, int D>
 cudaError_t launch_jac_adjoint_d(const DGData<T>& d, LinData<T> lin, const T* w, T* out, T* GT, const T* escale,
                                  T osc, cudaStream_t st);
@@ -167,43 +169,44 @@ template <class T, int D>
 cudaError_t launch_local_dt_d(const DGData<T>& d, const T* u, const double* cfl_dev, double cfl, T* dte,
                               double* dtmin, double* partials, unsigned* counter, cudaStream_t st);
 
-// out = R(u)  or  out = J(u) du  (du != nullptr); G is face-flux scratch [F][nfq][NV].
+// Entries of the face-flux scratch G of d's mesh and order (records padded to 16-byte vectors).
+template <class T>
+int64_t face_flux_size(const DGData<T>& d) {
+  return d.dim == 3 ? face_flux_size_d<T, 3>(d) : face_flux_size_d<T, 2>(d);
+}
+// Upload the reference tables of the context's (D, p) to the constant-memory copy read by the
+// element kernels (host tables of Setup; synchronises st; the same bytes for every context of that
+// order).
+template <class T>
+cudaError_t upload_tables(const DGData<T>& d, const double* Bv, const double* Dv, const double* Wv, const double* Bf,
+                          cudaStream_t st) {
+  return d.dim == 3 ? upload_tables_d<T, 3>(d, Bv, Dv, Wv, Bf, st) : upload_tables_d<T, 2>(d, Bv, Dv, Wv, Bf, st);
+}
+// out = R(u)  or  out = J(u) du  (du != nullptr); G is face-flux scratch (face_flux_size entries).
 // escale (nullable): per-element output factor.  skip (nullable): device flag, nonzero = no-op.
 // ev (nullable): three events recorded before the face kernel, between the
 // two kernels and after the element kernel.  oscale (nullable, device): one
-// more scalar factor on the output (the Krylov basis scale s_j).
+// more scalar factor on the output (the Krylov basis scale s_j).  tight (FP64 residual only): G
+// holds F * nfq * NV entries, unpadded.
 template <class T>
 cudaError_t launch_dg_operator(const DGData<T>& d, const T* u, const T* du, T* out, T* G,
                                const T* escale, const int* skip, cudaStream_t st,
-                               const cudaEvent_t* ev = nullptr, const double* oscale = nullptr) {
-  return d.dim == 3 ? launch_dg_operator_d<T, 3>(d, u, du, out, G, escale, skip, st, ev, oscale)
-                    : launch_dg_operator_d<T, 2>(d, u, du, out, G, escale, skip, st, ev, oscale);
+                               const cudaEvent_t* ev = nullptr, const double* oscale = nullptr, bool tight = false) {
+  return d.dim == 3 ? launch_dg_operator_d<T, 3>(d, u, du, out, G, escale, skip, st, ev, oscale, tight)
+                    : launch_dg_operator_d<T, 2>(d, u, du, out, G, escale, skip, st, ev, oscale, tight);
 }
-// Evaluate the point Jacobians at u (once per linearisation state): faces and volume, or
-// the face blocks only (faces_only, when the volume part of J v recomputes flux tangents).
+// Linearise at u (once per linearisation state): face blocks and volume points.
 template <class T>
-cudaError_t launch_linearize(const DGData<T>& d, const T* u, LinData<T> lin, cudaStream_t st,
-                             bool faces_only = false) {
-  return d.dim == 3 ? launch_linearize_d<T, 3>(d, u, lin, faces_only, st)
-                    : launch_linearize_d<T, 2>(d, u, lin, faces_only, st);
+cudaError_t launch_linearize(const DGData<T>& d, const T* u, LinData<T> lin, cudaStream_t st) {
+  return d.dim == 3 ? launch_linearize_d<T, 3>(d, u, lin, st) : launch_linearize_d<T, 2>(d, u, lin, st);
 }
-// out = J(u) dv: the face part from the face point Jacobians, or (face_tan, with u_elem) from
-// Riemann-flux tangents recomputed at u_elem; the volume part from the volume point
-// Jacobians (u_elem null) or the flux tangents at u_elem (same ev / escale / skip / oscale
-// conventions as the operator).
+// out = J(u) dv from the linearisation at u (same ev / escale / skip / oscale conventions as the
+// operator).
 template <class T>
 cudaError_t launch_jac_apply(const DGData<T>& d, LinData<T> lin, const T* dv, T* out, T* G, const T* escale,
-                             const int* skip, const double* oscale, cudaStream_t st, const cudaEvent_t* ev,
-                             const T* u_elem = nullptr, bool face_tan = false) {
-  return d.dim == 3 ? launch_jac_apply_d<T, 3>(d, lin, u_elem, dv, out, G, escale, skip, oscale, st, ev, face_tan)
-                    : launch_jac_apply_d<T, 2>(d, lin, u_elem, dv, out, G, escale, skip, oscale, st, ev, face_tan);
-}
-// Upload the reference tables [Bv | Dv] of the context's (D, p) to the constant-memory copy
-// read by the FP32 flux-tangent J v on tetrahedra (device-to-device, on st; same bytes for
-// every context of that order).  Triangles use the tile kernel, which reads the tables from
-// global memory.
-inline cudaError_t launch_tan_tables(const DGData<float>& d, cudaStream_t st) {
-  return d.dim == 3 ? launch_tan_tables_d<3>(d, st) : cudaSuccess;
+                             const int* skip, const double* oscale, cudaStream_t st, const cudaEvent_t* ev) {
+  return d.dim == 3 ? launch_jac_apply_d<T, 3>(d, lin, dv, out, G, escale, skip, oscale, st, ev)
+                    : launch_jac_apply_d<T, 2>(d, lin, dv, out, G, escale, skip, oscale, st, ev);
 }
 // out = (osc * diag(escale) * J(u))^T w from the point Jacobians; GT is scratch [F][nfq][2 NV].
 template <class T>

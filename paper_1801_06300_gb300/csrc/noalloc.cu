@@ -89,7 +89,7 @@ extern "C" int pcexp_residual_noalloc(pcexp_ctx* ctx, const double* U, double* R
   double* G = nullptr;
   r = scratch_address(device, &G);
   if (r != PCEXP_OK) return r;
-  cudaError_t e = launch_dg_operator<double>(d, U, nullptr, R, G, nullptr, nullptr, st);
+  cudaError_t e = launch_dg_operator<double>(d, U, nullptr, R, G, nullptr, nullptr, st, nullptr, nullptr, true);
   if (e != cudaSuccess) {
     const std::string m = std::string("pcexp_residual_noalloc: DG operator launch: ") + cudaGetErrorString(e);
     set_last_error(m.c_str());
