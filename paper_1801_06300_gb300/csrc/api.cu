@@ -199,6 +199,7 @@ DGData<T> dgdata(const pcexp_ctx* c) {
   d.E = c->E;
   d.E_loc = c->grp ? c->n_local : c->E;
   d.F = c->F;
+  d.F_int = c->host.F_interior;
   const double a = c->phys.alpha_deg * M_PI / 180.0;
   const double cinf = std::sqrt(c->phys.gamma * c->phys.p_inf / c->phys.rho_inf);
   d.fs.gamma = (T)c->phys.gamma;
@@ -1198,7 +1199,9 @@ int create_impl(pcexp_ctx* c, const pcexp_mesh* mesh, int p, const pcexp_physics
   PCEXP_TRY(valloc(&c->dte, c->E));
   PCEXP_TRY(valloc(&c->pts, (size_t)4 * c->E * c->nq));
   PCEXP_TRY(valloc(&c->GT, 2 * nv * nfp));
-  PCEXP_TRY(valloc(&c->Bface, 2 * nv * nv * nfp));
+  // FP32 on tetrahedra: 16 values per interior and nv^2 per boundary face point; else 2 nv^2 per point
+  const size_t nip = (size_t)c->host.F_interior * c->nfq;
+  PCEXP_TRY(valloc(&c->Bface, c->fp32 && c->dim == 3 ? 16 * nip + nv * nv * (nfp - nip) : 2 * nv * nv * nfp));
   PCEXP_TRY(dalloc(c, &c->io64a, Kp));
   PCEXP_TRY(dalloc(c, &c->io64b, Kp));
   PCEXP_TRY(dalloc(c, &c->ks, 1));

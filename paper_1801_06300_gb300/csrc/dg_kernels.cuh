@@ -79,6 +79,11 @@ template <class O> PCEXP_DEV int slot_face(int fs) { return fs >> 4; }
 PCEXP_DEV int slot_side(int fs) { return (fs >> 3) & 1; }
 PCEXP_DEV int slot_perm(int fs) { return fs & 7; }
 
+// FP32 on tetrahedra stores a record per interior face point (RoeRecord, 16 values in 16-byte chunks
+// [4][interior points][4]) and an nv x nv block per boundary point after them; the other forms
+// blocks for all points (bface_at).
+template <class T, int D> constexpr bool FACE_RECORDS = std::is_same<T, float>::value && D == 3;
+
 // Table rows and face-flux records are padded to whole 16-byte vectors where they are read with
 // 16-byte loads.
 template <class T> constexpr int VECW = 16 / (int)sizeof(T);
@@ -788,6 +793,18 @@ __global__ void __launch_bounds__(128) linearize_face_kernel(DGData<T> d, const 
   } else {
     ghost_farfield<D, T, T>(L, nr, d.fs, R);
   }
+  if constexpr (FACE_RECORDS<T, D>) {
+    if (eR >= 0) {
+      const RoeRecord<T, D> r = roe_record<D, T>(L, R, d.fs.gamma);
+      const int64_t ni = d.F_int * NFQ;
+      float4* o = reinterpret_cast<float4*>(Bface) + idx;
+      o[0] = make_float4(r.vL[0], r.vL[1], r.vL[2], r.HL);
+      o[ni] = make_float4(r.vR[0], r.vR[1], r.vR[2], r.HR);
+      o[2 * ni] = make_float4(r.rL, r.irL, r.rR, r.irR);
+      o[3 * ni] = make_float4(r.w, r.c, r.i2c, r.dp);
+      return;
+    }
+  }
 #pragma unroll 1
   for (int v = 0; v < NV; ++v) {
     T gb[NV], Lb[NV], Rb[NV];
@@ -799,8 +816,13 @@ __global__ void __launch_bounds__(128) linearize_face_kernel(DGData<T> d, const 
     face_flux_vjp<T, D>(d, eR, L, R, nr, vrn, gb, Lb, Rb);
 #pragma unroll
     for (int c = 0; c < NV; ++c) {
-      Bface[bface_at<T, 2 * NN>(v * NV + c, idx, n)] = wq * isdL * Lb[c];
-      Bface[bface_at<T, 2 * NN>(NN + v * NV + c, idx, n)] = eR >= 0 ? wq * isdR * Rb[c] : T(0);
+      if constexpr (FACE_RECORDS<T, D>) {
+        const int64_t ni = d.F_int * NFQ;  // boundary blocks [nv nv][boundary points] after the records
+        Bface[16 * ni + (v * NV + c) * (n - ni) + idx - ni] = wq * isdL * Lb[c];
+      } else {
+        Bface[bface_at<T, 2 * NN>(v * NV + c, idx, n)] = wq * isdL * Lb[c];
+        Bface[bface_at<T, 2 * NN>(NN + v * NV + c, idx, n)] = eR >= 0 ? wq * isdR * Rb[c] : T(0);
+      }
     }
   }
 }
@@ -894,6 +916,76 @@ __global__ void __launch_bounds__(256) face_apply_kernel(DGData<T> d, const T* _
   store_face_flux<T, D, P, true>(G, f, q, g);
 }
 
+// Face part of the FP32 J v on tetrahedra.  With stored Jacobians (50 values per point) it was bound
+// by their bytes, 85% of its traffic; it now recomputes the Roe flux's derivative from 16 stored
+// values of the linearisation (about 210 FMAs, next to 100 of the two traces): FP32 arithmetic is
+// cheap here, bytes are not.  Per launch 392 -> 279 us on 48^3 cubes at p = 2, 18.5 -> 12.5 us on
+// 21^3 cubes at p = 1.  What bounds it now is the latency of the gather face -> elements -> rows
+// against the warps in flight: with 70 registers (three blocks per SM) it took 340 us, with two
+// points per thread 366.  Boundary points, whose ghost state's derivative may hold powers, keep
+// their nv x nv block.  FP64 keeps blocks: there the arithmetic is the bound and a block product
+// (50 FMAs) is the cheaper form.
+template <int D, int P>
+__global__ void __launch_bounds__(256, 4) face_record_kernel(DGData<float> d, const float* __restrict__ rec,
+                                                          const float* __restrict__ dv, float* __restrict__ G,
+                                                          const int* __restrict__ skip) {
+  using O = Ord<D, P>;
+  constexpr int NB = O::NB, NFQ = O::NFQ, NV = O::NV, NPERM = O::NPERM, GEO = O::GEO, NBP = PADV<float, NB>;
+  if (skip && *skip) return;
+  const int64_t n = d.F * NFQ, ni = d.F_int * NFQ;
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= n) return;
+  const int64_t f = idx / NFQ;
+  const int q = (int)(idx - f * NFQ);
+  const int2 el = __ldg(reinterpret_cast<const int2*>(d.fel) + f);
+  const int loc = __ldg(d.floc + f);
+  // traces of dv from each side: a padded table row and the element's rows of dv
+  auto trace = [&](int64_t e, int row, float isd, float(&t)[NV]) {
+    float b[NBP];
+    load_row<float, NBP, true>(d.BfP + (int64_t)row * NBP, b);
+    const float* ve = dv + e * NV * NB;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      float c[NB];
+      load_coeffs<float, NB>(ve + v * NB, c);
+      float a = 0.f;
+#pragma unroll
+      for (int j = 0; j < NB; ++j) a = fmaf(b[j], c[j], a);
+      t[v] = a * isd;
+    }
+  };
+  float tL[NV], g[NV];
+  if (idx >= ni) {
+    trace(el.x, ((loc & 0xff) * NPERM) * NFQ + q, 1.f, tL);
+    const float* B = rec + 16 * ni + (idx - ni);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      g[v] = 0.f;
+#pragma unroll
+      for (int c = 0; c < NV; ++c) g[v] = fmaf(__ldg(B + (v * NV + c) * (n - ni)), tL[c], g[v]);
+    }
+    store_face_flux<float, D, P, true>(G, f, q, g);
+    return;
+  }
+  const float4* x = reinterpret_cast<const float4*>(rec) + idx;
+  const float4 xL = __ldg(x), xR = __ldg(x + ni), rho = __ldg(x + 2 * ni), m = __ldg(x + 3 * ni);
+  const float4 geo = __ldg(reinterpret_cast<const float4*>(d.fgeo) + f);
+  const float nr[D] = {geo.x, geo.y, geo.z};
+  float tR[NV], dF[NV];
+  trace(el.x, ((loc & 0xff) * NPERM) * NFQ + q, __ldg(d.geo + GEO * (int64_t)el.x + O::ISD), tL);
+  trace(el.y, (((loc >> 8) & 0xff) * NPERM + (loc >> 16)) * NFQ + q, __ldg(d.geo + GEO * (int64_t)el.y + O::ISD), tR);
+  RoeRecord<float, D> r;
+  r.vL[0] = xL.x, r.vL[1] = xL.y, r.vL[2] = xL.z, r.HL = xL.w;
+  r.vR[0] = xR.x, r.vR[1] = xR.y, r.vR[2] = xR.z, r.HR = xR.w;
+  r.rL = rho.x, r.irL = rho.y, r.rR = rho.z, r.irR = rho.w;
+  r.w = m.x, r.c = m.y, r.i2c = m.z, r.dp = m.w;
+  roe_derivative<D, float>(r, nr, d.fs.gamma, d.rot ? d.vrn[idx] : 0.f, tL, tR, dF);
+  const float wl = geo.w * __ldg(d.Wf + q);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) g[v] = wl * dF[v];
+  store_face_flux<float, D, P, true>(G, f, q, g);
+}
+
 template <class T, int D, int P>
 cudaError_t linearize_p(const DGData<T>& d, const T* u, LinData<T> lin, cudaStream_t st) {
   using O = Ord<D, P>;
@@ -910,7 +1002,11 @@ cudaError_t jac_apply_p(const DGData<T>& d, LinData<T> lin, const T* dv, T* out,
   using O = Ord<D, P>;
   const int64_t nf = d.F * O::NFQ;
   if (ev) cudaEventRecord(ev[0], st);
-  if (nf > 0) face_apply_kernel<T, D, P><<<(unsigned)((nf + 255) / 256), 256, 0, st>>>(d, lin.Bface, dv, G, skip);
+  if (nf > 0) {
+    const unsigned nb = (unsigned)((nf + 255) / 256);
+    if constexpr (FACE_RECORDS<T, D>) face_record_kernel<D, P><<<nb, 256, 0, st>>>(d, lin.Bface, dv, G, skip);
+    else face_apply_kernel<T, D, P><<<nb, 256, 0, st>>>(d, lin.Bface, dv, G, skip);
+  }
   if (ev) cudaEventRecord(ev[1], st);
   elem_op_launch<T, D, P, ELEM_STORED, true>(d, nullptr, dv, lin.pts, G, out, escale, skip, oscale, st);
   if (ev) cudaEventRecord(ev[2], st);

@@ -89,6 +89,7 @@ struct DGData {
   T om[3];
   int rot;
   int64_t E, F;
+  int64_t F_int;         // interior faces (they come first)
   int64_t E_loc;         // elements owned by this partition (E without partitions; ghosts follow)
   Free<T> fs;
   int p;
@@ -102,7 +103,9 @@ struct DGData {
 //                          s = L on boundary faces; in 16-byte chunks of VEC = 16 / sizeof(T)
 //                          entries, [NJF / VEC][F*nfq][VEC], the NJF % VEC left over in
 //                          [F*nfq][NJF % VEC] after them (bface_at), so a point's block loads as
-//                          16-byte vectors
+//                          16-byte vectors; FP32 on tetrahedra: a Roe record per interior
+//                          face point [4][F_int nfq][4], then dF~/dU_L of the boundary points
+//                          [NV NV][boundary points]
 // Index of entry k of face point idx (of n) in Bface.
 template <class T, int NJF>
 __host__ __device__ __forceinline__ int64_t bface_at(int k, int64_t idx, int64_t n) {

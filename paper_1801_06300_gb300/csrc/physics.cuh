@@ -699,4 +699,140 @@ PCEXP_DEV void ghost_farfield_vjp(const S (&U)[D + 2], const T (&n)[D], const Fr
   Ub[0] = Ub[0] - ir * ir * irb;
 }
 
+// ------------------------------------------------- Roe-flux derivative from a stored record
+// What the Roe flux's linearisation at (L, R) needs besides the normal; 14 values (D = 2: 12) that
+// replace its 2 (D + 2)^2 Jacobian entries.  H total enthalpy, w = sqrt(rho_L) / (sqrt(rho_L) +
+// sqrt(rho_R)), c Roe's sound speed, i2c = 1 / (2 c^2), dp = p_R - p_L.
+template <class T, int D>
+struct RoeRecord {
+  T vL[D], HL, rL, irL, vR[D], HR, rR, irR, w, c, i2c, dp;
+};
+
+template <int D, class T>
+PCEXP_DEV RoeRecord<T, D> roe_record(const T (&L)[D + 2], const T (&R)[D + 2], T g) {
+  constexpr int NV = D + 2;
+  const T gm = g - T(1);
+  RoeRecord<T, D> r;
+  r.rL = L[0];
+  r.rR = R[0];
+  r.irL = T(1) / L[0];
+  r.irR = T(1) / R[0];
+  T kL = T(0), kR = T(0), q2 = T(0);
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    r.vL[d] = L[1 + d] * r.irL;
+    r.vR[d] = R[1 + d] * r.irR;
+    kL += L[1 + d] * r.vL[d];
+    kR += R[1 + d] * r.vR[d];
+  }
+  const T pL = gm * (L[NV - 1] - T(0.5) * kL), pR = gm * (R[NV - 1] - T(0.5) * kR);
+  r.HL = (L[NV - 1] + pL) * r.irL;
+  r.HR = (R[NV - 1] + pR) * r.irR;
+  const T sL = sqrt_s(L[0]), sR = sqrt_s(R[0]), is = T(1) / (sL + sR);
+  r.w = sL * is;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    const T vh = (sL * r.vL[d] + sR * r.vR[d]) * is;
+    q2 += vh * vh;
+  }
+  const T cc = gm * ((sL * r.HL + sR * r.HR) * is - T(0.5) * q2);
+  r.c = sqrt_s(cc);
+  r.i2c = T(0.5) / cc;
+  r.dp = pR - pL;
+  return r;
+}
+
+// One side's primitive derivatives along a (its conservative direction), and its share of the
+// central flux's derivative added to C.
+template <class T, int D>
+struct SideDerivative {
+  T lr, v[D], p, q, H;  // d ln rho, dv, dp, d(v . n), dH
+};
+template <int D, class T>
+PCEXP_DEV SideDerivative<T, D> side_derivative(const T (&v)[D], T H, T ir, T qn, const T (&n)[D], T gm,
+                                               const T (&a)[D + 2], T (&C)[D + 2]) {
+  constexpr int NV = D + 2;
+  SideDerivative<T, D> s;
+  T k2 = T(0), e = a[NV - 1], mn = T(0);
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    k2 = fma(T(0.5) * v[d], v[d], k2);
+    e = fma(-v[d], a[1 + d], e);
+    mn = fma(a[1 + d], n[d], mn);
+    s.v[d] = fma(-v[d], a[0], a[1 + d]) * ir;
+  }
+  s.p = gm * fma(k2, a[0], e);
+  const T h = a[NV - 1] + s.p, w = fma(-qn, a[0], mn);  // d(E + p), rho dq
+  s.lr = a[0] * ir;
+  s.q = w * ir;
+  s.H = fma(-H, a[0], h) * ir;
+  C[0] += mn;
+#pragma unroll
+  for (int d = 0; d < D; ++d) C[1 + d] = fma(qn, a[1 + d], fma(v[d], w, fma(s.p, n[d], C[1 + d])));
+  C[NV - 1] = fma(qn, h, fma(H, w, C[NV - 1]));
+  return s;
+}
+
+// dF = dF~/dU_L a + dF~/dU_R b (the derivative of roe_flux, sign(0) = 0 for |x|).
+template <int D, class T>
+PCEXP_DEV void roe_derivative(const RoeRecord<T, D>& r, const T (&n)[D], T g, T vrn, const T (&a)[D + 2],
+                              const T (&b)[D + 2], T (&dF)[D + 2]) {
+  constexpr int NV = D + 2;
+  const T gm = g - T(1);
+  T qL = T(0), qR = T(0), C[NV];
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    qL = fma(r.vL[d], n[d], qL);
+    qR = fma(r.vR[d], n[d], qR);
+  }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) C[v] = T(0);
+  const SideDerivative<T, D> dL = side_derivative<D, T>(r.vL, r.HL, r.irL, qL, n, gm, a, C);
+  const SideDerivative<T, D> dR = side_derivative<D, T>(r.vR, r.HR, r.irR, qR, n, gm, b, C);
+  const T wL = r.w, wR = T(1) - r.w, t = T(0.5) * wL * wR * (dL.lr - dR.lr);  // t = dw_L
+  const T dH = r.HR - r.HL, dq = qR - qL, ddq = dR.q - dL.q;
+  const T Hh = fma(wR, dH, r.HL), qh = fma(wR, dq, qL), rh = fma(r.rL, wR, r.rR * wL);
+  const T dHh = fma(wL, dL.H, fma(wR, dR.H, -t * dH)), drh = T(0.5) * rh * (dL.lr + dR.lr);
+  T vh[D], dvh[D], dv[D], ddv[D], vhd = T(0), dqh = T(0), vdv = T(0), dvdv = T(0), k2 = T(0);
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    dv[d] = r.vR[d] - r.vL[d];
+    ddv[d] = dR.v[d] - dL.v[d];
+    vh[d] = fma(wR, dv[d], r.vL[d]);
+    dvh[d] = fma(wL, dL.v[d], fma(wR, dR.v[d], -t * dv[d]));
+    vhd = fma(vh[d], dvh[d], vhd);
+    dqh = fma(dvh[d], n[d], dqh);
+    vdv = fma(vh[d], dv[d], vdv);
+    dvdv = fma(dvh[d], dv[d], fma(vh[d], ddv[d], dvdv));
+    k2 = fma(T(0.5) * vh[d], vh[d], k2);
+  }
+  const T dcc = gm * (dHh - vhd), c = r.c, dc = dcc * r.i2c * c;  // c = sqrt(cc), i2c = 1 / (2 cc)
+  const T qs = qh - vrn;
+  const T s1 = sign_of(qs - c), s2 = sign_of(qs), s4 = sign_of(qs + c);
+  const T l1 = s1 * (qs - c), l2 = s2 * qs, l4 = s4 * (qs + c);
+  const T dl1 = s1 * (dqh - dc), dl2 = s2 * dqh, dl4 = s4 * (dqh + dc);
+  const T w0 = rh * c * dq, dw0 = fma(drh * c, dq, rh * fma(dc, dq, c * ddq));
+  const T ddp = dR.p - dL.p, ri = T(-2) * r.i2c * dcc;  // di2c = i2c ri
+  const T a1 = (r.dp - w0) * r.i2c, a4 = (r.dp + w0) * r.i2c, a2 = fma(T(-2) * r.dp, r.i2c, r.rR - r.rL);
+  const T da1 = fma(ddp - dw0, r.i2c, a1 * ri), da4 = fma(ddp + dw0, r.i2c, a4 * ri);
+  const T da2 = fma(T(-2) * r.i2c, fma(r.dp, ri, ddp), b[0] - a[0]);
+  const T t1 = l1 * a1, t4 = l4 * a4, t2 = l2 * a2, ts = l2 * rh;
+  const T dt1 = fma(dl1, a1, l1 * da1), dt4 = fma(dl4, a4, l4 * da4), dt2 = fma(dl2, a2, l2 * da2);
+  const T dts = fma(dl2, rh, l2 * drh);
+  const T e = t1 + t4, de = dt1 + dt4, S = e + t2, dS = de + dt2;
+  const T m = t4 - t1, mc = m * c, dmc = fma(dt4 - dt1, c, m * dc);
+  const T cn = dmc - fma(dts, dq, ts * ddq);
+  dF[0] = T(0.5) * (C[0] - dS);
+#pragma unroll
+  for (int d = 0; d < D; ++d)
+    dF[1 + d] = T(0.5) * (C[1 + d] - fma(dS, vh[d], fma(S, dvh[d], fma(cn, n[d], fma(dts, dv[d], ts * ddv[d])))));
+  const T dE = fma(de, Hh, fma(e, dHh, fma(dmc, qh, fma(mc, dqh, fma(dt2, k2, t2 * vhd))))) +
+               fma(dts, fma(-qh, dq, vdv), ts * (dvdv - fma(dqh, dq, qh * ddq)));
+  dF[NV - 1] = T(0.5) * (C[NV - 1] - dE);
+  if (vrn != T(0)) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) dF[v] = fma(T(-0.5) * vrn, a[v] + b[v], dF[v]);
+  }
+}
+
 }  // namespace pcexp
