@@ -433,15 +433,87 @@ PCEXP_DEV void cgs_grid_tail(const Acc<T>* red, int nred, int mode, int j, KStat
   if (threadIdx.x == 0) ks->counter = 0;
 }
 
-// Column-split Gram-Schmidt pass (PROJ, UPD_PROJ, UPD_NORM).  The 8 warps of a block walk
-// the same tiles of 32 x VN rows; warp w owns the columns c = w, w + 8, ... (NCW of them),
-// so a thread holds NCW accumulators instead of one per column and many blocks fit per SM
-// (more loads in flight).  Update modes: each warp forms its partial sum of coef_c z_c,
-// the partials meet in shared memory, warp 0 subtracts them in a fixed warp order, stores
-// the updated tile and publishes it, and each warp projects it on its own columns with
-// the chunks still in registers (two block barriers per tile).
+// FP32 projection pass (PROJ and PROJ2): h = V^T w and ||w||^2.  The 8 warps of a block walk the
+// same tiles of rows and warp w owns the columns w, w + 8, ... (NCW of them, NCW the least that
+// covers the columns), so a thread holds NCW accumulators instead of one per column.  A tile is U
+// chunks of 512 bytes per column: a warp reads U consecutive chunks of each of its columns, all
+// loads issued before their sums, and the grid is exactly one wave.  Bound by HBM bytes.
+// Against the form with NCW = 1, 2, 4, one chunk per column and step (time per launch, 48^3 cubes
+// at p = 2, K = 33.2 M; 8 / 16 / 20 / 24 / 30 columns): 188 / 340 / 520 / 537 / 622 -> 171 / 325 /
+// 400 / 462 / 568 us, 6.9 to 7.2 TB/s; on 131,072 triangles at p = 3 (K = 5.2 M) 39 / 64 / 92 / 97
+// / 110 -> 35 / 61 / 72 / 83 / 99 us.
 constexpr int CGS_WARPS = 8;
+template <int NCW, int U>
+__global__ void __launch_bounds__(256) cgs_proj_kernel(const float* __restrict__ Z, int64_t ldz, int64_t Kp, int j,
+                                                       const float* __restrict__ w, KState* ks,
+                                                       double* __restrict__ partials, double eta, int fmode) {
+  constexpr int VN = VecN<float>::N, CHUNK = 32 * VN, TR = CHUNK * U;
+  __shared__ Acc<float> red[CGS_WARPS * NCW + 1];
+  if (ks->done) return;  // breakdown reached earlier: uniform early exit
+  if (cgs_skipped(fmode, ks)) return;
+  const int nc = j + 1;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  Acc<float> acc[NCW + 1];
+#pragma unroll
+  for (int k = 0; k <= NCW; ++k) acc[k].zero();
+  const int64_t ntile = (Kp + TR - 1) / TR;
+  for (int64_t t = blockIdx.x; t < ntile; t += gridDim.x) {
+    const int64_t r = t * TR + lane * VN;
+    float x[U][VN], z[NCW][U][VN];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (r + u * CHUNK < Kp) {
+        load_vec<float, VN>(w + r + u * CHUNK, x[u]);
+      } else {
+#pragma unroll
+        for (int v = 0; v < VN; ++v) x[u][v] = 0.f;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < NCW; ++k) {
+      const int c = wid + CGS_WARPS * k;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (c < nc && r + u * CHUNK < Kp) {
+          load_vec<float, VN>(Z + (int64_t)c * ldz + r + u * CHUNK, z[k][u]);
+        } else {
+#pragma unroll
+          for (int v = 0; v < VN; ++v) z[k][u][v] = 0.f;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+#pragma unroll
+      for (int k = 0; k < NCW; ++k) acc_dot<float, VN>(acc[k], z[k][u], x[u]);
+      if (wid == 0) acc_dot<float, VN>(acc[NCW], x[u], x[u]);
+    }
+  }
+  // warp sums of the owned columns (fixed shuffle tree); each column has one owner warp.  Slots:
+  // columns 0..nc-1, the norm at nc
+#pragma unroll
+  for (int k = 0; k < NCW; ++k) {
+    for (int o = 16; o > 0; o >>= 1) acc[k].add_partner(o);
+    if (lane == 0 && wid + CGS_WARPS * k < nc) red[wid + CGS_WARPS * k] = acc[k];
+  }
+  if (wid == 0) {
+    for (int o = 16; o > 0; o >>= 1) acc[NCW].add_partner(o);
+    if (lane == 0) red[nc] = acc[NCW];
+  }
+  __syncthreads();
+  cgs_grid_tail<float>(red, nc + 1, fmode, j, ks, partials, eta);
+}
 
+// Column-split update-and-projection pass (FP32 with both passes on every column).  Warps and
+// columns as above; each warp forms its partial sum of coef_c z_c, the partials meet in shared
+// memory, warp 0 subtracts them in a fixed warp order, stores the updated tile and publishes it,
+// and each warp projects it on its own columns with the chunks still in registers (two block
+// barriers per tile).  Each thread copies its own chunks of the block's next tile into its own
+// shared-memory slots with cp.async while it works on the current tile (two stages), so the next
+// tile's loads are in flight across this tile's two block barriers without holding registers; no
+// other thread reads a thread's slots, so the copies need no barrier of their own (C5: 29.5 ->
+// 26.4 ms per step).
+//
 // 16-byte asynchronous copy global -> shared (bypassing L1), and its group fences
 PCEXP_DEV void cgs_cp16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
@@ -452,34 +524,27 @@ PCEXP_DEV void cgs_cp_commit() { asm volatile("cp.async.commit_group;" ::: "memo
 PCEXP_DEV void cgs_cp_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 PCEXP_DEV void cgs_cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-template <class T, int NCW, int MODE>
-__global__ void __launch_bounds__(256) cgs_cs_kernel(const T* __restrict__ Z, int64_t ldz, int64_t Kp, int j,
-                                                     T* __restrict__ w, T* __restrict__ out, KState* ks,
-                                                     double* __restrict__ partials, double eta, int fmode) {
-  constexpr int VN = VecN<T>::N, TR = 32 * VN;
-  __shared__ T scoef[CGS_WARPS * NCW];
-  __shared__ T part[(MODE == CGS_PROJ) ? 1 : CGS_WARPS * TR];
-  __shared__ T xs[(MODE == CGS_UPD_PROJ) ? TR : 1];
-  __shared__ Acc<T> red[CGS_WARPS * NCW + 1];
+template <int NCW>
+__global__ void __launch_bounds__(256) cgs_upd_proj_kernel(const float* __restrict__ Z, int64_t ldz, int64_t Kp, int j,
+                                                           float* __restrict__ w, KState* ks,
+                                                           double* __restrict__ partials, double eta, int fmode) {
+  constexpr int VN = VecN<float>::N, TR = 32 * VN;
+  __shared__ float scoef[CGS_WARPS * NCW];
+  __shared__ float part[CGS_WARPS * TR];
+  __shared__ float xs[TR];
+  __shared__ Acc<float> red[CGS_WARPS * NCW];
   if (ks->done) return;  // breakdown reached earlier: uniform early exit
   if (cgs_skipped(fmode, ks)) return;
   const int nc = j + 1;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int c = threadIdx.x; c < CGS_WARPS * NCW; c += blockDim.x) scoef[c] = c < nc ? (T)ks->coef[c] : T(0);
+  for (int c = threadIdx.x; c < CGS_WARPS * NCW; c += blockDim.x) scoef[c] = c < nc ? (float)ks->coef[c] : 0.f;
   __syncthreads();
-  Acc<T> acc[NCW + 1];
+  Acc<float> acc[NCW];
 #pragma unroll
-  for (int k = 0; k <= NCW; ++k) acc[k].zero();
+  for (int k = 0; k < NCW; ++k) acc[k].zero();
   const int64_t ntile = (Kp + TR - 1) / TR;
-  // FP32 update-and-projection pass: each thread copies its own chunks of the block's next
-  // tile into its own shared-memory slots with cp.async while it works on the current tile
-  // (two stages), so the next tile's loads are in flight across this tile's two block
-  // barriers without holding registers; no other thread reads a thread's slots, so the copies
-  // need no barrier of their own.  (C5: 29.5 -> 26.4 ms per step; the projection pass, which
-  // has no barriers, measured slower staged: 24.6 against 22.3 ms.)
-  constexpr bool STAGED = MODE == CGS_UPD_PROJ && sizeof(T) == 4;
   constexpr int SLOTS = NCW + 1;  // the thread's column chunks, then its chunk of w
-  __shared__ __align__(16) T stg[STAGED ? 2 * CGS_WARPS * SLOTS * TR : 1];
+  __shared__ __align__(16) float stg[2 * CGS_WARPS * SLOTS * TR];
   auto slot = [&](int buf, int k) { return stg + ((buf * CGS_WARPS + wid) * SLOTS + k) * TR + lane * VN; };
   auto issue = [&](int64_t t, int buf) {
     const int64_t r = t * TR + lane * VN;
@@ -487,113 +552,61 @@ __global__ void __launch_bounds__(256) cgs_cs_kernel(const T* __restrict__ Z, in
 #pragma unroll
     for (int k = 0; k < NCW; ++k)
       if (wid + CGS_WARPS * k < nc) cgs_cp16(slot(buf, k), Z + (wid + CGS_WARPS * k) * ldz + r);
-    if (MODE == CGS_PROJ || wid == 0) cgs_cp16(slot(buf, NCW), w + r);
+    if (wid == 0) cgs_cp16(slot(buf, NCW), w + r);
   };
-  if constexpr (STAGED) {
-    if ((int64_t)blockIdx.x < ntile) issue(blockIdx.x, 0);
-    cgs_cp_commit();
-  }
+  if ((int64_t)blockIdx.x < ntile) issue(blockIdx.x, 0);
+  cgs_cp_commit();
   int it = 0;
   for (int64_t t = blockIdx.x; t < ntile; t += gridDim.x, ++it) {
     const int64_t r = t * TR + lane * VN;
     const bool valid = r < Kp;
-    if constexpr (STAGED) {
-      if (t + gridDim.x < ntile) issue(t + gridDim.x, (it & 1) ^ 1);
-      cgs_cp_commit();
-      cgs_cp_wait_prev();  // this tile's copies (all but the group just committed) have landed
+    if (t + gridDim.x < ntile) issue(t + gridDim.x, (it & 1) ^ 1);
+    cgs_cp_commit();
+    cgs_cp_wait_prev();  // this tile's copies (all but the group just committed) have landed
+    float z[NCW][VN], x[VN], p[VN];
+#pragma unroll
+    for (int v = 0; v < VN; ++v) {
+      p[v] = 0.f;
+      x[v] = valid && wid == 0 ? slot(it & 1, NCW)[v] : 0.f;
     }
-    T z[NCW][VN];
 #pragma unroll
     for (int k = 0; k < NCW; ++k) {
-      const int c = wid + CGS_WARPS * k;
-      if (valid && c < nc) {
-        if constexpr (STAGED) {
+      const float cf = scoef[wid + CGS_WARPS * k];
 #pragma unroll
-          for (int v = 0; v < VN; ++v) z[k][v] = slot(it & 1, k)[v];
-        } else {
-          load_vec<T, VN>(Z + c * ldz + r, z[k]);
-        }
-      } else {
-#pragma unroll
-        for (int v = 0; v < VN; ++v) z[k][v] = T(0);
+      for (int v = 0; v < VN; ++v) {
+        z[k][v] = valid && wid + CGS_WARPS * k < nc ? slot(it & 1, k)[v] : 0.f;
+        p[v] = fmaf(cf, z[k][v], p[v]);
       }
     }
-    // every warp needs the tile of w for the projection; in the update modes only warp 0
-    // (which applies the update), loading it here so the load overlaps the column loads
-    T x[VN];
-    if (valid && (MODE == CGS_PROJ || wid == 0)) {
-      if constexpr (STAGED) {
 #pragma unroll
-        for (int v = 0; v < VN; ++v) x[v] = slot(it & 1, NCW)[v];
-      } else {
-        load_vec<T, VN>(w + r, x);
-      }
-    } else {
+    for (int v = 0; v < VN; ++v) part[wid * TR + lane * VN + v] = p[v];
+    __syncthreads();
+    // warp 0 forms the updated tile once (fixed warp order), stores it and publishes it
+    if (wid == 0) {
 #pragma unroll
-      for (int v = 0; v < VN; ++v) x[v] = T(0);
+      for (int q = 0; q < CGS_WARPS; ++q)
+#pragma unroll
+        for (int v = 0; v < VN; ++v) x[v] -= part[q * TR + lane * VN + v];
+      if (valid) store_vec<float, VN>(w + r, x);
+#pragma unroll
+      for (int v = 0; v < VN; ++v) xs[lane * VN + v] = x[v];
     }
-    if constexpr (MODE == CGS_PROJ) {
+    __syncthreads();
+    float xn[VN];
 #pragma unroll
-      for (int k = 0; k < NCW; ++k) acc_dot<T, VN>(acc[k], z[k], x);
-      if (wid == 0) acc_dot<T, VN>(acc[NCW], x, x);
-    } else {
-      T p[VN];
+    for (int v = 0; v < VN; ++v) xn[v] = xs[lane * VN + v];
 #pragma unroll
-      for (int v = 0; v < VN; ++v) p[v] = T(0);
-#pragma unroll
-      for (int k = 0; k < NCW; ++k) {
-        const T cf = scoef[wid + CGS_WARPS * k];
-#pragma unroll
-        for (int v = 0; v < VN; ++v) p[v] = fma(cf, z[k][v], p[v]);
-      }
-#pragma unroll
-      for (int v = 0; v < VN; ++v) part[wid * TR + lane * VN + v] = p[v];
-      __syncthreads();
-      // warp 0 forms the updated tile once (fixed warp order), stores it and publishes it
-      if (wid == 0) {
-#pragma unroll
-        for (int q = 0; q < CGS_WARPS; ++q)
-#pragma unroll
-          for (int v = 0; v < VN; ++v) x[v] -= part[q * TR + lane * VN + v];
-        if (valid) store_vec<T, VN>((MODE == CGS_UPD_PROJ ? w : out) + r, x);
-        if constexpr (MODE == CGS_UPD_PROJ) {
-#pragma unroll
-          for (int v = 0; v < VN; ++v) xs[lane * VN + v] = x[v];
-        } else {
-          acc_dot<T, VN>(acc[NCW], x, x);
-        }
-      }
-      __syncthreads();
-      if constexpr (MODE == CGS_UPD_PROJ) {
-        T xn[VN];
-#pragma unroll
-        for (int v = 0; v < VN; ++v) xn[v] = xs[lane * VN + v];
-#pragma unroll
-        for (int k = 0; k < NCW; ++k) acc_dot<T, VN>(acc[k], z[k], xn);
-      }
-    }
+    for (int k = 0; k < NCW; ++k) acc_dot<float, VN>(acc[k], z[k], xn);
   }
-  if constexpr (STAGED) cgs_cp_wait_all();  // no copy outlives the block
+  cgs_cp_wait_all();  // no copy outlives the block
   // warp sums of the owned columns (fixed shuffle tree); each column has one owner warp
-  if constexpr (MODE != CGS_UPD_NORM) {
 #pragma unroll
-    for (int k = 0; k < NCW; ++k) {
-      for (int o = 16; o > 0; o >>= 1) acc[k].add_partner(o);
-      if (lane == 0) red[wid + CGS_WARPS * k] = acc[k];
-    }
-  }
-  if (MODE != CGS_UPD_PROJ && wid == 0) {
-    for (int o = 16; o > 0; o >>= 1) acc[NCW].add_partner(o);
-    if (lane == 0) red[MODE == CGS_PROJ ? CGS_WARPS * NCW : 0] = acc[NCW];
+  for (int k = 0; k < NCW; ++k) {
+    for (int o = 16; o > 0; o >>= 1) acc[k].add_partner(o);
+    if (lane == 0) red[wid + CGS_WARPS * k] = acc[k];
   }
   __syncthreads();
-  // partial-sum slots: PROJ columns 0..nc-1 and the norm at nc; UPD_PROJ columns; UPD_NORM the norm
-  __shared__ Acc<T> ordered[MMAX + 1];
-  const int nred = (MODE == CGS_PROJ) ? nc + 1 : (MODE == CGS_UPD_PROJ ? nc : 1);
-  for (int c = threadIdx.x; c < nred; c += blockDim.x)
-    ordered[c] = (MODE == CGS_PROJ && c == nc) ? red[CGS_WARPS * NCW] : red[c];
-  __syncthreads();
-  cgs_grid_tail<T>(ordered, nred, fmode, j, ks, partials, eta);
+  cgs_grid_tail<float>(red, nc, fmode, j, ks, partials, eta);
 }
 
 template <class KernelT>
@@ -627,35 +640,40 @@ static void cgs_launch(const T* Z, int64_t ldz, int64_t Kp, int j, T* w, T* out,
   cgs_kernel<T, NC, MODE><<<grid_cache, 256, 0, st>>>(Z, ldz, Kp, j, w, out, ks, partials, eta, fmode);
 }
 
-template <class T, int NCW, int MODE>
-static void cgs_cs_launch(const T* Z, int64_t ldz, int64_t Kp, int j, T* w, T* out, KState* ks, double* partials,
-                          double eta, int fmode, cudaStream_t st) {
-  static unsigned grid_cache = 0;
-  static int64_t kp_cache = -1;
-  if (kp_cache != Kp) {
-    grid_cache = wave_grid(cgs_cs_kernel<T, NCW, MODE>, (Kp + 32 * VecN<T>::N - 1) / (32 * VecN<T>::N) * 256);
-    kp_cache = Kp;
-  }
-  cgs_cs_kernel<T, NCW, MODE><<<grid_cache, 256, 0, st>>>(Z, ldz, Kp, j, w, out, ks, partials, eta, fmode);
+// One launch of a streaming kernel on at most one wave of blocks.
+template <int NCW, int U>
+static void cgs_proj_launch(const float* Z, int64_t ldz, int64_t Kp, int j, const float* w, KState* ks,
+                            double* partials, double eta, int fmode, cudaStream_t st) {
+  static const unsigned wave = wave_grid(cgs_proj_kernel<NCW, U>, (int64_t)RED_BLOCKS * 256);
+  constexpr int TR = 32 * VecN<float>::N * U;
+  const int64_t tiles = (Kp + TR - 1) / TR;
+  cgs_proj_kernel<NCW, U><<<(unsigned)(tiles < wave ? tiles : wave), 256, 0, st>>>(Z, ldz, Kp, j, w, ks, partials, eta, fmode);
+}
+template <int NCW>
+static void cgs_upd_proj_launch(const float* Z, int64_t ldz, int64_t Kp, int j, float* w, KState* ks, double* partials,
+                                double eta, int fmode, cudaStream_t st) {
+  static const unsigned wave = wave_grid(cgs_upd_proj_kernel<NCW>, (int64_t)RED_BLOCKS * 256);
+  constexpr int TR = 32 * VecN<float>::N;
+  const int64_t tiles = (Kp + TR - 1) / TR;
+  cgs_upd_proj_kernel<NCW><<<(unsigned)(tiles < wave ? tiles : wave), 256, 0, st>>>(Z, ldz, Kp, j, w, ks, partials, eta, fmode);
 }
 
-// Which layout serves a precision and pass: the column-split kernel (column capacity
-// 8 x NCW, NCW = 1, 2, 4) or the row kernel (every thread accumulates all columns of its
-// rows).  Measured on GB300 (C2 and the 48^3 tetrahedra): the FP32 projections gain from
-// the column split (fewer registers, more loads in flight); the FP64 passes are bound by
-// the FP64 pipe and the update-and-norm pass keeps one accumulator, so the row kernel's
-// single barrier-free sweep is faster for those.
-template <class T, int MODE> struct CgsColumnSplit {
-  static constexpr bool value = sizeof(T) == 4 && MODE != CGS_UPD_NORM;
-};
-
+// Which kernel serves a precision and pass.  Measured on GB300 (192 x 64 bump and 48^3
+// tetrahedra): the FP32 projections gain from the column split (fewer registers, more loads in
+// flight); the FP64 passes are bound by the FP64 pipe and the update-and-norm pass keeps one
+// accumulator, so the row kernel's single barrier-free sweep is faster for those.
 template <class T, int MODE>
 static void cgs_dispatch(int nc, const T* Z, int64_t ldz, int64_t Kp, int j, T* w, T* out, KState* ks,
                          double* partials, double eta, int fmode, cudaStream_t st) {
-  if constexpr (CgsColumnSplit<T, MODE>::value) {
-    if (nc <= CGS_WARPS) cgs_cs_launch<T, 1, MODE>(Z, ldz, Kp, j, w, out, ks, partials, eta, fmode, st);
-    else if (nc <= 2 * CGS_WARPS) cgs_cs_launch<T, 2, MODE>(Z, ldz, Kp, j, w, out, ks, partials, eta, fmode, st);
-    else cgs_cs_launch<T, 4, MODE>(Z, ldz, Kp, j, w, out, ks, partials, eta, fmode, st);
+  if constexpr (sizeof(T) == 4 && MODE == CGS_PROJ) {
+    if (nc <= CGS_WARPS) cgs_proj_launch<1, 4>(Z, ldz, Kp, j, w, ks, partials, eta, fmode, st);
+    else if (nc <= 2 * CGS_WARPS) cgs_proj_launch<2, 3>(Z, ldz, Kp, j, w, ks, partials, eta, fmode, st);
+    else if (nc <= 3 * CGS_WARPS) cgs_proj_launch<3, 4>(Z, ldz, Kp, j, w, ks, partials, eta, fmode, st);
+    else cgs_proj_launch<4, 4>(Z, ldz, Kp, j, w, ks, partials, eta, fmode, st);
+  } else if constexpr (sizeof(T) == 4 && MODE == CGS_UPD_PROJ) {
+    if (nc <= CGS_WARPS) cgs_upd_proj_launch<1>(Z, ldz, Kp, j, w, ks, partials, eta, fmode, st);
+    else if (nc <= 2 * CGS_WARPS) cgs_upd_proj_launch<2>(Z, ldz, Kp, j, w, ks, partials, eta, fmode, st);
+    else cgs_upd_proj_launch<4>(Z, ldz, Kp, j, w, ks, partials, eta, fmode, st);
   } else {
     if (nc <= 4) cgs_launch<T, 4, MODE>(Z, ldz, Kp, j, w, out, ks, partials, eta, fmode, st);
     else if (nc <= 8) cgs_launch<T, 8, MODE>(Z, ldz, Kp, j, w, out, ks, partials, eta, fmode, st);
