@@ -45,7 +45,8 @@ extern "C" {
 #define PCEXP_ERR_CUDA (-3)        /* a CUDA runtime call failed */
 #define PCEXP_ERR_OOM (-4)         /* device allocation failed */
 #define PCEXP_ERR_NONFINITE (-5)   /* a norm, beta or h_{j+1,j} was NaN/Inf */
-#define PCEXP_ERR_TIMEOUT (-6)     /* a partition of a group missed a rendezvous (failed or stalled) */
+#define PCEXP_ERR_TIMEOUT (-6)     /* a partition of a group missed a rendezvous (failed or stalled), or
+                                      the blocks of a cooperative kernel did not meet in time */
 #define PCEXP_ERR_UNSUPPORTED (-7) /* valid request this build does not cover */
 
 /* ---- boundary tags (Sec. 4.4, Sec. 5.2) ---- */
@@ -347,7 +348,9 @@ int pcexp_output(pcexp_ctx* ctx, int kind, double* value);
 #define PCEXP_KC_LINEARIZE 12    /* point Jacobians at u_n (once per step) */
 #define PCEXP_KC_CGS_UPD1 13     /* selective form: w_1 = w - V h; ||w_1|| and the decision */
 #define PCEXP_KC_CGS_PROJ2 14    /* selective form: h2 = V^T w_1 where the first pass cancelled */
-#define PCEXP_KC_COUNT 15
+#define PCEXP_KC_CGS_COLUMN 15   /* a whole Gram-Schmidt column in one launch (vectors of up to a
+                                    few MB; the passes above serve longer ones) */
+#define PCEXP_KC_COUNT 16
 int pcexp_profile_enable(pcexp_ctx* ctx, int enable);
 int pcexp_profile_read(pcexp_ctx* ctx, int kernel_class, int64_t* launches, double* ms);
 

@@ -47,7 +47,7 @@ PCEXP_FUNC_VORTEX_L2 = 2
 PCEXP_FUNC_WALL_FZ = 3
 KERNEL_CLASSES = ["residual_face", "residual_elem", "jvp_face", "jvp_elem", "cgs_norm", "cgs_proj",
                   "cgs_upd_proj", "cgs_upd_norm", "phi", "axpy", "dt", "other", "linearize", "cgs_upd1",
-                  "cgs_proj2"]
+                  "cgs_proj2", "cgs_column"]
 
 
 class pcexp_mesh(C.Structure):

@@ -36,6 +36,8 @@ struct pcexp_ctx {
   double eta = 0;
   double ktol = 0;  // Krylov tolerance of the adaptive dimension (<= 0: fixed dimension)
   bool selective = false;  // Arnoldi: second Gram-Schmidt pass only after a cancelling first pass
+  ColumnPlan col{0, 0};    // one-launch Gram-Schmidt columns (blocks == 0: the separate passes)
+  unsigned long long* col_slots = nullptr;  // their exchange slots
   int basis_io = PCEXP_BASIS_PAPER;
   double volume = 0;
   pcexp_physics phys{};
@@ -483,6 +485,13 @@ int refresh_shadow(pcexp_ctx* c, int i) {
   return PCEXP_OK;
 }
 
+// Status of a nonzero KState.err / StepState.err: 1 a non-finite quantity, 2 an exchange of a
+// one-launch column that ran out of polls.
+int krylov_error(int err, const char* nonfinite) {
+  g_last_error = err == 2 ? "a Gram-Schmidt kernel's blocks did not meet in time" : nonfinite;
+  return err == 2 ? PCEXP_ERR_TIMEOUT : PCEXP_ERR_NONFINITE;
+}
+
 // Columns between checkpoints of the adaptive Krylov dimension.
 constexpr int KRYLOV_CHECK = 5;
 
@@ -497,13 +506,19 @@ int arnoldi(pcexp_ctx* c, const T* escale, int m, const double* dt_dev = nullptr
   T* G = reinterpret_cast<T*>(c->G);
   T* V = reinterpret_cast<T*>(c->V);
   (void)G;
-  PCEXP_LAUNCH(c, PCEXP_KC_OTHER, launch_reset_kstate(c->ks, c->st));
+  PCEXP_LAUNCH(c, PCEXP_KC_OTHER, launch_reset_kstate(c->ks, c->st, c->col_slots, &c->col));
   PCEXP_LAUNCH(c, PCEXP_KC_CGS_NORM, launch_cgs<T>(CGS_NORM, V, c->Kp, c->Kp, 0, V, nullptr, c->ks, c->partials, c->eta, c->st));
   PCEXP_TRY(group_cgs(c, CGS_NORM, 0));
   for (int j = 0; j < m; ++j) {
     // w = J v_j = s_j J z_j: the basis scale is applied to the output, so every
     // stored vector stays of the size of ||J|| (no growth like ||J||^j)
     PCEXP_TRY(jac_apply<T>(c, d, Vcol<T>(c, j), w, escale, &c->ks->done, &c->ks->s[j]));
+    if (c->col.blocks > 0) {
+      PCEXP_LAUNCH(c, PCEXP_KC_CGS_COLUMN, launch_cgs_column<T>(c->col, V, c->Kp, c->Kp, j, w, Vcol<T>(c, j + 1), c->ks, c->col_slots, c->eta, c->selective, c->st));
+      if (c->ktol > 0 && dt_dev && (j + 1) % KRYLOV_CHECK == 0 && j + 1 < m)
+        PCEXP_LAUNCH(c, PCEXP_KC_PHI, launch_phi_check(c->ks, dt_dev, c->ktol, c->st));
+      continue;
+    }
     PCEXP_LAUNCH(c, PCEXP_KC_CGS_PROJ, launch_cgs<T>(CGS_PROJ, V, c->Kp, c->Kp, j, w, nullptr, c->ks, c->partials, c->eta, c->st));
     PCEXP_TRY(group_cgs(c, CGS_PROJ, j));
     if (c->selective) {
@@ -726,10 +741,7 @@ int step_impl(pcexp_ctx* c, int scheme, int dt_mode, double dt_or_cfl, int m, pc
     info->krylov_err[1] = one_stage ? 0.0 : h.kerr[1];
     info->reorth_cols[0] = h.pass2[0];
     info->reorth_cols[1] = one_stage ? 0u : h.pass2[1];
-    if (h.err) {
-      g_last_error = "non-finite norm, beta or Hessenberg entry";
-      return PCEXP_ERR_NONFINITE;
-    }
+    if (h.err) return krylov_error(h.err, "non-finite norm, beta or Hessenberg entry");
   }
   return PCEXP_OK;
 }
@@ -819,10 +831,7 @@ int arnoldi_abi(pcexp_ctx* c, const double* U, const double* b, int m, double* V
   KState hk;
   PCEXP_CK(cudaMemcpyAsync(&hk, c->ks, sizeof(hk), cudaMemcpyDeviceToHost, c->st));
   PCEXP_CK(cudaStreamSynchronize(c->st));
-  if (hk.err) {
-    g_last_error = "non-finite Arnoldi quantity";
-    return PCEXP_ERR_NONFINITE;
-  }
+  if (hk.err) return krylov_error(hk.err, "non-finite Arnoldi quantity");
   const int kk = hk.k;
   if (k) *k = kk;
   if (beta) *beta = hk.beta;
@@ -1398,8 +1407,7 @@ int step_backward_impl(pcexp_ctx* c, const double* U, double dt, int m, const do
   PCEXP_CK(cudaStreamSynchronize(c->st));
   if (h1.err || h2.err) {
     c->prof = prof;
-    g_last_error = "non-finite quantity in the recomputed step";
-    return PCEXP_ERR_NONFINITE;
+    return krylov_error(std::max(h1.err, h2.err), "non-finite quantity in the recomputed step");
   }
   const int k1 = h1.k, k2 = h2.k;
   // ---- reverse
@@ -1522,6 +1530,11 @@ int pcexp_create(pcexp_ctx** out, const pcexp_mesh* mesh, int p, const pcexp_phy
   cudaGetDevice(&c->device);
   c->st = reinterpret_cast<cudaStream_t>(cuda_stream);
   int r = create_impl(c, mesh, p, phys, opt);
+  if (r == PCEXP_OK) {
+    // (a partition's columns keep the separate passes: their sums meet the other partitions' in between)
+    c->col = c->fp32 ? plan_cgs_column<float>(c->Kp) : plan_cgs_column<double>(c->Kp);
+    if (c->col.blocks > 0) r = dalloc(c, &c->col_slots, column_slots(c->col));
+  }
   if (r != PCEXP_OK) {
     std::string keep = g_last_error;
     pcexp_destroy(c);

@@ -307,6 +307,24 @@ enum CgsMode { CGS_PROJ = 0, CGS_UPD_PROJ = 1, CGS_UPD_NORM = 2, CGS_NORM = 3, C
 template <class T>
 cudaError_t launch_cgs(int mode, const T* Z, int64_t ldz, int64_t Kp, int j, T* w, T* out,
                        KState* ks, double* partials, double eta, cudaStream_t st);
+// A whole column in one cooperative launch (project, update, and the second pass where it runs),
+// for vectors whose share of one block fits its shared memory.  The plan is made per context;
+// blocks == 0: the separate passes serve this length.
+struct ColumnPlan {
+  int blocks, rows;
+};
+constexpr int COL_SUMS = MMAX + 2;       // slots per block of one exchange of sums
+constexpr int COL_MAX_BLOCKS = 160;
+// slots of a context's columns: two sets of four exchanges
+inline size_t column_slots(const ColumnPlan& p) { return (size_t)2 * 4 * COL_SUMS * p.blocks; }
+// Bytes of a block's rows up to which the one-launch column is the faster form (measured, see
+// cgs_column_kernel).
+template <class T> constexpr int64_t COLUMN_MAX_BYTES = sizeof(T) == 8 ? 100 * 1024 : 32 * 1024;
+template <class T>
+ColumnPlan plan_cgs_column(int64_t Kp);
+template <class T>
+cudaError_t launch_cgs_column(const ColumnPlan& plan, const T* Z, int64_t ldz, int64_t Kp, int j, const T* w, T* out,
+                              KState* ks, unsigned long long* slots, double eta, bool selective, cudaStream_t st);
 // phi_1/phi_2 of dt H_k (dt from *dt_dev when non-null, else dt) -> ks->y, ks->y2,
 // ks->acoef = factor * dt * beta * y_i * s_i (which = 1) or factor * dt * beta * y2_i * s_i (which = 2),
 // times dt / *dt_prev when dt_prev is non-null; records k and beta into ss->k[stage], ss->beta[stage].
@@ -353,7 +371,9 @@ template <class T>
 cudaError_t launch_zero_range(T* x, int64_t from, int64_t to, cudaStream_t st);
 // ss->cfl = min(ss->cfl, cap) (the Krylov-error cap of the steady march)
 cudaError_t launch_cap_cfl(StepState* ss, double cap, cudaStream_t st);
-cudaError_t launch_reset_kstate(KState* ks, cudaStream_t st);
+// slots (nullable): the one-launch columns' slots, the first set of which is emptied
+cudaError_t launch_reset_kstate(KState* ks, cudaStream_t st, unsigned long long* slots = nullptr,
+                                const ColumnPlan* plan = nullptr);
 // ---- reverse Krylov stage (adjoint.cu, FP64)
 // Reverse of the Krylov stage, step by step.  Each reduction (ybar, alpha, upd, b0dot) leaves
 // its sums in as->dots and finishes in its last block; in a partitioned run (as->group) it

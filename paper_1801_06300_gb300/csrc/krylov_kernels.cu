@@ -23,6 +23,7 @@
 // pairs converted to FP64 once per warp (FP32-mixed form).
 #include <cooperative_groups.h>
 #include <cfloat>
+#include <cstddef>
 
 #include "kernels.h"
 
@@ -699,6 +700,406 @@ cudaError_t launch_cgs(int mode, const T* Z, int64_t ldz, int64_t Kp, int j, T* 
   return cudaGetLastError();
 }
 
+// ------------------------------------------------ a whole Gram-Schmidt column in one launch
+// One cooperative kernel does what the separate passes do for column j: project, update, and
+// (CGS2, or where the selective form's first pass cancelled) project and update again.  A block
+// owns a contiguous range of rows and keeps its part of w in shared memory from the load to the
+// last update, so only the basis is read per sweep.
+//
+// Why: on vectors of up to a few MB the separate launches are bound by their tails, not by their
+// sweeps.  Each of them drains, reduces its block sums in one last block and starts the next
+// (8 to 30 us a pass in FP64 and 5 to 9 us in FP32 against 1 to 8 us of arithmetic), the
+// selective form pays two more launches that leave at once, and a row per thread puts a
+// 27,648-entry FP64 vector on 54 of the 152 SMs.  Here the rows are spread over all SMs and a sweep
+// ends in an all-to-all exchange of the block sums through L2 instead of a launch: every block
+// stores its sums and adds up all blocks' itself, in a fixed order.  A slot starts as a bit
+// pattern that no arithmetic result has, so a value is its own flag and the exchange takes one
+// store and one load, no counter.
+// An EXP1 step with 30 columns on periodic triangles at p = 2, separate -> one launch:
+//   FP64  K = 27,648 2010 -> 1464 us, 150,528 2810 -> 2243, 591,408 6641 -> 5976,
+//         1,503,792 14.04 -> 13.42 ms, 1,881,792 (97 KB per block) 17.49 -> 16.91 ms
+//   FP32, selective  K = 12,288 733 -> 642 us, 110,592 832 -> 720, 591,408 1176 -> 1042,
+//         1,080,000 (28 KB per block) 1791 -> 1691, 1,503,792 (39 KB) 2257 -> 2257,
+//         2,764,800 (71 KB) 3560 -> 3719
+// hence COLUMN_MAX_BYTES: 100 KB of rows per block in FP64 (longer ones were not tried), 32 KB in
+// FP32.
+// The projection gives each warp its own columns (one accumulator, so one warp sum per column:
+// the FP64 additions of a 32-column butterfly in every warp cost as much as the sweep of a small
+// vector); the update gives each thread its own rows.
+constexpr int COL_NT = 512, COL_WARPS = COL_NT / 32;
+constexpr unsigned COL_SPIN_LIMIT = 1u << 23;  // polls of an exchange (seconds) before giving up
+// An empty slot: a NaN, as a double and as a pair of floats alike; sums with that bit pattern are
+// stored as another NaN.
+constexpr unsigned long long COL_EMPTY = ~0ull;
+
+template <class T> struct ColumnSmem {
+  alignas(16) T upd[COL_NT * VecN<T>::N];  // partial updates of the column groups (16-byte accesses)
+  Acc<T> lanes[(MMAX + 1) * 32];           // per column: the projection's lane sums
+  Acc<T> gather[COL_WARPS][COL_SUMS];      // per warp: sums of the blocks it adds
+  Acc<T> sums[COL_SUMS];                   // this block's sums
+  double dots[COL_SUMS];                   // the grid's sums
+  double scale[MMAX + 1];                  // s_i
+  T coef[MMAX + 1];
+  int bad, late;
+};
+
+PCEXP_DEV unsigned long long column_peek(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// The grid's sums of sm.sums[0..n) -> sm.dots, identical in every block.  False if a block's sums
+// did not arrive within the limit of polls (ks->err = 2).  Every thread of every block calls this;
+// slots: [block][COL_SUMS], empty before, used by this reduction alone.
+template <class T>
+PCEXP_DEV bool column_grid_sum(ColumnSmem<T>& sm, int n, unsigned long long* slots, KState* ks) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nblk = gridDim.x;
+  __syncthreads();
+  if (threadIdx.x == 0) sm.late = 0;
+  for (int c = threadIdx.x; c < n; c += COL_NT) {
+    unsigned long long v = *reinterpret_cast<const unsigned long long*>(&sm.sums[c]);
+    if (v == COL_EMPTY) v >>= 1;  // a propagated input NaN of that payload: another NaN
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(slots + (int64_t)blockIdx.x * COL_SUMS + c), "l"(v)
+                 : "memory");
+  }
+  bool late = false;
+  if (n == 1) {  // thread = block; the warps that hold blocks add up theirs
+    const int q = threadIdx.x, nw = (nblk + 31) / 32;
+    if (wid < nw) {
+      unsigned long long v = 0ull;
+      unsigned polls = 0;
+      if (q < nblk)
+        do v = column_peek(slots + (int64_t)q * COL_SUMS);
+        while (v == COL_EMPTY && ++polls < COL_SPIN_LIMIT);
+      late = v == COL_EMPTY;
+      Acc<T> a = *reinterpret_cast<const Acc<T>*>(&v);
+      for (int o = 16; o > 0; o >>= 1) a.add_partner(o);
+      if (lane == 0) sm.gather[wid][0] = a;
+    }
+  } else {  // warp = every COL_WARPS-th block, lane = column
+    constexpr int PER = COL_MAX_BLOCKS / COL_WARPS;
+    for (int c = lane; c < n; c += 32) {
+      unsigned long long v[PER];
+      unsigned polls = 0;
+      bool all;
+      do {
+        all = true;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+          const int q = wid + i * COL_WARPS;
+          v[i] = q < nblk ? column_peek(slots + (int64_t)q * COL_SUMS + c) : 0ull;
+          all = all && v[i] != COL_EMPTY;
+        }
+      } while (!all && ++polls < COL_SPIN_LIMIT);
+      late = late || !all;
+      Acc<T> a = *reinterpret_cast<const Acc<T>*>(&v[0]);
+#pragma unroll
+      for (int i = 1; i < PER; ++i) a.add_acc(*reinterpret_cast<const Acc<T>*>(&v[i]));
+      sm.gather[wid][c] = a;
+    }
+  }
+  if (late) sm.late = 1;
+  __syncthreads();
+  if (sm.late) {
+    if (threadIdx.x == 0) {
+      ks->err = 2;
+      ks->done = 1;
+    }
+    return false;
+  }
+  if (n == 1) {
+    if (threadIdx.x == 0) {
+      Acc<T> a = sm.gather[0][0];
+      for (int q = 1; q < (nblk + 31) / 32; ++q) a.add_acc(sm.gather[q][0]);
+      sm.dots[0] = a.value();
+    }
+  } else {  // 16 threads per column add the warps' sums (warps without columns stay out)
+    static_assert(COL_WARPS == 16, "one thread per warp's sum");
+    for (int c0 = 2 * wid; c0 < n; c0 += 2 * COL_WARPS) {
+      const int c = c0 + lane / 16, q = lane % 16;
+      Acc<T> a;
+      a.zero();
+      if (c < n) a = sm.gather[q][c];
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) a.add_partner(o);
+      if (c < n && q == 0) sm.dots[c] = a.value();
+    }
+  }
+  __syncthreads();
+  return true;
+}
+
+// sm.sums[c] = <z_c, x> for c < nc and, with the norm, sm.sums[nc] = <x, x>, over this block's
+// nch chunks x (shared memory); Zb: the first column at the block's first row
+template <class T>
+PCEXP_DEV void column_project(ColumnSmem<T>& sm, const T* xs, const T* __restrict__ Zb, int64_t ldz, int nc, bool norm,
+                              int nch) {
+  constexpr int VN = VecN<T>::N;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int ncols = nc + (norm ? 1 : 0);
+  // warps: CG column groups times RS shares of the rows
+  int CG = 1;
+  while (CG < ncols && CG < COL_WARPS) CG *= 2;
+  const int RS = COL_WARPS / CG, rs = wid / CG;
+  for (int c = wid % CG; c < ncols; c += CG) {
+    Acc<T> acc;
+    acc.zero();
+    const T* z = Zb + (int64_t)c * ldz;
+    if (c < nc) {
+#pragma unroll 4
+      for (int ch = rs * 32 + lane; ch < nch; ch += RS * 32) {
+        T a[VN], x[VN];
+        load_vec<T, VN>(z + ch * VN, a);
+        load_vec<T, VN>(xs + ch * VN, x);
+        acc_dot<T, VN>(acc, a, x);
+      }
+    } else {
+      for (int ch = rs * 32 + lane; ch < nch; ch += RS * 32) {
+        T x[VN];
+        load_vec<T, VN>(xs + ch * VN, x);
+        acc_dot<T, VN>(acc, x, x);
+      }
+    }
+    sm.lanes[(c * RS + rs) * 32 + lane] = acc;  // c RS < 16 or RS = 1: within (MMAX + 1) * 32
+  }
+  __syncthreads();
+  int TPC = 32;  // threads per column
+  while (TPC * ncols > COL_NT) TPC /= 2;
+  const int c = threadIdx.x / TPC, part = threadIdx.x % TPC;
+  if (wid * (32 / TPC) < ncols) {  // warp-uniform
+    Acc<T> a;
+    a.zero();
+    if (c < ncols) {
+      a = sm.lanes[c * RS * 32 + part];
+      for (int i = part + TPC; i < RS * 32; i += TPC) a.add_acc(sm.lanes[c * RS * 32 + i]);
+    }
+    for (int o = TPC / 2; o > 0; o >>= 1) a.add_partner(o);
+    if (c < ncols && part == 0) sm.sums[c] = a;
+  }
+}
+
+// x -= sum_c coef_c z_c over this block's rows, in shared memory and to outb, and
+// sm.sums[0] = <x, x>
+template <class T>
+PCEXP_DEV void column_update(ColumnSmem<T>& sm, T* xs, T* __restrict__ outb, const T* __restrict__ Zb, int64_t ldz,
+                             int nc, int nch) {
+  constexpr int VN = VecN<T>::N;
+  constexpr int U = 8;
+  Acc<T> acc;
+  acc.zero();
+  // few chunks: G groups of threads share the columns, so that the loads of a chunk's columns are
+  // in flight together
+  const int G = nch > 0 && nch * 2 <= COL_NT ? min(8, COL_NT / nch) : 1;
+  if (G > 1) {
+    const int g = threadIdx.x / nch, ch = threadIdx.x - g * nch;
+    if (g < G) {
+      T p[VN];
+#pragma unroll
+      for (int v = 0; v < VN; ++v) p[v] = T(0);
+#pragma unroll 4
+      for (int c = g; c < nc; c += G) {
+        T z[VN];
+        load_vec<T, VN>(Zb + (int64_t)c * ldz + ch * VN, z);
+        const T cf = sm.coef[c];
+#pragma unroll
+        for (int v = 0; v < VN; ++v) p[v] = fma(cf, z[v], p[v]);
+      }
+      store_vec<T, VN>(sm.upd + threadIdx.x * VN, p);
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < nch) {
+      T x[VN];
+      load_vec<T, VN>(xs + threadIdx.x * VN, x);
+      for (int q = 0; q < G; ++q) {
+        T p[VN];
+        load_vec<T, VN>(sm.upd + (q * nch + threadIdx.x) * VN, p);
+#pragma unroll
+        for (int v = 0; v < VN; ++v) x[v] -= p[v];
+      }
+      store_vec<T, VN>(xs + threadIdx.x * VN, x);
+      store_vec<T, VN>(outb + threadIdx.x * VN, x);
+      acc_dot<T, VN>(acc, x, x);
+    }
+  } else {
+    for (int ch = threadIdx.x; ch < nch; ch += COL_NT) {
+      T x[VN];
+      load_vec<T, VN>(xs + ch * VN, x);
+      for (int c0 = 0; c0 < nc; c0 += U) {
+        T z[U][VN];
+#pragma unroll
+        for (int g = 0; g < U; ++g) load_vec<T, VN>(Zb + (int64_t)min(c0 + g, nc - 1) * ldz + ch * VN, z[g]);
+#pragma unroll
+        for (int g = 0; g < U; ++g)
+          if (c0 + g < nc)
+#pragma unroll
+            for (int v = 0; v < VN; ++v) x[v] = fma(-sm.coef[c0 + g], z[g][v], x[v]);
+      }
+      store_vec<T, VN>(xs + ch * VN, x);
+      store_vec<T, VN>(outb + ch * VN, x);
+      acc_dot<T, VN>(acc, x, x);
+    }
+  }
+  sm.lanes[threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.x < 64) {
+    Acc<T> a = sm.lanes[threadIdx.x];
+#pragma unroll
+    for (int i = 1; i < COL_NT / 64; ++i) a.add_acc(sm.lanes[threadIdx.x + 64 * i]);
+    for (int o = 16; o > 0; o >>= 1) a.add_partner(o);
+    if (threadIdx.x == 32) sm.sums[1] = a;
+    if (threadIdx.x == 0) sm.sums[0] = a;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) sm.sums[0].add_acc(sm.sums[1]);
+}
+
+// coefficients of the next update from the projections sm.dots (the scalar step of cgs_finalize's
+// PROJ and UPD_PROJ), in every block; block 0 records them.  False on a non-finite entry.
+template <class T>
+PCEXP_DEV bool column_coefficients(ColumnSmem<T>& sm, int j, bool first, KState* ks) {
+  if (threadIdx.x == 0) sm.bad = 0;
+  __syncthreads();
+  for (int i = threadIdx.x; i <= j; i += COL_NT) {
+    const double si = sm.scale[i], h = si * sm.dots[i];
+    if (!isfinite(h)) sm.bad = 1;
+    sm.coef[i] = (T)(si * h);
+    if (blockIdx.x == 0) {
+      if (first) {
+        ks->H[i * MMAX + j] = h;
+        ks->H1[i * MMAX + j] = h;
+      } else {
+        ks->H[i * MMAX + j] += h;
+      }
+    }
+  }
+  __syncthreads();
+  if (sm.bad && blockIdx.x == 0 && threadIdx.x == 0) {
+    ks->err = 1;
+    ks->done = 1;
+  }
+  return !sm.bad;
+}
+
+// rows: of one block (a multiple of 64; the last blocks may have fewer or none).  slots: two sets
+// of four reductions' slots; column j uses set j & 1 and empties the other for column j + 1 (set
+// 0 is emptied by reset_kstate before column 0).
+template <class T>
+__global__ void __launch_bounds__(COL_NT, 1) cgs_column_kernel(const T* __restrict__ Z, int64_t ldz, int64_t Kp, int j,
+                                                               const T* __restrict__ w, T* __restrict__ out,
+                                                               KState* ks, unsigned long long* slots, double eta,
+                                                               int rows, int selective) {
+  constexpr int VN = VecN<T>::N;
+  extern __shared__ __align__(16) unsigned char col_dyn[];
+  __shared__ __align__(16) ColumnSmem<T> sm;
+  static_assert(offsetof(ColumnSmem<T>, upd) % 16 == 0, "16-byte accesses");
+  // uniform over the grid: done is raised only after the sums of every block have been seen below
+  if (ks->done) return;
+  T* xs = reinterpret_cast<T*>(col_dyn);
+  const int64_t r0 = (int64_t)blockIdx.x * rows;
+  const int64_t left = Kp - r0;
+  const int nch = left <= 0 ? 0 : (int)((left < rows ? left : rows) / VN);
+  const T* Zb = Z + r0;
+  T* outb = out + r0;
+  const int nc = j + 1;
+  const int64_t red = (int64_t)gridDim.x * COL_SUMS;  // slots of one reduction
+  unsigned long long* mine = slots + (j & 1) * 4 * red;
+  {
+    unsigned long long* other = slots + ((j + 1) & 1) * 4 * red + (int64_t)blockIdx.x * COL_SUMS;
+    for (int i = threadIdx.x; i < 4 * COL_SUMS; i += COL_NT) other[i / COL_SUMS * red + i % COL_SUMS] = COL_EMPTY;
+  }
+  for (int i = threadIdx.x; i < nc; i += COL_NT) sm.scale[i] = ks->s[i];
+  for (int ch = threadIdx.x; ch < nch; ch += COL_NT) {
+    T x[VN];
+    load_vec<T, VN>(w + r0 + ch * VN, x);
+    store_vec<T, VN>(xs + ch * VN, x);
+  }
+  __syncthreads();
+  column_project<T>(sm, xs, Zb, ldz, nc, true, nch);
+  if (!column_grid_sum<T>(sm, nc + 1, mine, ks)) return;
+  const double wnorm0 = sqrt(sm.dots[nc]);
+  if (!column_coefficients<T>(sm, j, true, ks)) return;
+  column_update<T>(sm, xs, outb, Zb, ldz, nc, nch);
+  if (selective) {
+    // keep the first pass when it cancelled less than DGKS_KAPPA (cgs_finalize's UPD1)
+    if (!column_grid_sum<T>(sm, 1, mine + red, ks)) return;
+    const double n1 = sqrt(sm.dots[0]);
+    if (isfinite(n1) && n1 > 0.0 && n1 >= DGKS_KAPPA * wnorm0) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ks->H[(j + 1) * MMAX + j] = n1;
+        ks->k = j + 1;
+        ks->s[j + 1] = 1.0 / n1;
+      }
+      return;
+    }
+  }
+  __syncthreads();
+  column_project<T>(sm, xs, Zb, ldz, nc, false, nch);
+  if (!column_grid_sum<T>(sm, nc, mine + 2 * red, ks)) return;
+  if (!column_coefficients<T>(sm, j, false, ks)) return;
+  column_update<T>(sm, xs, outb, Zb, ldz, nc, nch);
+  if (!column_grid_sum<T>(sm, 1, mine + 3 * red, ks)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const double hn = sqrt(sm.dots[0]);
+    ks->pass2 |= 1u << j;
+    ks->H[(j + 1) * MMAX + j] = hn;
+    ks->k = j + 1;
+    if (!isfinite(hn)) {
+      ks->err = 1;
+      ks->done = 1;
+    } else if (hn == 0.0 || hn <= eta * wnorm0) {
+      ks->done = 1;  // happy breakdown: K_{j+1} is invariant
+    } else {
+      ks->s[j + 1] = 1.0 / hn;
+    }
+  }
+}
+
+template <class T>
+ColumnPlan plan_cgs_column(int64_t Kp) {
+  ColumnPlan plan{0, 0};
+  int dev = 0, sms = 0, coop = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
+    return plan;
+  const int blocks = sms < COL_MAX_BLOCKS ? sms : COL_MAX_BLOCKS;
+  const int64_t rows = ((Kp + blocks - 1) / blocks + VPAD - 1) / VPAD * VPAD;
+  const int64_t bytes = rows * (int64_t)sizeof(T);
+  if (bytes > COLUMN_MAX_BYTES<T>) return plan;
+  // every block of the grid must be resident (they exchange sums): one per SM
+  if (cudaFuncSetAttribute(cgs_column_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)COLUMN_MAX_BYTES<T>) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cgs_column_kernel<T>, COL_NT, (size_t)bytes) !=
+          cudaSuccess ||
+      per_sm < 1) {
+    cudaGetLastError();
+    return plan;
+  }
+  plan.blocks = blocks;
+  plan.rows = (int)rows;
+  return plan;
+}
+
+template <class T>
+cudaError_t launch_cgs_column(const ColumnPlan& plan, const T* Z, int64_t ldz, int64_t Kp, int j, const T* w, T* out,
+                              KState* ks, unsigned long long* slots, double eta, bool selective, cudaStream_t st) {
+  if (j + 1 > MMAX || plan.blocks < 1) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3((unsigned)plan.blocks);
+  cfg.blockDim = dim3(COL_NT);
+  cfg.dynamicSmemBytes = (size_t)plan.rows * sizeof(T);
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, cgs_column_kernel<T>, Z, ldz, Kp, j, w, out, ks, slots, eta, plan.rows,
+                            selective ? 1 : 0);
+}
+
 // ------------------------------------------------ Gram-Schmidt of a partitioned run
 __global__ void __launch_bounds__(256) cgs_group_finalize_kernel(int mode, int j, KState* ks, double eta) {
   __shared__ double dots[MMAX + 2];
@@ -1114,7 +1515,9 @@ cudaError_t launch_cast(const Tin* x, Tout* y, int64_t n, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-__global__ void reset_kstate_kernel(KState* ks) {
+__global__ void reset_kstate_kernel(KState* ks, unsigned long long* slots, int n) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) slots[i] = COL_EMPTY;
+  if (blockIdx.x != 0) return;
   if (threadIdx.x == 0) {
     ks->k = 0;
     ks->done = 0;
@@ -1127,8 +1530,9 @@ __global__ void reset_kstate_kernel(KState* ks) {
   }
   for (int i = threadIdx.x; i < (MMAX + 1) * MMAX; i += blockDim.x) ks->H[i] = 0.0;
 }
-cudaError_t launch_reset_kstate(KState* ks, cudaStream_t st) {
-  reset_kstate_kernel<<<1, 256, 0, st>>>(ks);
+cudaError_t launch_reset_kstate(KState* ks, cudaStream_t st, unsigned long long* slots, const ColumnPlan* plan) {
+  const int n = slots ? 4 * COL_SUMS * plan->blocks : 0;  // the first of the two sets
+  reset_kstate_kernel<<<n > 0 ? 32 : 1, 256, 0, st>>>(ks, slots, n);
   return cudaGetLastError();
 }
 
@@ -1167,6 +1571,12 @@ template cudaError_t launch_cgs<double>(int, const double*, int64_t, int64_t, in
                                         double, cudaStream_t);
 template cudaError_t launch_cgs<float>(int, const float*, int64_t, int64_t, int, float*, float*, KState*, double*,
                                        double, cudaStream_t);
+template ColumnPlan plan_cgs_column<double>(int64_t);
+template ColumnPlan plan_cgs_column<float>(int64_t);
+template cudaError_t launch_cgs_column<double>(const ColumnPlan&, const double*, int64_t, int64_t, int, const double*,
+                                               double*, KState*, unsigned long long*, double, bool, cudaStream_t);
+template cudaError_t launch_cgs_column<float>(const ColumnPlan&, const float*, int64_t, int64_t, int, const float*,
+                                              float*, KState*, unsigned long long*, double, bool, cudaStream_t);
 template cudaError_t launch_krylov_axpy<double>(const double*, double*, double*, double*, const double*, int64_t,
                                                 int64_t, const KState*, cudaStream_t);
 template cudaError_t launch_krylov_axpy<float>(const double*, double*, float*, float*, const float*, int64_t,
