@@ -157,21 +157,8 @@ __global__ void __launch_bounds__(256) density_norm_kernel(const T* __restrict__
     if (s) r /= (double)s[e];
     acc += r * r;
   }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double b = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b += red[w];
-    partials[blockIdx.x] = b;
-    __threadfence();
-    last = atomicAdd(&ss->counter, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (last && threadIdx.x == 0) {
-    double b = 0;
-    for (unsigned i = 0; i < gridDim.x; ++i) b += __ldcg(partials + i);
-    const double rn = sqrt(b) / volume;
+  if (grid_reduce<SumOf>(acc, red, last, partials, &ss->counter)) {
+    const double rn = sqrt(acc) / volume;
     ss->res_norm = rn;
     if (!isfinite(rn)) ss->err = 1;
     if (ramp_n > 0) {
@@ -179,7 +166,6 @@ __global__ void __launch_bounds__(256) density_norm_kernel(const T* __restrict__
       const double b2 = 1.0 + (double)(ramp_n - 1) / (2 * p + 1);
       ss->cfl = fmin(cfl_max, fmax(a, b2));
     }
-    ss->counter = 0;
   }
 }
 
@@ -221,23 +207,7 @@ __global__ void __launch_bounds__(256) entropy_sum_kernel(const double* __restri
       acc += Wv[q] * s * s * r * r;
     }
   }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double b = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b += red[w];
-    partials[blockIdx.x] = b;
-    __threadfence();
-    last = atomicAdd(counter, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (last && threadIdx.x == 0) {
-    double b = 0;
-    for (unsigned i = 0; i < gridDim.x; ++i) b += __ldcg(partials + i);
-    *value = b;
-    *counter = 0;
-  }
+  if (grid_reduce<SumOf>(acc, red, last, partials, counter)) *value = acc;
 }
 
 cudaError_t launch_entropy_sum(const double* u, const double* Bv, const double* Wv, const double* sd, int64_t E, int nb,

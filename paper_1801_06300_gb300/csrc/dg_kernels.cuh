@@ -1848,9 +1848,12 @@ __global__ void __launch_bounds__(256) local_dt_kernel(DGData<T> d, const T* __r
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < d.E_loc; e += (int64_t)gridDim.x * blockDim.x) {
     const T isd = d.geo[GEO * e + O::ISD];
     double U[NV];
+#pragma unroll
     for (int v = 0; v < NV; ++v) {
-      T a = 0;
-      for (int j = 0; j < NB; ++j) a += d.Bc[j] * u[e * NV * NB + v * NB + j];
+      T a = 0, c[NB];
+      load_coeffs<T, NB>(u + (e * NV + v) * NB, c);
+#pragma unroll
+      for (int j = 0; j < NB; ++j) a += d.Bc[j] * c[j];
       U[v] = (double)(a * isd);
     }
     const double gam = (double)d.fs.gamma;
@@ -1870,23 +1873,7 @@ __global__ void __launch_bounds__(256) local_dt_kernel(DGData<T> d, const T* __r
     if (dte) dte[e] = (T)dt;
     mn = fmin(mn, dt);
   }
-  for (int o = 16; o > 0; o >>= 1) mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mn;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double b = red[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) b = fmin(b, red[w]);
-    partials[blockIdx.x] = b;
-    __threadfence();
-    last = atomicAdd(counter, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (last && threadIdx.x == 0) {
-    double b = DBL_MAX;
-    for (unsigned i = 0; i < gridDim.x; ++i) b = fmin(b, __ldcg(partials + i));
-    *dtmin = b;
-    *counter = 0;
-  }
+  if (grid_reduce<MinOf>(mn, red, last, partials, counter)) *dtmin = mn;
 }
 
 // ------------------------------------------------------------------ launchers

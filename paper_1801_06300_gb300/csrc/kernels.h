@@ -13,6 +13,51 @@ constexpr int MMAX = 32;        // largest Krylov dimension
 constexpr int RED_BLOCKS = 608;  // blocks of the streaming reductions (4 x 152 SMs)
 constexpr int VPAD = 64;        // vector length padding (elements)
 
+// One scalar per thread of a 256-thread block -> one value, in a fixed order, valid in thread 0
+// (red: 8 values).  Every thread calls it; between two calls on the same red stands a barrier.
+struct SumOf {
+  static constexpr double none = 0.0;
+  PCEXP_DEV static double of(double a, double b) { return a + b; }
+};
+struct MinOf {
+  static constexpr double none = 1.7976931348623157e308;  // DBL_MAX
+  PCEXP_DEV static double of(double a, double b) { return fmin(a, b); }
+};
+template <class Op>
+PCEXP_DEV double block_reduce(double a, double* red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a = Op::of(a, __shfl_xor_sync(0xffffffffu, a, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    a = threadIdx.x < 8 ? red[threadIdx.x] : Op::none;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) a = Op::of(a, __shfl_xor_sync(0xffffffffu, a, o));
+  }
+  return a;
+}
+// The whole grid's value: each block stores its own, the last one to arrive reduces them all, its
+// threads side by side (one thread doing so took 20 to 30 us of FP64 latency for 512 blocks, most of
+// the 30 us of the density norm and half of the 60 us of the time step on 131,072 triangles at
+// p = 3).  True in thread 0 of that block, with the value in a.
+template <class Op>
+PCEXP_DEV bool grid_reduce(double& a, double* red, bool& last, double* partials, unsigned* counter) {
+  a = block_reduce<Op>(a, red);
+  if (threadIdx.x == 0) {
+    partials[blockIdx.x] = a;
+    __threadfence();
+    last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return false;
+  a = Op::none;
+  for (unsigned i = threadIdx.x; i < gridDim.x; i += 256) a = Op::of(a, __ldcg(partials + i));
+  a = block_reduce<Op>(a, red);
+  if (threadIdx.x != 0) return false;
+  *counter = 0;
+  return true;
+}
+
 // Device-resident Arnoldi state.  V holds unnormalised vectors z_i with
 // v_i = s_i z_i; the Hessenberg matrix is row-major with leading dimension MMAX.
 struct KState {
