@@ -28,25 +28,11 @@ PCEXP_DEV double warp_sum(double a) {
   return a;
 }
 
-// Block reduction of NACC per-thread sums into partials[c * gridDim + block]; returns
-// true in the one block that finishes last, after it has reduced every column into
-// as->dots (fixed order).
-template <int NACC>
-__device__ bool reduce_last(double (&acc)[NACC], int nred, double* partials, AdjState* as) {
-  __shared__ double red[8][NACC];
+// Every block has stored its sums in partials[c * gridDim + block]; returns true in the one block
+// that finishes last, after it has reduced every column into as->dots (fixed order).
+__device__ bool finish_last(int nred, const double* partials, AdjState* as) {
   __shared__ bool last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int c = 0; c < NACC; ++c) {
-    const double a = warp_sum(acc[c]);
-    if (lane == 0) red[wid][c] = a;
-  }
-  __syncthreads();
-  for (int c = threadIdx.x; c < nred; c += blockDim.x) {
-    double a = 0;
-    for (int q = 0; q < 8; ++q) a += red[q][c];
-    partials[(int64_t)c * gridDim.x + blockIdx.x] = a;
-  }
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) last = atomicAdd(&as->counter, 1u) == gridDim.x - 1;
@@ -65,6 +51,25 @@ __device__ bool reduce_last(double (&acc)[NACC], int nred, double* partials, Adj
   __syncthreads();
   if (threadIdx.x == 0) as->counter = 0;
   return !as->group;
+}
+
+// The same from NACC per-thread sums.
+template <int NACC>
+__device__ bool reduce_last(double (&acc)[NACC], int nred, double* partials, AdjState* as) {
+  __shared__ double red[8][NACC];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int c = 0; c < NACC; ++c) {
+    const double a = warp_sum(acc[c]);
+    if (lane == 0) red[wid][c] = a;
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < nred; c += blockDim.x) {
+    double a = 0;
+    for (int q = 0; q < 8; ++q) a += red[q][c];
+    partials[(int64_t)c * gridDim.x + blockIdx.x] = a;
+  }
+  return finish_last(nred, partials, as);
 }
 
 // The finishing steps of the reductions, from the summed as->dots (called by the last block of
@@ -135,16 +140,24 @@ __global__ void __launch_bounds__(256) alpha_kernel(const double* __restrict__ Z
 // mode 0 (W2): wb = vbar_{j+1}/eta + (etabar - alpha/eta) s_{j+1} z_{j+1}   (zero when last)
 // mode 1 (W1): wb = win + sum_i cb2_i z_i
 // then dots_i = z_i . wb (i <= j) and hbar = Hbar[i][j] - s_i dots_i, cb = hbar s_i
-template <int NC>
+//
+// Bound by FP64 arithmetic on vectors that stay in L2.  A block walks tiles of 256 rows: a row per
+// thread for the update, then warp w takes the dot products of the columns w, w + 8, ... (NCW of
+// them) over the tile.  A thread so ends with NCW sums instead of one per column, whose warp sums
+// (five FP64 additions a column in each of the 8 warps) took longer than the sweep.  K = 147,456,
+// up to 8 / 16 / 32 columns: 16.5 / 27.7 / 53.7 -> 10.3 / 16.4 / 25.3 us.
+template <int NCW>
 __global__ void __launch_bounds__(256) upd_proj_kernel(int mode, const double* __restrict__ Z, int64_t ldz,
                                                        const double* __restrict__ Vb, const double* __restrict__ win,
                                                        double* __restrict__ wb, int64_t Kp, int j, int last_col,
                                                        const KState* ks, AdjState* as, double* __restrict__ partials) {
-  __shared__ double cc[MMAX + 1];
+  constexpr int TR = 256, U = 8;
+  __shared__ double cc[MMAX + U], xs[TR];
   __shared__ double ca, cbz;
   const int nc = j + 1;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (mode == 1)
-    for (int i = threadIdx.x; i < nc; i += blockDim.x) cc[i] = as->cb2[i];
+    for (int i = threadIdx.x; i < MMAX + U; i += blockDim.x) cc[i] = i < nc ? as->cb2[i] : 0.0;
   if (threadIdx.x == 0) {
     if (mode == 0 && !last_col) {
       const double eta = ks->H[(j + 1) * MMAX + j];
@@ -157,25 +170,50 @@ __global__ void __launch_bounds__(256) upd_proj_kernel(int mode, const double* _
     }
   }
   __syncthreads();
-  double acc[NC];
+  double acc[NCW];
 #pragma unroll
-  for (int c = 0; c < NC; ++c) acc[c] = 0.0;
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < Kp; r += (int64_t)gridDim.x * blockDim.x) {
-    double x;
-    if (mode == 0) {
-      x = (last_col ? 0.0 : ca * Vb[(int64_t)(j + 1) * ldz + r] + cbz * Z[(int64_t)(j + 1) * ldz + r]);
-    } else {
-      x = win[r];
+  for (int k = 0; k < NCW; ++k) acc[k] = 0.0;
+  for (int64_t t = (int64_t)blockIdx.x * TR; t < Kp; t += (int64_t)gridDim.x * TR) {
+    const int64_t r = t + threadIdx.x;
+    if (r < Kp) {
+      double x;
+      if (mode == 0) {
+        x = (last_col ? 0.0 : ca * Vb[(int64_t)(j + 1) * ldz + r] + cbz * Z[(int64_t)(j + 1) * ldz + r]);
+      } else {
+        x = win[r];
+        for (int c0 = 0; c0 < nc; c0 += U) {
+          double z[U];
 #pragma unroll
-      for (int c = 0; c < NC; ++c)
-        if (c < nc) x = fma(cc[c], Z[(int64_t)c * ldz + r], x);
+          for (int g = 0; g < U; ++g) z[g] = Z[(int64_t)(c0 + g < nc ? c0 + g : j) * ldz + r];
+#pragma unroll
+          for (int g = 0; g < U; ++g)
+            if (c0 + g < nc) x = fma(cc[c0 + g], z[g], x);
+        }
+      }
+      wb[r] = x;
+      xs[threadIdx.x] = x;
     }
-    wb[r] = x;
+    __syncthreads();
+    const int n = Kp - t < TR ? (int)(Kp - t) : TR;
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-      if (c < nc) acc[c] = fma(Z[(int64_t)c * ldz + r], x, acc[c]);
+    for (int k = 0; k < NCW; ++k) {
+      const int c = wid + 8 * k;
+      if (c < nc) {
+        const double* z = Z + (int64_t)c * ldz + t;
+#pragma unroll
+        for (int i = 0; i < TR / 32; ++i)
+          if (lane + 32 * i < n) acc[k] = fma(z[lane + 32 * i], xs[lane + 32 * i], acc[k]);
+      }
+    }
+    __syncthreads();
   }
-  if (reduce_last<NC>(acc, nc, partials, as)) finish_upd(mode, j, ks, as);
+#pragma unroll
+  for (int k = 0; k < NCW; ++k) {
+    const int c = wid + 8 * k;
+    const double a = warp_sum(acc[k]);
+    if (lane == 0 && c < nc) partials[(int64_t)c * gridDim.x + blockIdx.x] = a;
+  }
+  if (finish_last(nc, partials, as)) finish_upd(mode, j, ks, as);
 }
 
 // Vbar_i += w1 hb2_i - wb2 h2_i + w0 hb1_i - wb1 h1_i (i <= j);  wb0 = wb1 + sum_i cb1_i z_i
@@ -287,10 +325,10 @@ __global__ void __launch_bounds__(256) theta_sum_kernel(const double* __restrict
   if (threadIdx.x < 2) acc[threadIdx.x] += red[threadIdx.x][0];
 }
 
-template <int NC>
+template <int NCW>
 void launch_upd(int mode, const double* Z, int64_t ldz, const double* Vb, const double* win, double* wb, int64_t Kp,
                 int j, int last_col, const KState* ks, AdjState* as, double* partials, cudaStream_t st) {
-  upd_proj_kernel<NC><<<AB, 256, 0, st>>>(mode, Z, ldz, Vb, win, wb, Kp, j, last_col, ks, as, partials);
+  upd_proj_kernel<NCW><<<AB, 256, 0, st>>>(mode, Z, ldz, Vb, win, wb, Kp, j, last_col, ks, as, partials);
 }
 
 }  // namespace
@@ -328,9 +366,10 @@ cudaError_t launch_adj_upd(int mode, const double* Z, int64_t ldz, const double*
                            cudaStream_t st) {
   const int nc = j + 1;
   if (nc > MMAX) return cudaErrorInvalidValue;
-  if (nc <= 8) launch_upd<8>(mode, Z, ldz, Vb, win, wb, Kp, j, last_col, ks, as, partials, st);
-  else if (nc <= 16) launch_upd<16>(mode, Z, ldz, Vb, win, wb, Kp, j, last_col, ks, as, partials, st);
-  else launch_upd<32>(mode, Z, ldz, Vb, win, wb, Kp, j, last_col, ks, as, partials, st);
+  if (nc <= 8) launch_upd<1>(mode, Z, ldz, Vb, win, wb, Kp, j, last_col, ks, as, partials, st);
+  else if (nc <= 16) launch_upd<2>(mode, Z, ldz, Vb, win, wb, Kp, j, last_col, ks, as, partials, st);
+  else if (nc <= 24) launch_upd<3>(mode, Z, ldz, Vb, win, wb, Kp, j, last_col, ks, as, partials, st);
+  else launch_upd<4>(mode, Z, ldz, Vb, win, wb, Kp, j, last_col, ks, as, partials, st);
   return cudaGetLastError();
 }
 
