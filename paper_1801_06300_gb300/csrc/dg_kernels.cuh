@@ -324,14 +324,14 @@ PCEXP_DEV void load_early(const double* p, double (&x)[4]) {
   asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(x[2]), "=d"(x[3]) : "l"(p + 2));
 }
 
-template <class T, int D, int P, int MODE> struct ElemTile {
+template <class T, int D, int P, int MODE, int SL = 1> struct ElemTile {
   using O = Ord<D, P>;
-  static constexpr int ET = 32, NT = ET * O::NV;
+  static constexpr int ET = 32 / SL, NT = 32 * O::NV;
   static constexpr int RS = O::NVB | 1;  // odd row stride: lanes (elements) hit distinct banks
   static constexpr int ROWS = ET * RS * (MODE == ELEM_TANGENT ? 2 : 1);
   static constexpr int FLUX = P == 0 ? 0 : O::NQ * D * O::NV * ET;
   // FP32: the threads' own face-flux records, copied in while the volume part is computed
-  static constexpr bool AHEAD = sizeof(T) == 4;
+  static constexpr bool AHEAD = sizeof(T) == 4 && SL == 1;
   static constexpr int GV = GSTRIDE<T, D, P> / VECW<T>;  // 16-byte vectors of a record
   static constexpr int ROWS4 = (ROWS + 3) / 4 * 4;       // the records start on a 16-byte boundary
   static constexpr int RECS = AHEAD ? O::NF * GV * NT * VECW<T> : 0;
@@ -359,13 +359,22 @@ template <class T, int D, int P, int MODE> struct ElemTile {
 // the flux derivative from u), FP32 131,072 triangles at p = 3 111 -> 32 us (lanes sharing an
 // element's test functions), FP64 20^3 cubes at p = 2 485 -> 427 us (stored D nv x nv Jacobians);
 // the residual's: FP64 24^3 cubes at p = 2 1117 -> 717 us.
-template <class T, int D, int P, int MODE, bool PADG>
-__global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P, MODE>::MINB)
+//
+// SL > 1: a block owns 32 / SL elements and SL lanes share one.  They split the points of phase 1 and
+// of the projection (its sums meet by shuffles) and the rows (test functions) of the lift and the
+// combination, so a tile takes about a third of the time at SL = 4 and four times the SMs work on a
+// small mesh; the tables are then read at SL addresses per warp and the splits leave lanes idle,
+// so the total work grows.  Per launch of the FP64 Krylov J v at p = 2: 14.5 -> 7.9 us on 1,152
+// triangles, but 24.0 -> 28.4 us on 6,144; residual calls on 4,608 triangles 77 -> 70 us and on
+// 10,082 105 -> 112 us.  FP32: 6.3 -> 5.8 us on 162 tetrahedra, 71 -> 76 us a J v call on 20,402
+// triangles.  Hence the limit of 32 elements per SM (one tile of 32 per SM).
+template <class T, int D, int P, int MODE, bool PADG, int SL>
+__global__ void __launch_bounds__(ElemTile<T, D, P, MODE, SL>::NT, ElemTile<T, D, P, MODE, SL>::MINB)
     elem_op_kernel(DGData<T> d, const T* __restrict__ u, const T* __restrict__ du, const T* __restrict__ pts,
                    const T* __restrict__ G, T* __restrict__ out, const T* __restrict__ escale,
                    const int* __restrict__ skip, const double* __restrict__ oscale) {
   using O = Ord<D, P>;
-  using L = ElemTile<T, D, P, MODE>;
+  using L = ElemTile<T, D, P, MODE, SL>;
   using X = TabLayout<D, P>;
   constexpr int NB = O::NB, NQ = O::NQ, NFQ = O::NFQ, NV = O::NV, NVB = O::NVB, GEO = O::GEO, NF = O::NF;
   constexpr int NPERM = O::NPERM, ET = L::ET, RS = L::RS, NB1 = X::NB1;
@@ -380,7 +389,8 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P,
   const int ne = (int)((d.E - e0) < ET ? (d.E - e0) : ET);
   // the warp's index through a shuffle, so that it is known to be uniform (table loads by it)
   const int lane = threadIdx.x & 31, w = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
-  const int64_t e = e0 + (lane < ne ? lane : 0);  // lanes past the last element repeat element e0; discarded
+  const int tl = SL == 1 ? lane : lane % ET, sub = SL == 1 ? 0 : lane / ET;
+  const int64_t e = e0 + (tl < ne ? tl : 0);  // lanes past the last element repeat element e0; discarded
   int slots[NF];
   if constexpr (NF == 4) {
     const int4 s4 = __ldg(reinterpret_cast<const int4*>(d.ef) + e);
@@ -392,12 +402,13 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P,
 #pragma unroll
     for (int k = 0; k < NF; ++k) slots[k] = __ldg(d.ef + NF * e + k);
   }
-  // the tile's rows: ET * NVB = NT * NB values, all loads issued before the first store
+  // the tile's rows: ET * NVB = NT * NB / SL values, all loads issued before the first store
   {
     const T* src = (MODE == ELEM_FLUX ? u : du) + e0 * NVB;
-    T x[NB], y[MODE == ELEM_TANGENT ? NB : 1];
+    constexpr int KR = (NB + SL - 1) / SL;
+    T x[KR], y[MODE == ELEM_TANGENT ? KR : 1];
 #pragma unroll
-    for (int k = 0; k < NB; ++k) {
+    for (int k = 0; k < KR; ++k) {
       const int i = threadIdx.x + k * L::NT;
       x[k] = i < ne * NVB ? src[i] : T(0);
       if constexpr (MODE == ELEM_TANGENT) y[k] = i < ne * NVB ? u[e0 * NVB + i] : T(0);
@@ -413,7 +424,7 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P,
       cp_async_commit();
     }
 #pragma unroll
-    for (int k = 0; k < NB; ++k) {
+    for (int k = 0; k < KR; ++k) {
       const int i = threadIdx.x + k * L::NT, r = i / NVB * RS + i % NVB;
       if (i < ne * NVB) {
         rows[r] = x[k];
@@ -424,21 +435,22 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P,
   T ge[GEO];
   load_row<T, GEO, true>(d.geo + GEO * e, ge);
   const T isd = ge[O::ISD];
-  constexpr int PP = P == 0 ? 1 : (NQ + NV - 1) / NV;  // points per warp
+  constexpr int WS = NV * SL, PP = P == 0 ? 1 : (NQ + WS - 1) / WS;  // shares of the points, points per share
+  const int q0 = w * SL + sub, qc = WS <= NQ || q0 < NQ ? q0 : 0;      // this lane's first point (in range: qc)
   T pv[MODE == ELEM_STORED ? PP : 1][4];
   if constexpr (MODE == ELEM_STORED && P > 0) {
 #pragma unroll
-    for (int i = 0; i < PP; ++i) load_early(pts + ((int64_t)(w + i * NV < NQ ? w + i * NV : w) * d.E + e) * 4, pv[i]);
+    for (int i = 0; i < PP; ++i) load_early(pts + ((int64_t)(q0 + i * WS < NQ ? q0 + i * WS : qc) * d.E + e) * 4, pv[i]);
   }
   __syncthreads();
-  const int el = lane < ne ? lane : 0;
+  const int el = tl < ne ? tl : 0;
   if constexpr (P > 0) {
     const T gm = d.fs.gamma - T(1);
     T Ai[D][D];
 #pragma unroll
     for (int k = 0; k < D * D; ++k) Ai[k / D][k % D] = ge[k];
-    // traces of this lane's element at the warp's points q = w, w + NV, ... (the last may be past NQ:
-    // it repeats the warp's first point and is not stored)
+    // traces of this lane's element at its points q0, q0 + WS, ... (the last may be past NQ: it repeats
+    // the first point and is not stored)
     T t[PP][NV], s[MODE == ELEM_TANGENT ? PP : 1][NV];
     const T* ra = rows + el * RS;
 #pragma unroll
@@ -455,7 +467,7 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P,
         if constexpr (MODE == ELEM_TANGENT) c2 = ra[ET * RS + v * NB + j];
 #pragma unroll
         for (int i = 0; i < PP; ++i) {
-          const int q = w + i * NV < NQ ? w + i * NV : w;
+          const int q = q0 + i * WS < NQ ? q0 + i * WS : qc;
           const T b = tab[X::BV + q * NB + j];
           t[i][v] = fma(b, c, t[i][v]);
           if constexpr (MODE == ELEM_TANGENT) s[i][v] = fma(b, c2, s[i][v]);
@@ -464,8 +476,8 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P,
     }
 #pragma unroll
     for (int i = 0; i < PP; ++i) {
-      const int q = w + i * NV;
-      if (q >= NQ) break;  // warp-uniform
+      const int q = q0 + i * WS;
+      if (q >= NQ) break;
       T vel[D], H, k2 = T(0);
       T F[D][NV];
       if constexpr (MODE == ELEM_STORED) {
@@ -540,15 +552,17 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P,
 #pragma unroll
       for (int dd = 0; dd < D; ++dd)
 #pragma unroll
-        for (int v = 0; v < NV; ++v) sF[((q * D + dd) * NV + v) * ET + lane] = F[dd][v];
+        for (int v = 0; v < NV; ++v) sF[((q * D + dd) * NV + v) * ET + tl] = F[dd][v];
     }
     __syncthreads();
   }
   // phase 2: variable w of this lane's element
   if constexpr (L::AHEAD) cp_async_wait_all();  // a thread reads its own copies only
-  T acc[NB];
+  constexpr int NR = (NB + SL - 1) / SL;  // rows sub, sub + SL, ... of this lane (past NB: repeated, not stored)
+  auto row = [&](int i) { return SL == 1 ? i : (i * SL + sub < NB ? i * SL + sub : NB - 1); };
+  T acc[NR];
 #pragma unroll
-  for (int i = 0; i < NB; ++i) acc[i] = T(0);
+  for (int i = 0; i < NR; ++i) acc[i] = T(0);
 #pragma unroll
   for (int k = 0; k < NF; ++k) {
     const int fs = slots[k];
@@ -576,23 +590,28 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P,
       const T* tb = d.BfP + ((k * NPERM + slot_perm(fs)) * NFQ) * PADV<T, NB>;
 #pragma unroll
       for (int q = 0; q < NFQ; ++q) {
-        T row[PADV<T, NB>];
-        load_row<T, PADV<T, NB>, true>(tb + q * PADV<T, NB>, row);
+        if constexpr (SL == 1) {
+          T tr[PADV<T, NB>];
+          load_row<T, PADV<T, NB>, true>(tb + q * PADV<T, NB>, tr);
 #pragma unroll
-        for (int i = 0; i < NB; ++i) acc[i] = fma(row[i], x[q], acc[i]);
+          for (int i = 0; i < NR; ++i) acc[i] = fma(tr[i], x[q], acc[i]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < NR; ++i) acc[i] = fma(__ldg(tb + q * PADV<T, NB> + row(i)), x[q], acc[i]);
+        }
       }
     } else {
 #pragma unroll
       for (int q = 0; q < NFQ; ++q)
 #pragma unroll
-        for (int i = 0; i < NB; ++i) acc[i] = fma(tab[X::BF + (k * NFQ + q) * NB + i], x[q], acc[i]);
+        for (int i = 0; i < NR; ++i) acc[i] = fma(tab[X::BF + (k * NFQ + q) * NB + row(i)], x[q], acc[i]);
     }
   }
   // the lift carries 1/sqrt|det|; the volume term sqrt|det| (flux) or nothing (the factors of the
   // trace and the test cancel in the derivative)
   const T ls = MODE == ELEM_FLUX ? isd * isd : isd;
 #pragma unroll
-  for (int i = 0; i < NB; ++i) acc[i] *= ls;
+  for (int i = 0; i < NR; ++i) acc[i] *= ls;
   if constexpr (P > 0) {
 #pragma unroll
     for (int dd = 0; dd < D; ++dd) {
@@ -600,12 +619,25 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P,
 #pragma unroll
       for (int k = 0; k < NB1; ++k) m[k] = T(0);
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        const T f = sF[((q * D + dd) * NV + w) * ET + lane];
+      for (int i = 0; i < (NQ + SL - 1) / SL; ++i) {
+        const bool in = NQ % SL == 0 || i * SL + sub < NQ;
+        const int q = in ? i * SL + sub : 0;
+        const T f = in ? sF[((q * D + dd) * NV + w) * ET + tl] : T(0);
 #pragma unroll
         for (int k = 0; k < NB1; ++k) m[k] = fma(tab[X::WM + q * NB1 + k], f, m[k]);
       }
-      combine_modes<T, D, P, 1>(tab + X::CM + dd * NB * NB1, m, acc);
+      if constexpr (SL == 1) {
+        combine_modes<T, D, P, 1>(tab + X::CM + dd * NB * NB1, m, acc);
+      } else {
+#pragma unroll
+        for (int k = 0; k < NB1; ++k)
+#pragma unroll
+          for (int o = ET; o < 32; o *= 2) m[k] += __shfl_xor_sync(0xffffffffu, m[k], o);
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+#pragma unroll
+          for (int k = 0; k < NB1; ++k) acc[i] = fma(tab[X::CM + (dd * NB + row(i)) * NB1 + k], m[k], acc[i]);
+      }
     }
   }
   T sc = oscale ? (T)*oscale : T(1);
@@ -614,27 +646,37 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE>::NT, ElemTile<T, D, P,
     const T so = MODE == ELEM_FLUX ? isd : T(1);
     const T* ra = rows + el * RS;
 #pragma unroll
-    for (int i = 0; i < NB; ++i) {
+    for (int i = 0; i < NR; ++i) {
       T m[D];
 #pragma unroll
-      for (int k = 0; k < D; ++k) m[k] = ra[(1 + k) * NB + i];
+      for (int k = 0; k < D; ++k) m[k] = ra[(1 + k) * NB + row(i)];
       acc[i] += rot_source<T, D>(d.om, m, w - 1) * so;
     }
   }
   if (d.rot) __syncthreads();  // the rows have been read before they are overwritten
   if constexpr (MODE == ELEM_FLUX) sc *= ge[O::SD];
 #pragma unroll
-  for (int i = 0; i < NB; ++i) rows[lane * RS + w * NB + i] = acc[i] * sc;
+  for (int i = 0; i < NR; ++i)
+    if (SL == 1 || i * SL + sub < NB) rows[tl * RS + w * NB + row(i)] = acc[i] * sc;
   __syncthreads();
   for (int i = threadIdx.x; i < ne * NVB; i += L::NT) out[e0 * NVB + i] = rows[i / NVB * RS + i % NVB];
 }
 
+// Elements per SM up to which four lanes share an element (measured, see elem_op_kernel).
+constexpr int FEW_ELEMENTS = 32;
 template <class T, int D, int P, int MODE, bool PADG>
 static void elem_op_launch(const DGData<T>& d, const T* u, const T* du, const T* pts, const T* G, T* out,
                            const T* escale, const int* skip, const double* oscale, cudaStream_t st) {
-  using L = ElemTile<T, D, P, MODE>;
-  elem_op_kernel<T, D, P, MODE, PADG><<<(unsigned)((d.E + L::ET - 1) / L::ET), L::NT, L::BYTES, st>>>(
-      d, u, du, pts, G, out, escale, skip, oscale);
+  auto run = [&](auto lanes) {
+    constexpr int SL = decltype(lanes)::value;
+    using L = ElemTile<T, D, P, MODE, SL>;
+    elem_op_kernel<T, D, P, MODE, PADG, SL><<<(unsigned)((d.E + L::ET - 1) / L::ET), L::NT, L::BYTES, st>>>(
+        d, u, du, pts, G, out, escale, skip, oscale);
+  };
+  if constexpr (P > 0) {
+    if (d.E <= FEW_ELEMENTS * (int64_t)sm_count()) return run(std::integral_constant<int, 4>());
+  }
+  run(std::integral_constant<int, 1>());
 }
 
 template <class T, int D, int P>
@@ -688,11 +730,11 @@ cudaError_t upload_tables_p(const double* Bv, const double* Dv, const double* Wv
   auto allow = [&](auto kernel, size_t bytes) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   };
-  allow(elem_op_kernel<T, D, P, ELEM_FLUX, true>, ElemTile<T, D, P, ELEM_FLUX>::BYTES);
-  allow(elem_op_kernel<T, D, P, ELEM_TANGENT, true>, ElemTile<T, D, P, ELEM_TANGENT>::BYTES);
-  allow(elem_op_kernel<T, D, P, ELEM_STORED, true>, ElemTile<T, D, P, ELEM_STORED>::BYTES);
+  allow(elem_op_kernel<T, D, P, ELEM_FLUX, true, 1>, ElemTile<T, D, P, ELEM_FLUX>::BYTES);
+  allow(elem_op_kernel<T, D, P, ELEM_TANGENT, true, 1>, ElemTile<T, D, P, ELEM_TANGENT>::BYTES);
+  allow(elem_op_kernel<T, D, P, ELEM_STORED, true, 1>, ElemTile<T, D, P, ELEM_STORED>::BYTES);
   if constexpr (std::is_same<T, double>::value)
-    allow(elem_op_kernel<T, D, P, ELEM_FLUX, false>, ElemTile<T, D, P, ELEM_FLUX>::BYTES);
+    allow(elem_op_kernel<T, D, P, ELEM_FLUX, false, 1>, ElemTile<T, D, P, ELEM_FLUX>::BYTES);
   return e;
 }
 
@@ -924,7 +966,9 @@ __global__ void __launch_bounds__(256) face_apply_kernel(DGData<T> d, const T* _
 // against the warps in flight: with 70 registers (three blocks per SM) it took 340 us, with two
 // points per thread 366.  Boundary points, whose ghost state's derivative may hold powers, keep
 // their nv x nv block.  FP64 keeps blocks: there the arithmetic is the bound and a block product
-// (50 FMAs) is the cheaper form.
+// (50 FMAs) is the cheaper form.  On triangles a block has 32 values and the gather of dv's rows
+// through L1 is the bound: 28.6 us with blocks, 28.8 with records (131,072 triangles at p = 3), so
+// blocks stay.
 template <int D, int P>
 __global__ void __launch_bounds__(256, 4) face_record_kernel(DGData<float> d, const float* __restrict__ rec,
                                                           const float* __restrict__ dv, float* __restrict__ G,

@@ -13,6 +13,14 @@ constexpr int MMAX = 32;        // largest Krylov dimension
 constexpr int RED_BLOCKS = 608;  // blocks of the streaming reductions (4 x 152 SMs)
 constexpr int VPAD = 64;        // vector length padding (elements)
 
+// SMs of the current device
+inline int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    n = 0;
+  return n > 0 ? n : 152;
+}
+
 // One scalar per thread of a 256-thread block -> one value, in a fixed order, valid in thread 0
 // (red: 8 values).  Every thread calls it; between two calls on the same red stands a barrier.
 struct SumOf {
