@@ -19,6 +19,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -165,11 +166,11 @@ def algorithmic_bytes(kind, T, K, E, F, dim, p, m, face_jacobians=True, gs=None)
     g_elem = E * (geo * T + 4 * nf)    # inverse map, sqrt(det), h, 1/sqrt(det); face slots
     G = F * nfq * nv * T
     avg_j = (m - 1) / 2.0              # mean column index over one Arnoldi process
-    if T == 8:   # FP64: the volume part applies the stored point Jacobians
-        jvp_elem = 2 * K * T + dim * nv * nv * E * nq * T + E * (T + 4 * nf) + G
-    else:        # FP32-mixed: flux tangents recomputed from the linearisation state
-        jvp_elem = 3 * K * T + g_elem + G
-    if face_jacobians:  # face point Jacobians at u_n (both sides) applied to the traces of v
+    # the volume part derives the fluxes from four stored values per volume point
+    jvp_elem = 2 * K * T + 4 * E * nq * T + g_elem + G
+    if face_jacobians and T == 4 and dim == 3:  # 16 values per face point, the derivative recomputed
+        jvp_face = K * T + 16 * F * nfq * T + g_face + G
+    elif face_jacobians:  # face point Jacobians at u_n (both sides) applied to the traces of v
         jvp_face = K * T + 2 * nv * nv * F * nfq * T + F * 12 + G
     else:               # Riemann-flux tangents recomputed from the traces of u_n and v
         jvp_face = 2 * K * T + g_face + G
@@ -181,6 +182,7 @@ def algorithmic_bytes(kind, T, K, E, F, dim, p, m, face_jacobians=True, gs=None)
         "residual_elem": 2 * K * T + g_elem + G,
         "cgs_proj": (avg_j + 2) * K * T,
         "cgs_upd_proj": (avg_j + 3) * K * T,
+        "cgs_column": (avg_j + 3) * K * T,
         "cgs_upd_norm": (gs[0] * (gs[1] + 3) if gs else avg_j + 3) * K * T,
         "cgs_upd1": (avg_j + 3) * K * T,
         "cgs_proj2": (gs[0] * (gs[1] + 2) if gs else avg_j + 2) * K * T,
@@ -190,22 +192,24 @@ def algorithmic_bytes(kind, T, K, E, F, dim, p, m, face_jacobians=True, gs=None)
 def algorithmic_flops(kind, K, E, F, dim, p, m, T=8, gs=None):
     """Floating-point operations per launch of a kernel class (an FMA counts 2).
 
-    jvp_elem, FP64 (stored point Jacobians): per element, nq points x (trace nv nb + Jacobian
-    d nv^2) FMA and nv nb outputs x (volume d nq + lift nf nfq) FMA.  FP32-mixed (flux
-    tangents): nq points x (traces of u_n and v, 2 nv nb; mapping of the flux tangent to
-    reference directions, d^2 nv) FMA and the same test and lift; the Euler-flux tangent itself
-    (a few hundred operations per point) is not counted, so the fraction is a lower bound.
-    jvp_face: per face point 2 nv nb trace + 2 nv^2 FMA; CGS kernels: per unknown and column,
-    1 (projection) or 2 (update + projection) FMA, averaged over the columns of one Arnoldi
-    process."""
+    jvp_elem: per element, nq points x trace nv nb FMA and per variable the projection of d nq
+    fluxes on the nb1 functions of degree p - 1, their combination (d nb nb1) and the lift
+    (nb nf nfq); the flux derivative itself (about 40 operations per point) is not counted, so
+    the fraction is a lower bound.  jvp_face: per face point 2 nv nb trace + 2 nv^2 FMA (the
+    FP32 form on tetrahedra recomputes the block's product with about 210); CGS kernels: per
+    unknown and column, 1 (projection) or 2 (update + projection) FMA, averaged over the
+    columns of one Arnoldi process; a whole column: projection and update of one pass, and of
+    the second where it runs."""
     nb, nq, nfq, nv, nf = shape(dim, p)
+    nb1 = math.comb(p - 1 + dim, dim) if p > 0 else 0
     nc = (m + 1) / 2.0
-    vol = nq * (nv * nb + dim * nv * nv) if T == 8 else nq * (2 * nv * nb + dim * dim * nv)
+    passes = 1 + gs[0] if gs else 2
     fma = {
-        "jvp_elem": E * (vol + nv * nb * (dim * nq + nf * nfq)),
+        "jvp_elem": E * nv * (nq * nb + dim * nb1 * (nq + nb) + nb * nf * nfq),
         "jvp_face": F * nfq * (2 * nv * nb + 2 * nv * nv),
         "cgs_proj": K * (nc + 1),
         "cgs_upd_proj": K * 2 * nc,
+        "cgs_column": K * passes * (2 * nc + 1),
         "cgs_upd_norm": K * (gs[0] * (gs[1] + 2) if gs else nc + 1),
         "cgs_upd1": K * (nc + 1),
         "cgs_proj2": K * (gs[0] * (gs[1] + 2) if gs else nc + 1),
@@ -216,9 +220,7 @@ def algorithmic_flops(kind, K, E, F, dim, p, m, T=8, gs=None):
 # DRAM bytes (read + write) per launch from one ncu capture of the same kernel on the same
 # workload, keyed (workload, element bytes, kernel class); an entry is dropped when its
 # kernel changes.  The summaries under profiles/ give the commands.
-NCU_TRAFFIC = {
-    ("vortex3d", 4, "jvp_elem"): (608250112, "profiles/traffic_vortex3d_48_p2_m30_fp32.md"),
-}
+NCU_TRAFFIC = {}
 
 
 def fp64_peak(capi):

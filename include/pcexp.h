@@ -229,7 +229,7 @@ int pcexp_arnoldi(pcexp_ctx* ctx, const double* U, const double* b, int m,
  * matrix H (row-major, leading dimension ldh; host arrays), evaluated on the
  * device in FP64 from the exponential of the augmented matrix
  * [[dt H, e_1, 0], [0, 0, 1], [0, 0, 0]] by scaling and squaring with a
- * diagonal Pade approximant.  phi2 may be NULL.  k <= PCEXP_MAX_KRYLOV. */
+ * Taylor polynomial.  phi2 may be NULL.  k <= PCEXP_MAX_KRYLOV. */
 int pcexp_phi(pcexp_ctx* ctx, const double* H, int k, int ldh, double dt,
               double* phi1, double* phi2);
 
