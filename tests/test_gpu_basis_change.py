@@ -8,7 +8,9 @@ import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-MESHES = [("tri", 2, 2), ("tri", 8, 4), ("tri", 11, 3), ("tet", 2, 0), ("tet", 3, 0)]  # 8, 64, 66, 48, 162 elements
+# 8, 64, 66, 2432, 2448, 48, 162, 1296, 2058 elements (an entry per thread up to 9728 rows, a row above)
+MESHES = [("tri", 2, 2), ("tri", 8, 4), ("tri", 11, 3), ("tri", 38, 32), ("tri", 51, 24),
+          ("tet", 2, 0), ("tet", 3, 0), ("tet", 6, 0), ("tet", 7, 0)]
 
 
 def mesh_of(kind, nx, ny):
