@@ -78,7 +78,9 @@ __global__ void __launch_bounds__(QBlocks<D, P>::NT) change_basis_kernel(const T
 
 // The same with a thread per entry (src and dst distinct): a chain of at most 6 FMAs instead of the 46
 // of a row (p = 2 on tetrahedra), at 30% more FP64 instructions.  162 tetrahedra: 6.4 -> 2.2 us a
-// launch; residual calls (two conversions) on 1,152 triangles at p = 2 in FP64 58.9 -> 55.9 us.
+// launch; residual calls (two conversions) on 6,000 tetrahedra at p = 2 in FP32-mixed 75 -> 64 us,
+// where the row form on 2,058 was slower than a thread per output of the full matrix (64 against 60
+// us, now 57).  At 256 rows per SM both forms are bound by the FP64 pipe.
 template <class Tin, class Tout, int D, int P, bool TRANS>
 __global__ void __launch_bounds__(256) change_basis_entry_kernel(const Tin* __restrict__ src, Tout* __restrict__ dst,
                                                                  float* __restrict__ dst2,
@@ -112,7 +114,7 @@ __global__ void __launch_bounds__(256) change_basis_entry_kernel(const Tin* __re
 }
 
 // Rows per SM up to which the entry form is the faster one (measured above).
-constexpr int64_t ENTRY_ROWS = 64;
+constexpr int64_t ENTRY_ROWS = 256;
 
 template <class Tin, class Tout, int D, int P, bool TRANS>
 static cudaError_t change_basis_p(const Tin* src, Tout* dst, float* dst2, const double* Q, int64_t E, cudaStream_t st) {

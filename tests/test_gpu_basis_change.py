@@ -8,9 +8,9 @@ import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-# 8, 64, 66, 2432, 2448, 48, 162, 1296, 2058 elements (an entry per thread up to 9728 rows, a row above)
-MESHES = [("tri", 2, 2), ("tri", 8, 4), ("tri", 11, 3), ("tri", 38, 32), ("tri", 51, 24),
-          ("tet", 2, 0), ("tet", 3, 0), ("tet", 6, 0), ("tet", 7, 0)]
+# 8, 64, 66, 9728, 9856, 48, 162, 6000, 7986 elements (an entry per thread up to 38,912 rows, a row above)
+MESHES = [("tri", 2, 2), ("tri", 8, 4), ("tri", 11, 3), ("tri", 76, 64), ("tri", 77, 64),
+          ("tet", 2, 0), ("tet", 3, 0), ("tet", 10, 0), ("tet", 11, 0)]
 
 
 def mesh_of(kind, nx, ny):
