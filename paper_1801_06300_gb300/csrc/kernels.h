@@ -58,6 +58,7 @@ PCEXP_DEV bool grid_reduce(double& a, double* red, bool& last, double* partials,
   }
   __syncthreads();
   if (!last) return false;
+  __threadfence();  // every thread reads the other blocks' values: ordered after the atomic that saw them counted
   a = Op::none;
   for (unsigned i = threadIdx.x; i < gridDim.x; i += 256) a = Op::of(a, __ldcg(partials + i));
   a = block_reduce<Op>(a, red);
