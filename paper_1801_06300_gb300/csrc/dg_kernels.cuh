@@ -236,11 +236,13 @@ __global__ void __launch_bounds__(256) face_kernel(DGData<T> d, const T* __restr
 //   Wm [nq][nb1]       w_q phi_k at the volume points, k < nb1 (the basis of order p - 1)
 //   Cm [D][nb][nb1]    <d phi_i / d xi_d, phi_k>: the gradients of the basis in the basis of order p - 1
 //   Bf [nf][nfq][nb]   phi_j at the face points, the element's own face-vertex order
+//   Ch, Cl [D][nb]     int d phi_i / d xi_d (the test of a constant) and what its rounding lost
 template <int D, int P> struct TabLayout {
   using O = Ord<D, P>;
   static constexpr int NB1 = P == 0 ? 0 : Ord<D, P == 0 ? 0 : P - 1>::NB;
   static constexpr int BV = 0, WM = BV + O::NQ * O::NB, CM = WM + O::NQ * NB1, BF = CM + D * O::NB * NB1;
-  static constexpr int N = BF + O::NF * O::NFQ * O::NB;
+  static constexpr int CH = BF + O::NF * O::NFQ * O::NB, CL = CH + D * O::NB;
+  static constexpr int N = CL + D * O::NB;
 };
 template <class T, int D, int P> __constant__ T c_tab[TabLayout<D, P>::N];
 
@@ -337,7 +339,7 @@ template <class T, int D, int P, int MODE, int SL = 1> struct ElemTile {
   static constexpr int RECS = AHEAD ? O::NF * GV * NT * VECW<T> : 0;
   static constexpr size_t BYTES = sizeof(T) * (size_t)(ROWS4 + RECS + FLUX);
   // blocks per SM the registers are bounded for (the shared memory allows as many or more)
-  static constexpr int MINB = sizeof(T) == 4 ? (D == 3 ? 4 : 5) : (D == 3 ? 2 : 3);
+  static constexpr int MINB = sizeof(T) == 4 ? (D == 3 ? 4 : MODE == ELEM_STORED ? 7 : 5) : (D == 3 ? 2 : 3);
 };
 
 // A block owns 32 elements and has a warp per variable.
@@ -359,6 +361,19 @@ template <class T, int D, int P, int MODE, int SL = 1> struct ElemTile {
 // the flux derivative from u), FP32 131,072 triangles at p = 3 111 -> 32 us (lanes sharing an
 // element's test functions), FP64 20^3 cubes at p = 2 485 -> 427 us (stored D nv x nv Jacobians);
 // the residual's: FP64 24^3 cubes at p = 2 1117 -> 717 us.
+//
+// FP32 sums: one chain of FMAs per entry through all faces, points and directions adds the rounding
+// of up to 50 terms, and R is the small difference of its volume and face terms.  So every face and
+// every direction has a sum of its own and the sums are added (PARTS); the projection of the
+// derivatives runs in two chains (HALVES); and the projection of R's fluxes takes their differences
+// from the first point's, the test of that constant coming from a table rounded to twice FP32
+// (SHIFT: a smooth flux loses only the rounding of its variation; on the derivatives along rough
+// Krylov vectors it would add 5 to 8%).  Error against 64 bits, one chain -> this (two to four lanes
+// sharing the sums, as the kernels before this one did): a step on 48^3 cubes at p = 2 1.85e-7 ->
+// 1.31e-7 (1.47e-7), on 131,072 triangles at p = 3 2.14e-7 -> 1.48e-7 (1.69e-7); R on 24^3 cubes at
+// p = 2 8.5e-5 -> 7.2e-5 (7.6e-5).  It costs 0.2 of 277 us per J v on the cubes, 1.5 of 37.5 us on
+// the triangles (the second chain's registers; seven blocks per SM instead of five keep it there: 41
+// us with five) and 14 of 266 us per R on the cubes.  FP64 keeps one chain: its pipe is the bound.
 //
 // SL > 1: a block owns 32 / SL elements and SL lanes share one.  They split the points of phase 1 and
 // of the projection (its sums meet by shuffles) and the rows (test functions) of the lift and the
@@ -559,6 +574,8 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE, SL>::NT, ElemTile<T, D
   // phase 2: variable w of this lane's element
   if constexpr (L::AHEAD) cp_async_wait_all();  // a thread reads its own copies only
   constexpr int NR = (NB + SL - 1) / SL;  // rows sub, sub + SL, ... of this lane (past NB: repeated, not stored)
+  // the order of the FP32 sums (see above)
+  constexpr bool PARTS = sizeof(T) == 4, SHIFT = PARTS && MODE == ELEM_FLUX, HALVES = PARTS && MODE != ELEM_FLUX;
   auto row = [&](int i) { return SL == 1 ? i : (i * SL + sub < NB ? i * SL + sub : NB - 1); };
   T acc[NR];
 #pragma unroll
@@ -585,6 +602,9 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE, SL>::NT, ElemTile<T, D
       }
     }
     face_fluxes<T, D, P, GS>(r, fs, x);
+    T face[NR];
+#pragma unroll
+    for (int i = 0; i < NR; ++i) face[i] = PARTS ? T(0) : acc[i];
     if constexpr (D == 3 && P == 1) {
       // the collapsed face rule is not symmetric: the table of the side's vertex permutation
       const T* tb = d.BfP + ((k * NPERM + slot_perm(fs)) * NFQ) * PADV<T, NB>;
@@ -594,18 +614,20 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE, SL>::NT, ElemTile<T, D
           T tr[PADV<T, NB>];
           load_row<T, PADV<T, NB>, true>(tb + q * PADV<T, NB>, tr);
 #pragma unroll
-          for (int i = 0; i < NR; ++i) acc[i] = fma(tr[i], x[q], acc[i]);
+          for (int i = 0; i < NR; ++i) face[i] = fma(tr[i], x[q], face[i]);
         } else {
 #pragma unroll
-          for (int i = 0; i < NR; ++i) acc[i] = fma(__ldg(tb + q * PADV<T, NB> + row(i)), x[q], acc[i]);
+          for (int i = 0; i < NR; ++i) face[i] = fma(__ldg(tb + q * PADV<T, NB> + row(i)), x[q], face[i]);
         }
       }
     } else {
 #pragma unroll
       for (int q = 0; q < NFQ; ++q)
 #pragma unroll
-        for (int i = 0; i < NR; ++i) acc[i] = fma(tab[X::BF + (k * NFQ + q) * NB + row(i)], x[q], acc[i]);
+        for (int i = 0; i < NR; ++i) face[i] = fma(tab[X::BF + (k * NFQ + q) * NB + row(i)], x[q], face[i]);
     }
+#pragma unroll
+    for (int i = 0; i < NR; ++i) acc[i] = PARTS ? acc[i] + face[i] : face[i];
   }
   // the lift carries 1/sqrt|det|; the volume term sqrt|det| (flux) or nothing (the factors of the
   // trace and the test cancel in the derivative)
@@ -615,19 +637,30 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE, SL>::NT, ElemTile<T, D
   if constexpr (P > 0) {
 #pragma unroll
     for (int dd = 0; dd < D; ++dd) {
-      T m[NB1 > 0 ? NB1 : 1];
+      T m[NB1 > 0 ? NB1 : 1], m2[NB1 > 0 ? NB1 : 1], vol[NR];
 #pragma unroll
-      for (int k = 0; k < NB1; ++k) m[k] = T(0);
+      for (int k = 0; k < NB1; ++k) m[k] = m2[k] = T(0);
+      const T f0 = SHIFT ? sF[(dd * NV + w) * ET + tl] : T(0);
 #pragma unroll
       for (int i = 0; i < (NQ + SL - 1) / SL; ++i) {
         const bool in = NQ % SL == 0 || i * SL + sub < NQ;
         const int q = in ? i * SL + sub : 0;
-        const T f = in ? sF[((q * D + dd) * NV + w) * ET + tl] : T(0);
+        T f = in ? sF[((q * D + dd) * NV + w) * ET + tl] : T(0);
+        if constexpr (SHIFT) f = in ? f - f0 : T(0);
 #pragma unroll
-        for (int k = 0; k < NB1; ++k) m[k] = fma(tab[X::WM + q * NB1 + k], f, m[k]);
+        for (int k = 0; k < NB1; ++k) {
+          if (HALVES && (i & 1)) m2[k] = fma(tab[X::WM + q * NB1 + k], f, m2[k]);
+          else m[k] = fma(tab[X::WM + q * NB1 + k], f, m[k]);
+        }
       }
+      if constexpr (HALVES) {
+#pragma unroll
+        for (int k = 0; k < NB1; ++k) m[k] += m2[k];
+      }
+#pragma unroll
+      for (int i = 0; i < NR; ++i) vol[i] = PARTS ? T(0) : acc[i];
       if constexpr (SL == 1) {
-        combine_modes<T, D, P, 1>(tab + X::CM + dd * NB * NB1, m, acc);
+        combine_modes<T, D, P, 1>(tab + X::CM + dd * NB * NB1, m, vol);
       } else {
 #pragma unroll
         for (int k = 0; k < NB1; ++k)
@@ -636,8 +669,15 @@ __global__ void __launch_bounds__(ElemTile<T, D, P, MODE, SL>::NT, ElemTile<T, D
 #pragma unroll
         for (int i = 0; i < NR; ++i)
 #pragma unroll
-          for (int k = 0; k < NB1; ++k) acc[i] = fma(tab[X::CM + (dd * NB + row(i)) * NB1 + k], m[k], acc[i]);
+          for (int k = 0; k < NB1; ++k) vol[i] = fma(tab[X::CM + (dd * NB + row(i)) * NB1 + k], m[k], vol[i]);
       }
+      if constexpr (SHIFT) {
+#pragma unroll
+        for (int i = 0; i < NR; ++i)
+          vol[i] = fma(tab[X::CH + dd * NB + row(i)], f0, fma(tab[X::CL + dd * NB + row(i)], f0, vol[i]));
+      }
+#pragma unroll
+      for (int i = 0; i < NR; ++i) acc[i] = PARTS ? acc[i] + vol[i] : vol[i];
     }
   }
   T sc = oscale ? (T)*oscale : T(1);
@@ -723,6 +763,13 @@ cudaError_t upload_tables_p(const double* Bv, const double* Dv, const double* Wv
         for (int q = 0; q < NQ; ++q) a += Dv[(dd * NQ + q) * NB + i] * Bv[q * NB + k];
         tab[X::CM + (dd * NB + i) * NB1 + k] = (T)a;
       }
+  for (int dd = 0; dd < D; ++dd)
+    for (int i = 0; i < NB; ++i) {
+      double a = 0;
+      for (int q = 0; q < NQ; ++q) a += Dv[(dd * NQ + q) * NB + i];
+      tab[X::CH + dd * NB + i] = (T)a;
+      tab[X::CL + dd * NB + i] = (T)(a - (double)(T)a);
+    }
   for (int f = 0; f < O::NF; ++f)
     for (int i = 0; i < O::NFQ * NB; ++i) tab[X::BF + f * O::NFQ * NB + i] = (T)Bf[(f * O::NPERM) * O::NFQ * NB + i];
   cudaError_t e = cudaMemcpyToSymbolAsync(c_tab<T, D, P>, tab, sizeof(tab), 0, cudaMemcpyHostToDevice, st);
