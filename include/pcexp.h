@@ -46,7 +46,12 @@ extern "C" {
 #define PCEXP_ERR_OOM (-4)         /* device allocation failed */
 #define PCEXP_ERR_NONFINITE (-5)   /* a norm, beta or h_{j+1,j} was NaN/Inf */
 #define PCEXP_ERR_TIMEOUT (-6)     /* a partition of a group missed a rendezvous (failed or stalled), or
-                                      the blocks of a cooperative kernel did not meet in time */
+                                      the blocks of a cooperative kernel did not meet in time: the
+                                      Krylov stage they belong to added nothing to the state.
+                                      pcexp_arnoldi, pcexp_step_backward, the march and a step with
+                                      info report it themselves; after a step without info the
+                                      context's next call that finds it does, once (a call that
+                                      reports it on entry has done nothing else) */
 #define PCEXP_ERR_UNSUPPORTED (-7) /* valid request this build does not cover */
 
 /* ---- boundary tags (Sec. 4.4, Sec. 5.2) ---- */
@@ -386,6 +391,12 @@ int pcexp_fp32_fma_rate(double* tflops);
 
 /* Waits for all work queued on the context's stream. */
 int pcexp_synchronize(pcexp_ctx* ctx);
+
+/* Polls after which the blocks of a one-launch Gram-Schmidt column (PCEXP_KC_CGS_COLUMN) give up
+ * waiting for each other's sums and the call ends with PCEXP_ERR_TIMEOUT; default 2^23 (seconds).
+ * 0: every exchange counts as missed, for the tests of a host's handling of that status.  Waits for
+ * the context's stream.  Errors: INVALID_ARG, CUDA. */
+int pcexp_set_exchange_polls(pcexp_ctx* ctx, uint32_t polls);
 
 /* ---- partitioned runs (an element decomposition; the paper runs on one processor)
  *

@@ -112,6 +112,7 @@ SIGNATURES = {
     "pcexp_functional_params": (C.c_int, [_P, C.c_int, _D, C.c_int, _P, _D, _P, C.c_int]),
     "pcexp_set_physics": (C.c_int, [_P, C.POINTER(pcexp_physics)]),
     "pcexp_synchronize": (C.c_int, [_P]),
+    "pcexp_set_exchange_polls": (C.c_int, [_P, C.c_uint32]),
     "pcexp_residual_noalloc": (C.c_int, [_P, _P, _P]),
     "pcexp_profile_enable": (C.c_int, [_P, C.c_int]),
     "pcexp_profile_read": (C.c_int, [_P, C.c_int, C.POINTER(C.c_int64), _D]),
@@ -399,6 +400,9 @@ class Context:
         prm = np.ascontiguousarray(params, np.float64)
         check(self.lib.pcexp_project_state(self.ctx, kind, prm.ctypes.data_as(_D) if prm.size else None,
                                            prm.size), "pcexp_project_state")
+
+    def set_exchange_polls(self, polls: int):
+        check(self.lib.pcexp_set_exchange_polls(self.ctx, polls), "pcexp_set_exchange_polls")
 
     def residual(self, U, out=None):
         out = (np.empty(self.K) if isinstance(U, np.ndarray) else U.new_empty(self.K)) if out is None else out

@@ -36,7 +36,7 @@ struct pcexp_ctx {
   double eta = 0;
   double ktol = 0;  // Krylov tolerance of the adaptive dimension (<= 0: fixed dimension)
   bool selective = false;  // Arnoldi: second Gram-Schmidt pass only after a cancelling first pass
-  ColumnPlan col{0, 0};    // one-launch Gram-Schmidt columns (blocks == 0: the separate passes)
+  ColumnPlan col{};        // one-launch Gram-Schmidt columns (blocks == 0: the separate passes)
   unsigned long long* col_slots = nullptr;  // their exchange slots
   int basis_io = PCEXP_BASIS_PAPER;
   double volume = 0;
@@ -492,6 +492,16 @@ int krylov_error(int err, const char* nonfinite) {
   return err == 2 ? PCEXP_ERR_TIMEOUT : PCEXP_ERR_NONFINITE;
 }
 
+// Reports (once) a step or Arnoldi process that lost an exchange; complete after a synchronisation of
+// the context's stream.  A step called without info returns before it has run, so the next call that
+// finds the flag reports it (and waits first, so that the step's other stage cannot raise it again).
+int lost_exchange(const pcexp_ctx* c) {
+  if (!c->col.lost || !*(volatile int*)c->col.lost) return PCEXP_OK;
+  PCEXP_CK(cudaStreamSynchronize(c->st));
+  *(volatile int*)c->col.lost = 0;
+  return krylov_error(2, "");
+}
+
 // Columns between checkpoints of the adaptive Krylov dimension.
 constexpr int KRYLOV_CHECK = 5;
 
@@ -741,6 +751,7 @@ int step_impl(pcexp_ctx* c, int scheme, int dt_mode, double dt_or_cfl, int m, pc
     info->krylov_err[1] = one_stage ? 0.0 : h.kerr[1];
     info->reorth_cols[0] = h.pass2[0];
     info->reorth_cols[1] = one_stage ? 0u : h.pass2[1];
+    PCEXP_TRY(lost_exchange(c));
     if (h.err) return krylov_error(h.err, "non-finite norm, beta or Hessenberg entry");
   }
   return PCEXP_OK;
@@ -769,6 +780,7 @@ int march_impl(pcexp_ctx* c, int scheme, double cfl_max, double decades, int max
     StepState h;
     PCEXP_CK(cudaMemcpyAsync(&h, c->ss, sizeof(h), cudaMemcpyDeviceToHost, c->st));
     PCEXP_CK(cudaStreamSynchronize(c->st));
+    PCEXP_TRY(lost_exchange(c));
     rn = h.res_norm;
     if (c->grp) {
       // the norm over the whole mesh from the partitions' sums of squares (each partition's norm
@@ -831,6 +843,7 @@ int arnoldi_abi(pcexp_ctx* c, const double* U, const double* b, int m, double* V
   KState hk;
   PCEXP_CK(cudaMemcpyAsync(&hk, c->ks, sizeof(hk), cudaMemcpyDeviceToHost, c->st));
   PCEXP_CK(cudaStreamSynchronize(c->st));
+  PCEXP_TRY(lost_exchange(c));
   if (hk.err) return krylov_error(hk.err, "non-finite Arnoldi quantity");
   const int kk = hk.k;
   if (k) *k = kk;
@@ -1112,7 +1125,7 @@ int check_ctx(const pcexp_ctx* c) {
     g_last_error = cudaGetErrorString(e);
     return PCEXP_ERR_CUDA;
   }
-  return PCEXP_OK;
+  return lost_exchange(c);
 }
 
 int create_impl(pcexp_ctx* c, const pcexp_mesh* mesh, int p, const pcexp_physics* phys, const pcexp_options* opt,
@@ -1407,6 +1420,7 @@ int step_backward_impl(pcexp_ctx* c, const double* U, double dt, int m, const do
   PCEXP_CK(cudaStreamSynchronize(c->st));
   if (h1.err || h2.err) {
     c->prof = prof;
+    PCEXP_TRY(lost_exchange(c));
     return krylov_error(std::max(h1.err, h2.err), "non-finite quantity in the recomputed step");
   }
   const int k1 = h1.k, k2 = h2.k;
@@ -1533,7 +1547,14 @@ int pcexp_create(pcexp_ctx** out, const pcexp_mesh* mesh, int p, const pcexp_phy
   if (r == PCEXP_OK) {
     // (a partition's columns keep the separate passes: their sums meet the other partitions' in between)
     c->col = c->fp32 ? plan_cgs_column<float>(c->Kp) : plan_cgs_column<double>(c->Kp);
-    if (c->col.blocks > 0) r = dalloc(c, &c->col_slots, column_slots(c->col));
+    if (c->col.blocks > 0) {
+      r = dalloc(c, &c->col_slots, column_slots(c->col));
+      if (r == PCEXP_OK && cudaHostAlloc(&c->col.lost, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
+        g_last_error = "cudaHostAlloc of the exchange's status";
+        r = PCEXP_ERR_OOM;
+      }
+      if (r == PCEXP_OK) *c->col.lost = 0;
+    }
   }
   if (r != PCEXP_OK) {
     std::string keep = g_last_error;
@@ -1553,6 +1574,7 @@ int pcexp_destroy(pcexp_ctx* c) {
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
   for (auto& g : c->graphs) cudaGraphExecDestroy(g.exec);
   if (c->cap_st) cudaStreamDestroy(c->cap_st);
+  if (c->col.lost) cudaFreeHost(c->col.lost);
   delete c;
   return PCEXP_OK;
 }
@@ -1579,7 +1601,8 @@ int pcexp_set_state(pcexp_ctx* c, const double* U, int on_device) {
 int pcexp_get_state(pcexp_ctx* c, double* U, int on_device) {
   PCEXP_TRY(check_ctx(c));
   if (!U) return PCEXP_ERR_INVALID_ARG;
-  return export_vec<double>(c, c->U64[c->cur], U, on_device);
+  PCEXP_TRY(export_vec<double>(c, c->U64[c->cur], U, on_device));
+  return on_device ? PCEXP_OK : lost_exchange(c);  // on the device the copy is only queued
 }
 
 int pcexp_project_state(pcexp_ctx* c, int kind, const double* params, int n_params) {
@@ -1904,6 +1927,7 @@ int pcexp_output(pcexp_ctx* c, int kind, double* value) {
     double sum = 0;
     PCEXP_CK(cudaMemcpyAsync(&sum, &c->ss->dtmin_scratch, sizeof(double), cudaMemcpyDeviceToHost, c->st));
     PCEXP_CK(cudaStreamSynchronize(c->st));
+    PCEXP_TRY(lost_exchange(c));
     if (!std::isfinite(sum)) {
       g_last_error = "non-finite entropy integral";
       return PCEXP_ERR_NONFINITE;
@@ -1925,6 +1949,7 @@ int pcexp_output(pcexp_ctx* c, int kind, double* value) {
   StepState h;
   PCEXP_CK(cudaMemcpyAsync(&h, c->ss, sizeof(h), cudaMemcpyDeviceToHost, c->st));
   PCEXP_CK(cudaStreamSynchronize(c->st));
+  PCEXP_TRY(lost_exchange(c));
   *value = h.res_norm;
   return PCEXP_OK;
 }
@@ -1952,6 +1977,15 @@ int pcexp_profile_read(pcexp_ctx* c, int kernel_class, int64_t* launches, double
 int pcexp_synchronize(pcexp_ctx* c) {
   PCEXP_TRY(check_ctx(c));
   PCEXP_CK(cudaStreamSynchronize(c->st));
+  return lost_exchange(c);
+}
+
+int pcexp_set_exchange_polls(pcexp_ctx* c, uint32_t polls) {
+  PCEXP_TRY(check_ctx(c));
+  PCEXP_CK(cudaStreamSynchronize(c->st));
+  c->col.polls = polls;
+  for (auto& g : c->graphs) cudaGraphExecDestroy(g.exec);  // they hold the limit they were recorded with
+  c->graphs.clear();
   return PCEXP_OK;
 }
 
@@ -1977,7 +2011,7 @@ const char* pcexp_status_string(int status) {
     case PCEXP_ERR_CUDA: return "CUDA error";
     case PCEXP_ERR_OOM: return "out of device memory";
     case PCEXP_ERR_NONFINITE: return "non-finite value";
-    case PCEXP_ERR_TIMEOUT: return "wait timed out (partition rendezvous)";
+    case PCEXP_ERR_TIMEOUT: return "a rendezvous of partitions or of a kernel's blocks timed out";
     case PCEXP_ERR_UNSUPPORTED: return "unsupported request";
   }
   return "unknown status";

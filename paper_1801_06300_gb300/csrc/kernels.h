@@ -366,7 +366,10 @@ cudaError_t launch_cgs(int mode, const T* Z, int64_t ldz, int64_t Kp, int j, T* 
 // blocks == 0: the separate passes serve this length.
 struct ColumnPlan {
   int blocks, rows;
+  unsigned polls;  // polls of an exchange before a block gives up
+  int* lost;       // host memory: set to 1 when one did (nullable)
 };
+constexpr unsigned COL_POLLS = 1u << 23;  // the default: seconds
 constexpr int COL_SUMS = MMAX + 2;       // slots per block of one exchange of sums
 constexpr int COL_MAX_BLOCKS = 160;
 // slots of a context's columns: two sets of four exchanges

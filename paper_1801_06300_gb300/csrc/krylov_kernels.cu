@@ -727,7 +727,6 @@ cudaError_t launch_cgs(int mode, const T* Z, int64_t ldz, int64_t Kp, int j, T* 
 // the FP64 additions of a 32-column butterfly in every warp cost as much as the sweep of a small
 // vector); the update gives each thread its own rows.
 constexpr int COL_NT = 512, COL_WARPS = COL_NT / 32;
-constexpr unsigned COL_SPIN_LIMIT = 1u << 23;  // polls of an exchange (seconds) before giving up
 // An empty slot: a NaN, as a double and as a pair of floats alike; sums with that bit pattern are
 // stored as another NaN.
 constexpr unsigned long long COL_EMPTY = ~0ull;
@@ -750,10 +749,11 @@ PCEXP_DEV unsigned long long column_peek(const unsigned long long* p) {
 }
 
 // The grid's sums of sm.sums[0..n) -> sm.dots, identical in every block.  False if a block's sums
-// did not arrive within the limit of polls (ks->err = 2).  Every thread of every block calls this;
+// did not arrive within the limit of polls (ks->err = 2, *lost = 1).  Every thread of every block calls this;
 // slots: [block][COL_SUMS], empty before, used by this reduction alone.
 template <class T>
-PCEXP_DEV bool column_grid_sum(ColumnSmem<T>& sm, int n, unsigned long long* slots, KState* ks) {
+PCEXP_DEV bool column_grid_sum(ColumnSmem<T>& sm, int n, unsigned long long* slots, KState* ks, unsigned limit,
+                               int* lost) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nblk = gridDim.x;
   __syncthreads();
@@ -768,11 +768,8 @@ PCEXP_DEV bool column_grid_sum(ColumnSmem<T>& sm, int n, unsigned long long* slo
   if (n == 1) {  // thread = block; the warps that hold blocks add up theirs
     const int q = threadIdx.x, nw = (nblk + 31) / 32;
     if (wid < nw) {
-      unsigned long long v = 0ull;
-      unsigned polls = 0;
-      if (q < nblk)
-        do v = column_peek(slots + (int64_t)q * COL_SUMS);
-        while (v == COL_EMPTY && ++polls < COL_SPIN_LIMIT);
+      unsigned long long v = q < nblk ? COL_EMPTY : 0ull;
+      for (unsigned polls = 0; v == COL_EMPTY && polls < limit; ++polls) v = column_peek(slots + (int64_t)q * COL_SUMS);
       late = v == COL_EMPTY;
       Acc<T> a = *reinterpret_cast<const Acc<T>*>(&v);
       for (int o = 16; o > 0; o >>= 1) a.add_partner(o);
@@ -781,10 +778,9 @@ PCEXP_DEV bool column_grid_sum(ColumnSmem<T>& sm, int n, unsigned long long* slo
   } else {  // warp = every COL_WARPS-th block, lane = column
     constexpr int PER = COL_MAX_BLOCKS / COL_WARPS;
     for (int c = lane; c < n; c += 32) {
-      unsigned long long v[PER];
-      unsigned polls = 0;
-      bool all;
-      do {
+      unsigned long long v[PER] = {};
+      bool all = false;
+      for (unsigned polls = 0; !all && polls < limit; ++polls) {
         all = true;
 #pragma unroll
         for (int i = 0; i < PER; ++i) {
@@ -792,7 +788,7 @@ PCEXP_DEV bool column_grid_sum(ColumnSmem<T>& sm, int n, unsigned long long* slo
           v[i] = q < nblk ? column_peek(slots + (int64_t)q * COL_SUMS + c) : 0ull;
           all = all && v[i] != COL_EMPTY;
         }
-      } while (!all && ++polls < COL_SPIN_LIMIT);
+      }
       late = late || !all;
       Acc<T> a = *reinterpret_cast<const Acc<T>*>(&v[0]);
 #pragma unroll
@@ -806,6 +802,7 @@ PCEXP_DEV bool column_grid_sum(ColumnSmem<T>& sm, int n, unsigned long long* slo
     if (threadIdx.x == 0) {
       ks->err = 2;
       ks->done = 1;
+      if (lost) *(volatile int*)lost = 1;
     }
     return false;
   }
@@ -989,7 +986,7 @@ template <class T>
 __global__ void __launch_bounds__(COL_NT, 1) cgs_column_kernel(const T* __restrict__ Z, int64_t ldz, int64_t Kp, int j,
                                                                const T* __restrict__ w, T* __restrict__ out,
                                                                KState* ks, unsigned long long* slots, double eta,
-                                                               int rows, int selective) {
+                                                               int rows, int selective, unsigned limit, int* lost) {
   constexpr int VN = VecN<T>::N;
   extern __shared__ __align__(16) unsigned char col_dyn[];
   __shared__ __align__(16) ColumnSmem<T> sm;
@@ -1017,13 +1014,13 @@ __global__ void __launch_bounds__(COL_NT, 1) cgs_column_kernel(const T* __restri
   }
   __syncthreads();
   column_project<T>(sm, xs, Zb, ldz, nc, true, nch);
-  if (!column_grid_sum<T>(sm, nc + 1, mine, ks)) return;
+  if (!column_grid_sum<T>(sm, nc + 1, mine, ks, limit, lost)) return;
   const double wnorm0 = sqrt(sm.dots[nc]);
   if (!column_coefficients<T>(sm, j, true, ks)) return;
   column_update<T>(sm, xs, outb, Zb, ldz, nc, nch);
   if (selective) {
     // keep the first pass when it cancelled less than DGKS_KAPPA (cgs_finalize's UPD1)
-    if (!column_grid_sum<T>(sm, 1, mine + red, ks)) return;
+    if (!column_grid_sum<T>(sm, 1, mine + red, ks, limit, lost)) return;
     const double n1 = sqrt(sm.dots[0]);
     if (isfinite(n1) && n1 > 0.0 && n1 >= DGKS_KAPPA * wnorm0) {
       if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1036,10 +1033,10 @@ __global__ void __launch_bounds__(COL_NT, 1) cgs_column_kernel(const T* __restri
   }
   __syncthreads();
   column_project<T>(sm, xs, Zb, ldz, nc, false, nch);
-  if (!column_grid_sum<T>(sm, nc, mine + 2 * red, ks)) return;
+  if (!column_grid_sum<T>(sm, nc, mine + 2 * red, ks, limit, lost)) return;
   if (!column_coefficients<T>(sm, j, false, ks)) return;
   column_update<T>(sm, xs, outb, Zb, ldz, nc, nch);
-  if (!column_grid_sum<T>(sm, 1, mine + 3 * red, ks)) return;
+  if (!column_grid_sum<T>(sm, 1, mine + 3 * red, ks, limit, lost)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     const double hn = sqrt(sm.dots[0]);
     ks->pass2 |= 1u << j;
@@ -1058,7 +1055,7 @@ __global__ void __launch_bounds__(COL_NT, 1) cgs_column_kernel(const T* __restri
 
 template <class T>
 ColumnPlan plan_cgs_column(int64_t Kp) {
-  ColumnPlan plan{0, 0};
+  ColumnPlan plan{0, 0, COL_POLLS, nullptr};
   int dev = 0, sms = 0, coop = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -1097,7 +1094,7 @@ cudaError_t launch_cgs_column(const ColumnPlan& plan, const T* Z, int64_t ldz, i
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, cgs_column_kernel<T>, Z, ldz, Kp, j, w, out, ks, slots, eta, plan.rows,
-                            selective ? 1 : 0);
+                            selective ? 1 : 0, plan.polls, plan.lost);
 }
 
 // ------------------------------------------------ Gram-Schmidt of a partitioned run
