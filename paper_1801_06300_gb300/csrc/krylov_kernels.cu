@@ -22,6 +22,7 @@
 // Partial products are accumulated in FP64 (FP64 form) or in compensated FP32
 // pairs converted to FP64 once per warp (FP32-mixed form).
 #include <cooperative_groups.h>
+#include <atomic>
 #include <cfloat>
 #include <cstddef>
 
@@ -1400,14 +1401,21 @@ __global__ void __cluster_dims__(PHI_CTAS, 1, 1) __launch_bounds__(256)
   }
 }
 
+// Raises a kernel's dynamic shared-memory limit on the current device, once per device (bits of
+// done): the limit belongs to the device's context.
+static cudaError_t allow_shared(const void* kernel, size_t bytes, std::atomic<unsigned long long>& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+  if (done.load() & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess) done.fetch_or(bit);
+  return e;
+}
 static cudaError_t phi_smem_attr(size_t smem) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(phi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  return cudaSuccess;
+  static std::atomic<unsigned long long> done{0};
+  return allow_shared((const void*)phi_kernel, smem, done);
 }
 
 cudaError_t launch_phi(KState* ks, const double* dt_dev, double dt, double factor, StepState* ss, int stage,
@@ -1431,12 +1439,9 @@ cudaError_t launch_phi_adjoint(const double* H, int k, int ldh, double dt, const
                                cudaStream_t st) {
   if (k < 1 || k > MMAX) return cudaErrorInvalidValue;
   const size_t smem = 5 * PN2 * PN2 * sizeof(double);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(phi_adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static std::atomic<unsigned long long> done{0};
+  const cudaError_t e = allow_shared((const void*)phi_adjoint_kernel, smem, done);
+  if (e != cudaSuccess) return e;
   phi_adjoint_kernel<<<PHI_CTAS, 256, smem, st>>>(H, k, ldh, dt, ybar, Hbar, err);
   return cudaGetLastError();
 }
