@@ -4,4 +4,5 @@
 namespace pcexp {
 PCEXP_INST_D(double, 2)
 PCEXP_INST_D(float, 2)
+PCEXP_INST_FP64(2)
 }  // namespace pcexp

@@ -4,4 +4,5 @@
 namespace pcexp {
 PCEXP_INST_D(double, 3)
 PCEXP_INST_D(float, 3)
+PCEXP_INST_FP64(3)
 }  // namespace pcexp

@@ -1119,6 +1119,7 @@ __global__ void __launch_bounds__(256) face_adjoint_kernel(DGData<T> d, const T*
   using O = Ord<D, P>;
   constexpr int NB = O::NB, NFQ = O::NFQ, NV = O::NV, NPERM = O::NPERM, GEO = O::GEO, NN = NV * NV;
   constexpr bool SM = O::SMEM_BF;
+  static_assert(!FACE_RECORDS<T, D>, "this kernel reads a block per face point, not a record");
   __shared__ T sBf[SM ? O::NBF : 1];
   if constexpr (SM)
     for (int i = threadIdx.x; i < O::NBF; i += blockDim.x) sBf[i] = d.Bf[i];
@@ -2104,8 +2105,6 @@ cudaError_t launch_local_dt_d(const DGData<T>& d, const T* u, const double* cfl_
   template cudaError_t upload_tables_d<T, D>(const DGData<T>&, const double*, const double*, const double*,        \
                                              const double*, cudaStream_t);                                         \
   template int64_t face_flux_size_d<T, D>(const DGData<T>&);                                                       \
-  template cudaError_t launch_jac_adjoint_d<T, D>(const DGData<T>&, LinData<T>, const T*, T*, T*, const T*, T,     \
-                                                  cudaStream_t);                                                   \
   template cudaError_t launch_jvp_state_adjoint_d<T, D>(const DGData<T>&, const T*, const T*, const T*, T*, T*,    \
                                                         const T*, T, cudaStream_t, const ThetaSums<T>&);           \
   template cudaError_t launch_vjp_d<T, D>(const DGData<T>&, const T*, const T*, T*, T*, cudaStream_t);             \
@@ -2119,5 +2118,10 @@ cudaError_t launch_local_dt_d(const DGData<T>& d, const T* u, const double* cfl_
                                                         const double*, double*, double*, unsigned*, cudaStream_t); \
   template cudaError_t launch_param_adjoint_d<T, D>(const DGData<T>&, int64_t, const T*, const T*, double,         \
                                                     const double*, double*, double*, unsigned*, cudaStream_t);
+
+// (the stored-block forms of double precision alone)
+#define PCEXP_INST_FP64(D)                                                                                         \
+  template cudaError_t launch_jac_adjoint_d<double, D>(const DGData<double>&, LinData<double>, const double*,      \
+                                                       double*, double*, const double*, double, cudaStream_t);
 
 }  // namespace pcexp
