@@ -377,6 +377,8 @@ inline size_t column_slots(const ColumnPlan& p) { return (size_t)2 * 4 * COL_SUM
 // Bytes of a block's rows up to which the one-launch column is the faster form (measured, see
 // cgs_column_kernel).
 template <class T> constexpr int64_t COLUMN_MAX_BYTES = sizeof(T) == 8 ? 100 * 1024 : 32 * 1024;
+// Rows of a block from which more blocks stop paying (measured, see plan_cgs_column).
+template <class T> constexpr int64_t COLUMN_MIN_ROWS = sizeof(T) == 8 ? 256 : 1408;
 template <class T>
 ColumnPlan plan_cgs_column(int64_t Kp);
 template <class T>

@@ -711,7 +711,7 @@ cudaError_t launch_cgs(int mode, const T* Z, int64_t ldz, int64_t Kp, int j, T* 
 // sweeps.  Each of them drains, reduces its block sums in one last block and starts the next
 // (8 to 30 us a pass in FP64 and 5 to 9 us in FP32 against 1 to 8 us of arithmetic), the
 // selective form pays two more launches that leave at once, and a row per thread puts a
-// 27,648-entry FP64 vector on 54 of the 152 SMs.  Here the rows are spread over all SMs and a sweep
+// 27,648-entry FP64 vector on 54 of the 152 SMs.  Here the rows are spread over up to all SMs and a sweep
 // ends in an all-to-all exchange of the block sums through L2 instead of a launch: every block
 // stores its sums and adds up all blocks' itself, in a fixed order.  A slot starts as a bit
 // pattern that no arithmetic result has, so a value is its own flag and the exchange takes one
@@ -980,11 +980,11 @@ PCEXP_DEV bool column_coefficients(ColumnSmem<T>& sm, int j, bool first, KState*
   return !sm.bad;
 }
 
-// rows: of one block (a multiple of 64; the last blocks may have fewer or none).  slots: two sets
+// rows: of one block (a multiple of 64; the last block may have fewer).  slots: two sets
 // of four reductions' slots; column j uses set j & 1 and empties the other for column j + 1 (set
 // 0 is emptied by reset_kstate before column 0).
 template <class T>
-__global__ void __launch_bounds__(COL_NT, 1) cgs_column_kernel(const T* __restrict__ Z, int64_t ldz, int64_t Kp, int j,
+__global__ void __launch_bounds__(COL_NT, 2) cgs_column_kernel(const T* __restrict__ Z, int64_t ldz, int64_t Kp, int j,
                                                                const T* __restrict__ w, T* __restrict__ out,
                                                                KState* ks, unsigned long long* slots, double eta,
                                                                int rows, int selective, unsigned limit, int* lost) {
@@ -1054,6 +1054,20 @@ __global__ void __launch_bounds__(COL_NT, 1) cgs_column_kernel(const T* __restri
   }
 }
 
+// Blocks of a column: at most one per SM, each with at least COLUMN_MIN_ROWS rows.  Every block adds up
+// all blocks' sums, and contexts on several streams run side by side only while their grids fit the
+// chip together (two blocks per SM: 64 registers, and up to 90 KB of rows).  Time of a PCEXP step in
+// one context / of each when four threads step a context each (us), on one block per SM whatever K ->
+// this rule (the separate passes):
+//   FP64  K = 6,144, m = 10      778 / 1694 -> 762 / 817   (1191 / 1313)
+//         K = 27,648, m = 30     2508 / 6958 -> 2544 / 5157 (4268 / 5151)
+//         K = 110,592, m = 30    3850 / 12506 -> 3847 / 11684 (5871 / 11129)
+//   FP32  K = 6,144, m = 10      441 / 966 -> 413 / 462    (582 / 688)
+//         K = 27,648, m = 30     1278 / 3104 -> 1220 / 1393 (1950 / 2224)
+//         K = 110,592, m = 30    1401 / 3573 -> 1355 / 2210 (2091 / 3020)
+//         K = 442,368, m = 30    1708 / 6009 -> 1674 / 5006 (2714 / 5977)
+// Fewer, longer blocks help several contexts further and cost the single one: FP64 K = 27,648 with 320
+// rows 2594 / 4609, with 192 rows 2493 / 5801; FP32 K = 110,592 with 2,048 rows 1381 / 2063.
 template <class T>
 ColumnPlan plan_cgs_column(int64_t Kp) {
   ColumnPlan plan{0, 0, COL_POLLS, nullptr};
@@ -1062,11 +1076,11 @@ ColumnPlan plan_cgs_column(int64_t Kp) {
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
     return plan;
-  const int blocks = sms < COL_MAX_BLOCKS ? sms : COL_MAX_BLOCKS;
-  const int64_t rows = ((Kp + blocks - 1) / blocks + VPAD - 1) / VPAD * VPAD;
+  const int64_t most = sms < COL_MAX_BLOCKS ? sms : COL_MAX_BLOCKS, share = (Kp + most - 1) / most;
+  const int64_t rows = ((share > COLUMN_MIN_ROWS<T> ? share : COLUMN_MIN_ROWS<T>) + VPAD - 1) / VPAD * VPAD;
   const int64_t bytes = rows * (int64_t)sizeof(T);
   if (bytes > COLUMN_MAX_BYTES<T>) return plan;
-  // every block of the grid must be resident (they exchange sums): one per SM
+  // every block of the grid must be resident (they exchange sums): at most one per SM
   if (cudaFuncSetAttribute(cgs_column_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)COLUMN_MAX_BYTES<T>) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cgs_column_kernel<T>, COL_NT, (size_t)bytes) !=
@@ -1075,7 +1089,7 @@ ColumnPlan plan_cgs_column(int64_t Kp) {
     cudaGetLastError();
     return plan;
   }
-  plan.blocks = blocks;
+  plan.blocks = (int)((Kp + rows - 1) / rows);
   plan.rows = (int)rows;
   return plan;
 }
