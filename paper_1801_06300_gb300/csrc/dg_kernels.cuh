@@ -338,7 +338,8 @@ template <class T, int D, int P, int MODE, int SL = 1> struct ElemTile {
   static constexpr int ROWS4 = (ROWS + 3) / 4 * 4;       // the records start on a 16-byte boundary
   static constexpr int RECS = AHEAD ? O::NF * GV * NT * VECW<T> : 0;
   static constexpr size_t BYTES = sizeof(T) * (size_t)(ROWS4 + RECS + FLUX);
-  // blocks per SM the registers are bounded for (the shared memory allows as many or more)
+  // blocks per SM the registers are bounded for (the shared memory allows as many or more, but for
+  // FP32 TANGENT on tetrahedra at p = 2: 60 KB, three blocks; its 80 registers spill nothing)
   static constexpr int MINB = sizeof(T) == 4 ? (D == 3 ? 4 : MODE == ELEM_STORED ? 7 : 5) : (D == 3 ? 2 : 3);
 };
 
@@ -358,7 +359,7 @@ template <class T, int D, int P, int MODE, int SL = 1> struct ElemTile {
 // 509 us without that).  FP64 is bound by its pipe.
 // Measured against the kernels this one replaces, per launch of the Krylov J v: FP32 48^3 cubes at
 // p = 2 449 -> 277 us (a persistent kernel whose six warps each kept 50 partial sums and recomputed
-// the flux derivative from u), FP32 131,072 triangles at p = 3 111 -> 32 us (lanes sharing an
+// the flux derivative from u), FP32 131,072 triangles at p = 3 111 -> 34 us (lanes sharing an
 // element's test functions), FP64 20^3 cubes at p = 2 485 -> 427 us (stored D nv x nv Jacobians);
 // the residual's: FP64 24^3 cubes at p = 2 1117 -> 717 us.
 //

@@ -717,11 +717,11 @@ cudaError_t launch_cgs(int mode, const T* Z, int64_t ldz, int64_t Kp, int j, T* 
 // pattern that no arithmetic result has, so a value is its own flag and the exchange takes one
 // store and one load, no counter.
 // An EXP1 step with 30 columns on periodic triangles at p = 2, separate -> one launch:
-//   FP64  K = 27,648 2010 -> 1464 us, 150,528 2810 -> 2243, 591,408 6641 -> 5976,
-//         1,503,792 14.04 -> 13.42 ms, 1,881,792 (97 KB per block) 17.49 -> 16.91 ms
-//   FP32, selective  K = 12,288 733 -> 642 us, 110,592 832 -> 720, 591,408 1176 -> 1042,
-//         1,080,000 (28 KB per block) 1791 -> 1691, 1,503,792 (39 KB) 2257 -> 2257,
-//         2,764,800 (71 KB) 3560 -> 3719
+//   FP64  K = 27,648 2010 -> 1274 us, 150,528 2810 -> 2230, 591,408 6641 -> 5960,
+//         1,503,792 14.04 -> 13.49 ms, 1,881,792 (97 KB per block) 17.49 -> 16.98 ms
+//   FP32, selective  K = 12,288 733 -> 602 us, 110,592 832 -> 708, 591,408 1176 -> 1011,
+//         1,080,000 (28 KB per block) 1791 -> 1649; one block of 80 registers per SM took 2257 as
+//         the separate passes on 1,503,792 (39 KB) and 3719 against 3560 on 2,764,800 (71 KB)
 // hence COLUMN_MAX_BYTES: 100 KB of rows per block in FP64 (longer ones were not tried), 32 KB in
 // FP32.
 // The projection gives each warp its own columns (one accumulator, so one warp sum per column:

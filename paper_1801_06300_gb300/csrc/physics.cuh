@@ -700,7 +700,7 @@ PCEXP_DEV void ghost_farfield_vjp(const S (&U)[D + 2], const T (&n)[D], const Fr
 }
 
 // ------------------------------------------------- Roe-flux derivative from a stored record
-// What the Roe flux's linearisation at (L, R) needs besides the normal; 14 values (D = 2: 12) that
+// What the Roe flux's linearisation at (L, R) needs besides the normal; 16 values (D = 2: 14) that
 // replace its 2 (D + 2)^2 Jacobian entries.  H total enthalpy, w = sqrt(rho_L) / (sqrt(rho_L) +
 // sqrt(rho_R)), c Roe's sound speed, i2c = 1 / (2 c^2), dp = p_R - p_L.
 template <class T, int D>
