@@ -220,7 +220,10 @@ def algorithmic_flops(kind, K, E, F, dim, p, m, T=8, gs=None):
 # DRAM bytes (read + write) per launch from one ncu capture of the same kernel on the same
 # workload, keyed (workload, element bytes, kernel class); an entry is dropped when its
 # kernel changes.  The summaries under profiles/ give the commands.
-NCU_TRAFFIC = {}
+NCU_TRAFFIC = {
+    ("vortex3d", 4, "jvp_elem"): (651137536, "profiles/traffic_vortex3d_48_p2_fp32.md"),
+    ("vortex3d", 4, "jvp_face"): (990264064, "profiles/traffic_vortex3d_48_p2_fp32.md"),
+}
 
 
 def fp64_peak(capi):
